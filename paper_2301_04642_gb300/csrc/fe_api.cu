@@ -6,7 +6,7 @@
 // number of 128-row panels and precision policy, filled by the autotuners).  A solve (or a batch of solves) is:
 //   bounds rows + reduce + X0 init              (per problem)
 //   repeat:  control (1 block / problem)  ->  tensor-core step over the tiles
-//            of all problems  ->  FP64 step over the 64x64 tiles of all
+//            of all problems  ->  FP64 step over the 16x16 tiles of all
 //            problems                      (kernels skip problems whose state
 //                                             says the step is not theirs)
 //   finalize (D out, tr(Hp D), tr D)            (per problem)
@@ -74,7 +74,7 @@ struct Slot {
     int ldy = 0, lds = 0, ldx = 0;
     std::vector<TileEnt> tiles;   // tensor-core tiles 128 x 256
     std::vector<TileEnt> tilesN;  // tensor-core tiles 128 x 128
-    std::vector<Tile64> tiles64;
+    std::vector<TileF64> tilesF;  // FP64 tiles, listed when the FP64 schedule first needs them
     std::vector<TileEnt> tilesD;  // digit-product tiles (zero temperature)
     MmaProb hp;  // host image of the device descriptor (H filled per solve)
 };
@@ -89,10 +89,10 @@ struct Engine {
     size_t probs_cap = 0;
     TileEnt *d_tiles = nullptr;
     size_t tiles_cap = 0;
-    Tile64 *d_tiles64 = nullptr;
-    size_t tiles64_cap = 0;
+    TileF64 *d_tilesF = nullptr;
+    size_t tilesF_cap = 0;
     TileEnt *d_tilesD = nullptr;
-    std::vector<int> off64, cnt64;  // each problem's range in the FP64 tile list
+    std::vector<int> offF, cntF;  // each problem's range in the FP64 tile list
     MmaProb *d_chk = nullptr;       // table of the problems certifying their bounds together
     size_t chk_cap = 0;
     size_t tilesD_cap = 0;
@@ -102,7 +102,7 @@ struct Engine {
     size_t h_done_cap = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaEvent_t ev_setup = nullptr, ev_loop = nullptr;  // end of set-up, end of the step loop
-    int ntc = 0, n64 = 0, nD = 0;    // tile counts of the uploaded lists
+    int ntc = 0, nF = 0, nD = 0;    // tile counts of the uploaded lists
     bool any_tc = false, any_fp64 = false, any_digit = false;
     // the step loop as a CUDA graph: WHILE(any problem active) { IF(tc) k_sym_mma;
     // IF(fp64) k_fp64_step; IF(digit) k_digit_prep, k_digit_mma; k_control }
@@ -245,16 +245,26 @@ void build_tiles(Slot *s) {
     const int TP = ceil_div(T, 2);
     push_banded(s->tiles, T, TP, kBandTc, [](int I) { return I / 2; });
     push_banded(s->tilesN, T, T, kBandTcN, [](int I) { return I; });
-    s->tiles64.clear();
-    const int T64 = ceil_div(s->n, kTile64);
-    int slot = 0;
-    for (int I = 0; I < T64; ++I)
-        for (int J = I; J < T64; ++J) s->tiles64.push_back(Tile64{0, I, J, slot++});
     s->tilesD.clear();
     if (s->method == kMethodSp2) {
         const int TD = ceil_div(s->n, kDigitN);
         push_banded(s->tilesD, T, TD, kBandDigit, [](int I) { return 2 * I; });
     }
+}
+
+// Upper-triangle FP64 tiles of an n x n product.
+int64_t num_tiles_f64(int64_t n) {
+    const int64_t T = (n + kTileF64 - 1) / kTileF64;
+    return T * (T + 1) / 2;
+}
+
+void build_tiles_f64(Slot *s) {
+    if (!s->tilesF.empty()) return;
+    const int T = ceil_div(s->n, kTileF64);
+    s->tilesF.reserve(static_cast<size_t>(num_tiles_f64(s->n)));
+    int slot = 0;
+    for (int I = 0; I < T; ++I)
+        for (int J = I; J < T; ++J) s->tilesF.push_back(TileF64{0, I, J, slot++});
 }
 
 // Matrices held per method: zero temperature keeps one FP32 master (Y) and two
@@ -268,13 +278,12 @@ size_t slot_bytes(int n, int method, int *ldy, int *lds, int *ldx, size_t *npart
     *lds = static_cast<int>(align_up(n, 8));
     *ldx = n;
     const int T = ceil_div(n, kTileM);
-    const int T64 = ceil_div(n, kTile64);
     const size_t ntiles = static_cast<size_t>(T) * (T + 1) / 2;  // >= T ceil(T/2): either width
-    const size_t nt64 = static_cast<size_t>(T64) * (T64 + 1) / 2;
+    const size_t ntF = method == kMethodSp2 ? static_cast<size_t>(num_tiles_f64(n)) : 0;
     const size_t TD = static_cast<size_t>(ceil_div(n, kDigitN));
     size_t ntD = 0;
     for (size_t I = 0; I < static_cast<size_t>(T); ++I) ntD += (TD > 2 * I) ? TD - 2 * I : 0;
-    *nparts = std::max<size_t>({static_cast<size_t>(kInitBlocks), ntiles, nt64, ntD,
+    *nparts = std::max<size_t>({static_cast<size_t>(kInitBlocks), ntiles, ntF, ntD,
                                 static_cast<size_t>(kFinBlocks)});
     const size_t nn = static_cast<size_t>(n);
     size_t b = 0;
@@ -462,7 +471,7 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
     s->hp.lds = lds;
     s->hp.ntiles = static_cast<int>(s->tiles.size());
     s->hp.bn = kTileN;
-    s->hp.ntiles64 = static_cast<int>(s->tiles64.size());
+    s->hp.ntilesF = static_cast<int>(num_tiles_f64(n));
     s->hp.ntilesD = static_cast<int>(s->tilesD.size());
     s->hp.lzv = s->lzv;
     s->hp.Xd[0] = s->Xd[0];
@@ -688,7 +697,7 @@ void eng_free(Engine &e) {
     if (e.d_err) cudaFree(e.d_err);
     if (e.d_probs) cudaFree(e.d_probs);
     if (e.d_tiles) cudaFree(e.d_tiles);
-    if (e.d_tiles64) cudaFree(e.d_tiles64);
+    if (e.d_tilesF) cudaFree(e.d_tilesF);
     if (e.d_tilesD) cudaFree(e.d_tilesD);
     if (e.d_chk) cudaFree(e.d_chk);
     if (e.h_states) cudaFreeHost(e.h_states);
@@ -705,11 +714,11 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
     const int np = static_cast<int>(jobs.size());
     std::vector<MmaProb> hprobs(np);
     std::vector<TileEnt> tiles;
-    std::vector<Tile64> tiles64;
+    std::vector<TileF64> tilesF;
     std::vector<TileEnt> tilesD;
     e.any_tc = e.any_fp64 = e.any_digit = false;
-    e.off64.assign(np, 0);
-    e.cnt64.assign(np, 0);
+    e.offF.assign(np, 0);
+    e.cntF.assign(np, 0);
     for (int k = 0; k < np; ++k) {
         const Job &j = jobs[k];
         hprobs[k] = j.slot->hp;
@@ -731,12 +740,13 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
             hprobs[k].ntiles = static_cast<int>(tl.size());
             hprobs[k].bn = bn;
         }
-        e.off64[k] = static_cast<int>(tiles64.size());
-        e.cnt64[k] = 0;
+        e.offF[k] = static_cast<int>(tilesF.size());
+        e.cntF[k] = 0;
         if (pr == FE_PREC_FP64 && !fermi && !trfoe) {
             e.any_fp64 = true;
-            for (Tile64 t : j.slot->tiles64) { t.prob = k; tiles64.push_back(t); }
-            e.cnt64[k] = static_cast<int>(j.slot->tiles64.size());
+            build_tiles_f64(j.slot);
+            for (TileF64 t : j.slot->tilesF) { t.prob = k; tilesF.push_back(t); }
+            e.cntF[k] = static_cast<int>(j.slot->tilesF.size());
         }
         if ((pr == FE_PREC_MIXED || pr == FE_PREC_TRY_FP16 || (trfoe && pr == FE_PREC_FP64)) && !fermi) {
             e.any_digit = true;
@@ -745,7 +755,7 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
     }
     int rc = ensure_dev(ctx, &e.d_probs, &e.probs_cap, np);
     if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tiles, &e.tiles_cap, tiles.size());
-    if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tiles64, &e.tiles64_cap, tiles64.size());
+    if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tilesF, &e.tilesF_cap, tilesF.size());
     if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tilesD, &e.tilesD_cap, tilesD.size());
     if (rc == FE_OK) rc = ensure_pinned(ctx, &e.h_states, &e.h_states_cap, np);
     if (rc == FE_OK) rc = ensure_pinned(ctx, &e.h_done, &e.h_done_cap, np + 1);  // + error word
@@ -755,8 +765,8 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
     if (!tiles.empty())
         FE_CUDA(ctx, cudaMemcpyAsync(e.d_tiles, tiles.data(), sizeof(TileEnt) * tiles.size(),
                                      cudaMemcpyHostToDevice, e.stream));
-    if (!tiles64.empty())
-        FE_CUDA(ctx, cudaMemcpyAsync(e.d_tiles64, tiles64.data(), sizeof(Tile64) * tiles64.size(),
+    if (!tilesF.empty())
+        FE_CUDA(ctx, cudaMemcpyAsync(e.d_tilesF, tilesF.data(), sizeof(TileF64) * tilesF.size(),
                                      cudaMemcpyHostToDevice, e.stream));
     if (!tilesD.empty())
         FE_CUDA(ctx, cudaMemcpyAsync(e.d_tilesD, tilesD.data(), sizeof(TileEnt) * tilesD.size(),
@@ -764,7 +774,7 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
     // the copies read host vectors that go out of scope here
     FE_CUDA(ctx, cudaStreamSynchronize(e.stream));
     e.ntc = static_cast<int>(tiles.size());
-    e.n64 = static_cast<int>(tiles64.size());
+    e.nF = static_cast<int>(tilesF.size());
     e.nD = static_cast<int>(tilesD.size());
     return FE_OK;
 }
@@ -792,7 +802,7 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
         k_bounds_rows<<<ceil_div(n, 8), 256, 0, s>>>(e.d_probs, k, j.slot->rowinfo, j.slot->bad);
         k_bounds_reduce<<<1, 1024, 0, s>>>(e.d_probs, k, j.slot->rowinfo, j.slot->bad);
         ctx->launches += 2;
-        if (j.lanczos) (e.cnt64[k] > 0 ? f64_chk : tc_chk).push_back(k);
+        if (j.lanczos) (e.cntF[k] > 0 ? f64_chk : tc_chk).push_back(k);
     }
     const bool any_lz = !tc_chk.empty() || !f64_chk.empty();
     if (any_lz) {
@@ -843,8 +853,8 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
             const MmaProb *one = e.d_probs + k;
             k_control<<<1, 256, 0, s>>>(one, 1, e.d_err, nullptr, 0, 0, 0, 0, 0u);
             for (int c = 0; c < kCheckSteps; ++c) {
-                k_fp64_step<<<std::max(1, std::min(e.cnt64[k], 4 * ctx->num_sms)), 256, 0, s>>>(
-                    e.d_probs, e.d_tiles64 + e.off64[k], e.cnt64[k]);
+                k_fp64_step<<<std::max(1, std::min(e.cntF[k], 8 * ctx->num_sms)), 256, 0, s>>>(
+                    e.d_probs, e.d_tilesF + e.offF[k], e.cntF[k]);
                 k_control<<<1, 256, 0, s>>>(one, 1, e.d_err, nullptr, 0, 0, 0, 0, 0u);
             }
             ctx->launches += 1 + 2 * kCheckSteps;
@@ -867,7 +877,7 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
 void eng_steps(fe_ctx *ctx, Engine &e, int np, int count, const std::vector<cudaEvent_t> *pev) {
     cudaStream_t s = e.stream;
     const int grid_tc = ctx->num_sms;  // the kernel itself uses at most (work / largest tile) CTAs
-    const int grid_64 = std::max(1, std::min(e.n64, 4 * ctx->num_sms));
+    const int grid_f = std::max(1, std::min(e.nF, 8 * ctx->num_sms));
     const size_t smem = mma_smem_bytes();
     const int grid_d = std::max(1, std::min(e.nD, ctx->num_sms));
     for (int it = 0; it < count; ++it) {
@@ -880,7 +890,7 @@ void eng_steps(fe_ctx *ctx, Engine &e, int np, int count, const std::vector<cuda
         if (pev) cudaEventRecord((*pev)[4 * it + 1], s);
         if (pev) cudaEventRecord((*pev)[4 * it + 2], s);
         if (e.any_fp64) {
-            k_fp64_step<<<grid_64, 256, 0, s>>>(e.d_probs, e.d_tiles64, e.n64);
+            k_fp64_step<<<grid_f, 256, 0, s>>>(e.d_probs, e.d_tilesF, e.nF);
             ++ctx->launches;
         }
         if (e.any_digit) {
@@ -957,9 +967,9 @@ void fill_result(const SolveState &st, int herr, double ms, fe_result &r) {
 // kernels that have work run, with no host round trip.
 int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     std::vector<uintptr_t> key = {reinterpret_cast<uintptr_t>(e.d_probs), reinterpret_cast<uintptr_t>(e.d_tiles),
-                                  reinterpret_cast<uintptr_t>(e.d_tiles64), reinterpret_cast<uintptr_t>(e.d_tilesD),
+                                  reinterpret_cast<uintptr_t>(e.d_tilesF), reinterpret_cast<uintptr_t>(e.d_tilesD),
                                   static_cast<uintptr_t>(np), static_cast<uintptr_t>(e.ntc),
-                                  static_cast<uintptr_t>(e.n64), static_cast<uintptr_t>(e.nD),
+                                  static_cast<uintptr_t>(e.nF), static_cast<uintptr_t>(e.nD),
                                   static_cast<uintptr_t>(e.any_tc), static_cast<uintptr_t>(e.any_fp64),
                                   static_cast<uintptr_t>(e.any_digit)};
     if (e.gexec && key == e.gkey) return FE_OK;
@@ -1040,11 +1050,11 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     if (e.any_fp64) {
         cudaGraph_t ib;
         FE_CUDA(ctx, add_if(hf, &ib));
-        const Tile64 *tl = e.d_tiles64;
-        int nt = e.n64;
+        const TileF64 *tl = e.d_tilesF;
+        int nt = e.nF;
         void *args[] = {&probs, &tl, &nt};
         FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_fp64_step),
-                                std::max(1, std::min(e.n64, 4 * ctx->num_sms)), 256, 0, args, nullptr, &kn));
+                                std::max(1, std::min(e.nF, 8 * ctx->num_sms)), 256, 0, args, nullptr, &kn));
     }
     if (e.any_digit) {
         cudaGraph_t ib;

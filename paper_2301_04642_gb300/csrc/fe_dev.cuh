@@ -103,9 +103,9 @@ constexpr int kHistCols = 6;
 // one or two FP16 slices per operand; kTcElem: no product, epilogue only;
 // kTcDelta: the second product of an FP64-accurate polishing pair, a split
 // product of small matrices added to the FP64 iterate), the FP64-accurate
-// SIMT kernel (kFp64 native, kDf double-float), or the FP64-accurate digit
+// SIMT kernel (kFp64), or the FP64-accurate digit
 // product on the tensor cores (kDigit).
-enum Kind : int { kNone = 0, kTcSingle = 1, kTcSplit = 2, kFp64 = 3, kDf = 4, kTcElem = 5,
+enum Kind : int { kNone = 0, kTcSingle = 1, kTcSplit = 2, kFp64 = 3, kTcElem = 5,
                   kDigit = 6, kTcDelta = 7 };
 enum Phase : int { kPhaseSingle = 0, kPhaseSplit = 1, kPhaseFp64 = 2, kPhaseDone = 3 };
 enum Prec : int { kPrecMixed = 0, kPrecFp64 = 1, kPrecFp32 = 2, kPrecTryFp16 = 3 };

@@ -36,7 +36,7 @@ struct MmaProb {
     SolveState *st;
     double *part;                    // per-tile partial slots (kPartStride doubles each)
     int n, ldy, lds, ntiles;         // ntiles: tensor-core tiles of the problem's tile width
-    int ntiles64, bn;                // bn: tensor-core tile width, 128 or 256 columns
+    int ntilesF, bn;                 // bn: tensor-core tile width, 128 or 256 columns
     int tc_tile0, tc_ntiles;         // this problem's range in the launch's tensor-core tile list
     float *lzv;                      // Lanczos vectors: v_prev, v, w (n FP32 each)
     float *Y;                        // FP32 master of the zero-temperature iterate
@@ -65,8 +65,8 @@ struct TileEnt {
 // A digit-product tile uses TileEnt with Jp = J: rows [I*128, +128) x
 // columns [J*64, +64), J >= 2I.
 
-// One FP64 tile: rows [I*64, +64) x columns [J*64, +64), J >= I.
-struct Tile64 {
+// One FP64 tile: rows [I*16, +16) x columns [J*16, +16), J >= I.
+struct TileF64 {
     int prob;
     int I;
     int J;
@@ -172,7 +172,7 @@ __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, S
                           cudaGraphConditionalHandle h_fp64, cudaGraphConditionalHandle h_digit,
                           unsigned hvalid);
 // FP64-accurate product + SP2 update (upper tiles, mirrored), per-tile partials.
-__global__ void k_fp64_step(const MmaProb *probs, const Tile64 *tiles, int ntiles);
+__global__ void k_fp64_step(const MmaProb *probs, const TileF64 *tiles, int ntiles);
 // D = X -> out (FP64, ld), partials of tr(H D) and tr D.
 __global__ void k_finalize(const MmaProb *probs, int prob, double *D, long long ldd);
 __global__ void k_finalize_reduce(const MmaProb *probs, int prob);
@@ -190,7 +190,7 @@ __global__ void k_make_slices(const float *Y, int n, int ldy, float s, __half *h
 
 constexpr int kInitBlocks = 608;   // 4 x 152 SMs (k_init_x0: 8 warps each, one row per warp)
 constexpr int kFinBlocks = 304;
-constexpr int kTile64 = 64;
+constexpr int kTileF64 = 16;
 
 // ---- products either side of the expansion in subspace iteration (k_gemm.cu)
 // C = A B^T from K-major FP16 slices (hi, lo), tiles 128 x kGemmN.

@@ -149,7 +149,7 @@ __device__ void control_sp2(SolveState *st, double trV, double sumsq, double rsq
         st->c = st->c_next;
         st->s_cur = st->s_next;
         st->cur ^= 1;
-    } else if (prev_kind == kFp64 || prev_kind == kDf || prev_kind == kDigit || prev_kind == kTcDelta) {
+    } else if (prev_kind == kFp64 || prev_kind == kDigit || prev_kind == kTcDelta) {
         st->xcur ^= 1;
         st->x_fp64 = 1;
     }
@@ -249,7 +249,7 @@ __device__ void control_sp2(SolveState *st, double trV, double sumsq, double rsq
             else phase = kPhaseFp64;
         }
     } else if (phase == kPhaseFp64 &&
-               (prev_kind == kFp64 || prev_kind == kDf || prev_kind == kDigit || prev_kind == kTcDelta)) {
+               (prev_kind == kFp64 || prev_kind == kDigit || prev_kind == kTcDelta)) {
         const int nfp64 = st->it_phase[kPhaseFp64];
         if (st->prec == kPrecFp64) {
             const bool idem_ok = fabs(idem) <= 2e-10 ||
@@ -445,7 +445,7 @@ __device__ void control_trfoe(SolveState *st, double trV, double sumsq) {
         st->c = st->c_next;
         st->s_cur = st->s_next;
         st->cur ^= 1;
-    } else if (prev_kind == kFp64 || prev_kind == kDf || prev_kind == kDigit) {
+    } else if (prev_kind == kFp64 || prev_kind == kDigit) {
         st->xcur ^= 1;
         st->x_fp64 = 1;
     }
@@ -982,7 +982,7 @@ __device__ void control_one(const MmaProb &pr, const DevCtl *ctl) {
     // number of partial slots written by the previous producer
     int nparts;
     if (st->kind == kNone) nparts = kInitBlocks;
-    else if (st->kind == kFp64 || st->kind == kDf) nparts = pr.ntiles64;
+    else if (st->kind == kFp64) nparts = pr.ntilesF;
     else if (st->kind == kDigit) nparts = pr.ntilesD;
     else nparts = pr.ntiles;
 
@@ -1045,7 +1045,7 @@ __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, S
         if (!*reinterpret_cast<const volatile int *>(&st->done)) {
             bits |= kStepActive;
             if (kind == kTcSingle || kind == kTcSplit || kind == kTcElem || kind == kTcDelta) bits |= kStepTc;
-            if (kind == kFp64 || kind == kDf) bits |= kStepFp64;
+            if (kind == kFp64) bits |= kStepFp64;
             if (kind == kDigit) bits |= kStepDigit;
         }
     }
