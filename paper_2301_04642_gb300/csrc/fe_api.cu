@@ -1915,7 +1915,7 @@ int run_gemm(fe_ctx *ctx, const GemmArgs &ga, const std::vector<TileEnt> &tl, co
     ctx->launches += 1;
     FE_CUDA(ctx, cudaEventRecord(eg.ev_loop, q));
     if (ga.nsplit > 0) {
-        k_gemm_reduce<<<ga.ntiles, 256, 0, q>>>(ctx->d_gargs, ctx->d_gtiles);
+        k_gemm_reduce<<<dim3(ga.ntiles, kGemmN / 16), 256, 0, q>>>(ctx->d_gargs, ctx->d_gtiles);
         ctx->launches += 1;
     }
     FE_CUDA(ctx, cudaEventRecord(eg.ev1, q));
