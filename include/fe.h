@@ -198,10 +198,13 @@ FE_API int fe_submit(fe_ctx *ctx, const fe_problem *p, fe_ticket *t);
 FE_API int fe_poll(fe_ctx *ctx, fe_ticket t, fe_result *r);
 
 /* Tile-shape autotuner.  The split-FP16 / single-FP16 symmetric products
- * (Sec. III-B: the matrix product is the cost) run over upper-triangle tiles of
- * 128 x 256 or 128 x 128 elements.  Wide tiles halve the operand traffic per
+ * (Sec. III-B: the matrix product is the cost) run over upper-triangle tiles up
+ * to 256 or 128 columns wide; the library itself chooses narrower ones (down to
+ * 32) where a launch has few tiles.  Wide tiles halve the operand traffic per
  * flop; narrow ones waste less work at the diagonal and the ragged edge and
- * give more tiles to balance over the SMs, which pays for small n.  The
+ * give more tiles to balance over the SMs, which pays for small n.  The width
+ * also places the cut of a tile's K sum, so results differ in their last bits
+ * between the two.  The
  * context keeps a table from (number of 128-row panels, precision policy) to
  * the width; a problem uses the entry for its panel count, else the nearest
  * one under its policy, else 256.  Problems of different widths share one

@@ -100,13 +100,13 @@ FE_API int fe_k_narrow_bounds(fe_ctx *ctx, double factor);
 
 /* Failure-detection hook (no counterpart in the paper).  Every wait inside
  * the tensor-core kernels (TMA data, shared-memory stages, tensor-memory
- * hand-offs, the partner of a tile split between two CTAs) is bounded: when
+ * hand-offs, the meetings of all CTAs between two steps) is bounded: when
  * one runs out the kernel records an error code, waits (bounded) for its own
  * copies and products in flight, frees its tensor memory and returns; the
  * control kernel then ends every problem of the run, and the call returns
  * FE_ETIMEOUT with the context still usable.  This sets the limit of those
  * waits for later solves on ctx (limit_ms, default 2000) and, with
- * fail_partner != 0, makes the second CTA of every split tile wait on a word
+ * fail_partner != 0, makes the meetings of all CTAs in k_sym_mma watch a word
  * that nothing writes, so that its wait runs out: a way to exercise the
  * expiry path without any fault.  Call it while no submitted solve runs.
  * Errors: FE_EINVAL (ctx NULL, limit_ms outside (0, 60000]), FE_ECUDA. */

@@ -411,7 +411,7 @@ class Context:
 
     def set_wait(self, limit_ms=2000.0, fail_partner=False):
         """Failure-detection hook: the limit of the kernels' bounded waits and
-        the test word that makes the split-tile partner wait run out."""
+        the test word that makes the step kernel's meetings of all CTAs run out."""
         rc = self.L.fe_k_set_wait(self.h, float(limit_ms), 1 if fail_partner else 0)
         if rc != FE_OK:
             raise FeError(rc, self.last_error())

@@ -72,8 +72,7 @@ struct Slot {
     RowInfo *rowinfo = nullptr;
     int *bad = nullptr;
     int ldy = 0, lds = 0, ldx = 0;
-    std::vector<TileEnt> tiles;   // tensor-core tiles 128 x 256
-    std::vector<TileEnt> tilesN;  // tensor-core tiles 128 x 128
+    std::map<std::pair<int, int>, std::vector<TileEnt>> tiles;  // tensor-core tiles by widths, listed when first needed
     std::vector<TileF64> tilesF;  // FP64 tiles, listed when the FP64 schedule first needs them
     std::vector<TileEnt> tilesD;  // digit-product tiles (zero temperature)
     MmaProb hp;  // host image of the device descriptor (H filled per solve)
@@ -103,14 +102,13 @@ struct Engine {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaEvent_t ev_setup = nullptr, ev_loop = nullptr;  // end of set-up, end of the step loop
     int ntc = 0, nF = 0, nD = 0;    // tile counts of the uploaded lists
-    bool any_tc = false, any_fp64 = false, any_digit = false;
-    // the step loop as a CUDA graph: WHILE(any problem active) { IF(tc) k_sym_mma;
-    // IF(fp64) k_fp64_step; IF(digit) k_digit_prep, k_digit_mma; k_control }
+    bool any_tc = false, any_fp64 = false, any_digit = false, any_fermi = false;
+    // the step loop as a CUDA graph (eng_graph)
     StepFlags *d_flags = nullptr;
     StepFlags h_flags{};
-    // Stream-K hand-off of split tiles in k_sym_mma: one slot and two counters per SM
-    float *d_skws = nullptr;
-    int *d_skcnt = nullptr;
+    float *d_runs = nullptr;         // k_sym_mma: first-run sums of cut tiles, one slot per CTA
+    char *d_sched = nullptr;         // k_sym_mma: schedule rows of tables beyond kSchedTabProbs problems
+    size_t sched_cap = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     std::vector<uintptr_t> gkey;     // what the instantiated graph was built for
@@ -136,7 +134,7 @@ struct Req {
     bool accel_off = false;         // FE_METHOD_ASP2 estimates proved inconsistent: plain SP2
     bool deferred = false;          // waited at least once for a free part of the HBM budget
     int wasted = 0;                 // products of attempts that were started again
-    int bn = 0;                     // tensor-core tile width, fixed when the solve starts
+    int bn = 0, bn2 = 0, ref_bn = 0;  // tensor-core tile widths, fixed when the solve starts
     bool done = false;
     fe_result res{};
     std::chrono::steady_clock::time_point t_submit;
@@ -151,6 +149,7 @@ struct fe_ctx {
     uint32_t prec_default = FE_PREC_MIXED;
     int num_sms = 148;
     int lz_grid = 0;                 // blocks of the cooperative Lanczos launch (all resident)
+    int sym_grid = 0;                // CTAs of a k_sym_mma launch (resident pairs)
     Engine eng;                      // blocking solves and batches
     std::mutex smu;                  // slots, used
     std::vector<Slot *> slots;
@@ -230,26 +229,53 @@ void push_banded(std::vector<TileEnt> &out, int nI, int nJ, int band, Jmin jmin)
         const int b1 = std::min(nI, b0 + band);
         for (int J = jmin(b0); J < nJ; ++J)
             for (int I = b0; I < b1; ++I)
-                if (J >= jmin(I)) out.push_back(TileEnt{0, I, J, row0[I] + J - jmin(I)});
+                if (J >= jmin(I)) out.push_back(TileEnt{0, I, J, row0[I] + J - jmin(I), 0});
     }
 }
 
-// 128-row panels per band: the tensor-core tiles read 128 x K and 256 x K
-// (or 128 x K) panels (two FP16 slices each), the digit tiles 128 x K and
-// 64 x K panels of seven digits; the bands balance row-panel and column-panel
-// bytes over a wave of about 150 tiles.
-constexpr int kBandTc = 16, kBandTcN = 12, kBandDigit = 8;
+// Row panels per band: the tensor-core tiles read 256 x K and bn x K panels
+// (two FP16 slices each), the digit tiles 128 x K and 64 x K panels of seven
+// digits; the bands balance row-panel and column-panel bytes over a wave of
+// about 76 (150) tiles.
+constexpr int kBandTc = 8, kBandDigit = 8;
+constexpr int kWidths[4] = {256, 128, 64, 32};
+
+// Tensor-core tiles of width bn of an n x n product, and their list.
+int64_t num_tiles_tc(int64_t n, int bn) {
+    const int64_t P = (n + 255) / 256, C = (n + bn - 1) / bn, step = 256 / bn;
+    return P * C - step * (P * (P - 1) / 2);
+}
+
+// Tiles of width bn; with bn2 < bn those beyond the last whole round over `pairs`
+// CTA pairs are cut into tiles of width bn2.
+const std::vector<TileEnt> &tiles_tc(Slot *s, int bn, int bn2, int pairs) {
+    std::vector<TileEnt> &t = s->tiles[{bn, bn2}];
+    if (!t.empty()) return t;
+    push_banded(t, ceil_div(s->n, 256), ceil_div(s->n, bn), kBandTc, [&](int I) { return I * (256 / bn); });
+    for (TileEnt &e : t) e.bn = bn;
+    if (bn2 >= bn) return t;
+    const size_t whole = t.size() / pairs * pairs;
+    const std::vector<TileEnt> rest(t.begin() + whole, t.end());
+    t.resize(whole);
+    for (TileEnt e : rest)
+        for (int x = 0; x < bn / bn2; ++x)
+            if ((e.Jp * (bn / bn2) + x) * bn2 < s->n) t.push_back(TileEnt{0, e.I, e.Jp * (bn / bn2) + x, 0, bn2});
+    for (size_t k = 0; k < t.size(); ++k) t[k].slot = static_cast<int>(k);
+    return t;
+}
+
+// Reference tiles of width ref_bn (256 or 128) x 128 rows.
+int num_tiles_ref(int n, int ref_bn) {
+    const int T = ceil_div(n, kTileM);
+    int c = 0;
+    for (int I = 0; I < T; ++I) c += (ref_bn == kTileM) ? T - I : ceil_div(T, 2) - I / 2;
+    return c;
+}
 
 void build_tiles(Slot *s) {
-    const int T = ceil_div(s->n, kTileM);
-    const int TP = ceil_div(T, 2);
-    push_banded(s->tiles, T, TP, kBandTc, [](int I) { return I / 2; });
-    push_banded(s->tilesN, T, T, kBandTcN, [](int I) { return I; });
     s->tilesD.clear();
-    if (s->method == kMethodSp2) {
-        const int TD = ceil_div(s->n, kDigitN);
-        push_banded(s->tilesD, T, TD, kBandDigit, [](int I) { return 2 * I; });
-    }
+    if (s->method == kMethodSp2)
+        push_banded(s->tilesD, ceil_div(s->n, kTileM), ceil_div(s->n, kDigitN), kBandDigit, [](int I) { return 2 * I; });
 }
 
 // Upper-triangle FP64 tiles of an n x n product.
@@ -278,7 +304,7 @@ size_t slot_bytes(int n, int method, int *ldy, int *lds, int *ldx, size_t *npart
     *lds = static_cast<int>(align_up(n, 8));
     *ldx = n;
     const int T = ceil_div(n, kTileM);
-    const size_t ntiles = static_cast<size_t>(T) * (T + 1) / 2;  // >= T ceil(T/2): either width
+    const size_t ntiles = 2 * static_cast<size_t>(num_tiles_tc(n, 32));  // the narrowest width has most
     const size_t ntF = method == kMethodSp2 ? static_cast<size_t>(num_tiles_f64(n)) : 0;
     const size_t TD = static_cast<size_t>(ceil_div(n, kDigitN));
     size_t ntD = 0;
@@ -297,7 +323,10 @@ size_t slot_bytes(int n, int method, int *ldy, int *lds, int *ldx, size_t *npart
     add(8 * 3 * nn);                                 // Lanczos vectors
     if (method == kMethodSp2)
         for (int a = 0; a < kDigits; ++a) add(2 * nn * (*lds));  // digits of X/4
-    if (method == kMethodFermi) add(12 * kNumMats * align_up(nn, 8));  // FP64 diagonals + FP32 copies
+    if (method == kMethodFermi) {
+        add(12 * kNumMats * align_up(nn, 8));             // FP64 diagonals + FP32 copies
+        add(4 * ((nn + 7) / 8) * align_up(nn, 32));       // 8-column sums (MmaProb::rsum)
+    }
     add(8 * kPartStride * (*nparts));                // partials
     add(sizeof(SolveState));
     add(sizeof(RowInfo) * nn);
@@ -415,6 +444,8 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
         for (int a = 0; a < kDigits; ++a) digs[a] = reinterpret_cast<__half *>(take(2 * nn * lds));
     const size_t dstride = align_up(nn, 8);  // 64-byte aligned vectors
     double *diags = (method == kMethodFermi) ? reinterpret_cast<double *>(take(12 * kNumMats * dstride)) : nullptr;
+    const size_t ldr = align_up(nn, 32);
+    float *rsum = (method == kMethodFermi) ? reinterpret_cast<float *>(take(4 * ((nn + 7) / 8) * ldr)) : nullptr;
     s->part = reinterpret_cast<double *>(take(8 * kPartStride * nparts));
     s->st = reinterpret_cast<SolveState *>(take(sizeof(SolveState)));
     s->rowinfo = reinterpret_cast<RowInfo *>(take(sizeof(RowInfo) * nn));
@@ -425,8 +456,10 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
     for (int m = 0; m < num_slice_sets(method); ++m) {
         MatSlot &ms = s->hp.mats[m];
         for (int b = 0; b < kMaxSlices; ++b) {
-            int rc = encode_map(ctx, &ms.tmA[b], slices[m][b], n, lds, kTileM);
-            if (rc == FE_OK) rc = encode_map(ctx, &ms.tmB[b], slices[m][b], n, lds, kTileN);
+            int rc = encode_map(ctx, &ms.tm128[b], slices[m][b], n, lds, 128);
+            if (rc == FE_OK) rc = encode_map(ctx, &ms.tm64[b], slices[m][b], n, lds, 64);
+            if (rc == FE_OK) rc = encode_map(ctx, &ms.tm32[b], slices[m][b], n, lds, 32);
+            if (rc == FE_OK) rc = encode_map(ctx, &ms.tm16[b], slices[m][b], n, lds, 16);
             if (rc != FE_OK) {
                 free_slot(ctx, s);
                 return rc;
@@ -469,8 +502,9 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
     s->hp.n = n;
     s->hp.ldy = ldy;
     s->hp.lds = lds;
-    s->hp.ntiles = static_cast<int>(s->tiles.size());
-    s->hp.bn = kTileN;
+    s->hp.ref_bn = kTileN;
+    s->hp.rsum = rsum;
+    s->hp.ldr = static_cast<int>(ldr);
     s->hp.ntilesF = static_cast<int>(num_tiles_f64(n));
     s->hp.ntilesD = static_cast<int>(s->tilesD.size());
     s->hp.lzv = s->lzv;
@@ -536,6 +570,14 @@ int slot_method(const fe_problem *p) { return method_of(p) == kMethodFermi ? kMe
 // doubling (square, Newton-Schulz pairs, final product) for up to ~40
 // doublings, plus the shift-only refinements.
 constexpr int kFermiMaxSteps = 640;
+
+// Time of one tensor-core tile in clocks, as tile_cost estimates it (fitted to
+// step times at n = 200 to 8192 with every width).
+constexpr double kCostChunkMma = 8.0;     // one chunk, per column: MMAs and their hand-over
+constexpr double kCostChunkMin = 1200.0;  // ... at least: the hand-over's latency
+constexpr double kCostChunkCol = 1.5;     // ... growing a little with the columns
+constexpr double kCostTile = 10000.0;     // fill, hand-offs, partials
+constexpr double kCostStore = 230.0;      // store phase, per column
 
 int validate(fe_ctx *ctx, const fe_problem *p) {
     if (!p) return set_err(ctx, FE_EINVAL, "problem is NULL");
@@ -630,7 +672,7 @@ struct Job {
     int64_t ldstage = 0;
     bool lanczos = true;            // estimate the spectral bounds (else Gershgorin)
     bool accel = true;              // FE_METHOD_ASP2: folds on (off after an inconsistent attempt)
-    int bn = 0;                     // tensor-core tile width, fixed for the whole solve (0: look up)
+    int bn = 0, bn2 = 0, ref_bn = 0;  // tensor-core tile widths (tiles_tc), reference tile width (0: choose)
 };
 
 Job make_job(const fe_problem *p, Slot *s) {
@@ -677,9 +719,7 @@ int eng_init(fe_ctx *ctx, Engine &e, cudaStream_t user_stream) {
     }
     FE_CUDA(ctx, cudaMalloc(&e.d_flags, sizeof(StepFlags)));
     FE_CUDA(ctx, cudaMemset(e.d_flags, 0, sizeof(StepFlags)));
-    FE_CUDA(ctx, cudaMalloc(&e.d_skws, sizeof(float) * kSkSlotFloats * ctx->num_sms));
-    FE_CUDA(ctx, cudaMalloc(&e.d_skcnt, sizeof(int) * 2 * ctx->num_sms));
-    FE_CUDA(ctx, cudaMemset(e.d_skcnt, 0, sizeof(int) * 2 * ctx->num_sms));
+    FE_CUDA(ctx, cudaMalloc(&e.d_runs, sizeof(float) * kRunSlotFloats * ctx->num_sms));
     FE_CUDA(ctx, cudaEventCreate(&e.ev0));
     FE_CUDA(ctx, cudaEventCreate(&e.ev1));
     FE_CUDA(ctx, cudaEventCreate(&e.ev_setup));
@@ -692,8 +732,8 @@ void eng_free(Engine &e) {
     if (e.gexec) cudaGraphExecDestroy(e.gexec);
     if (e.graph) cudaGraphDestroy(e.graph);
     if (e.d_flags) cudaFree(e.d_flags);
-    if (e.d_skws) cudaFree(e.d_skws);
-    if (e.d_skcnt) cudaFree(e.d_skcnt);
+    if (e.d_runs) cudaFree(e.d_runs);
+    if (e.d_sched) cudaFree(e.d_sched);
     if (e.d_err) cudaFree(e.d_err);
     if (e.d_probs) cudaFree(e.d_probs);
     if (e.d_tiles) cudaFree(e.d_tiles);
@@ -710,13 +750,81 @@ void eng_free(Engine &e) {
     e = Engine();
 }
 
-int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
+// Tile fields of a table entry.
+void set_tiles(MmaProb *hp, const std::vector<TileEnt> &tl, int ref_bn) {
+    hp->ref_bn = ref_bn;
+    hp->tc_ntiles = static_cast<int>(tl.size());
+    hp->ntiles = 2 * hp->tc_ntiles;
+    hp->ref_ntiles = num_tiles_ref(hp->n, ref_bn);
+}
+
+// Cost of one tensor-core tile of an n x n product in clocks: its K loop (MMAs, or
+// the hand-over of its chunks where that takes longer) and its store phase.
+double tile_cost(int64_t n, int bn) {
+    const double chunks = static_cast<double>((n + kTileK - 1) / kTileK);
+    return chunks * std::max(kCostChunkMin + kCostChunkCol * bn, kCostChunkMma * bn) + kCostTile + kCostStore * bn;
+}
+
+// Tile widths of a table's problems that have none yet.  Equal tiles run in whole
+// rounds over the CTA pairs.  Few tiles: narrower ones shorten every CTA's share;
+// many: wide ones take in fewer bytes per product and store better.  A problem
+// alone in its table runs its whole rounds in wide tiles and may cut what is left
+// over into narrower ones (n = 3000, 78 wide tiles for 76 pairs: 206 us a step in
+// two rounds, 176 with the two left over cut up).  The tile-shape table caps the
+// width (ref_bn).
+void choose_widths(fe_ctx *ctx, std::vector<Job> &jobs) {
+    const int pairs = ctx->sym_grid / 2;
+    for (Job &j : jobs)
+        if (!j.ref_bn) j.ref_bn = tile_width(ctx, j.p->n, prec_of(ctx, j.p));
+    if (jobs.size() == 1 && !jobs[0].bn) {
+        Job &j = jobs[0];
+        const int64_t n = j.p->n;
+        double best = DBL_MAX;
+        for (int bn : kWidths)
+            for (int bn2 : kWidths) {
+                if (bn > j.ref_bn || bn2 > bn) continue;
+                const int64_t c = num_tiles_tc(n, bn), rest = c % pairs;
+                const int64_t r2 = (rest * (bn / bn2) + pairs - 1) / pairs;  // rounds of the narrower tiles
+                const double cost = static_cast<double>(c / pairs) * tile_cost(n, bn) + r2 * tile_cost(n, bn2);
+                if (cost < best) {
+                    best = cost;
+                    j.bn = bn;
+                    j.bn2 = bn2;
+                }
+            }
+        return;
+    }
+    int width = kWidths[0];
+    double best = DBL_MAX;
+    for (int w : kWidths) {
+        double work = 0.0, longest = 0.0;
+        for (const Job &j : jobs) {
+            const int bn = j.bn ? j.bn : std::min(j.ref_bn, w);
+            const double t = tile_cost(j.p->n, bn);
+            work += t * static_cast<double>(num_tiles_tc(j.p->n, bn));
+            longest = std::max(longest, t);
+        }
+        // the tiles run largest first and end within about half a tile
+        const double cost = std::max(work / pairs + 0.5 * longest, longest);
+        if (cost < best) {
+            best = cost;
+            width = w;
+        }
+    }
+    for (Job &j : jobs)
+        if (!j.bn) j.bn = j.bn2 = std::min(j.ref_bn, width);
+}
+
+// `jobs` get their tile widths here; a problem keeps its widths for the whole
+// solve (the control step reduces the partial slots of the last product's tiles).
+int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
     const int np = static_cast<int>(jobs.size());
+    choose_widths(ctx, jobs);
     std::vector<MmaProb> hprobs(np);
     std::vector<TileEnt> tiles;
     std::vector<TileF64> tilesF;
     std::vector<TileEnt> tilesD;
-    e.any_tc = e.any_fp64 = e.any_digit = false;
+    e.any_tc = e.any_fp64 = e.any_digit = e.any_fermi = false;
     e.offF.assign(np, 0);
     e.cntF.assign(np, 0);
     for (int k = 0; k < np; ++k) {
@@ -725,20 +833,16 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
         hprobs[k].H = j.H;
         hprobs[k].ldh = j.ldh;
         const bool fermi = method_of(j.p) == kMethodFermi;
+        e.any_fermi = e.any_fermi || fermi;
         const bool trfoe = method_of(j.p) == kMethodTrfoe;  // its FP64 schedule runs digit products
         const uint32_t pr = prec_of(ctx, j.p);
         hprobs[k].tc_tile0 = static_cast<int>(tiles.size());
         hprobs[k].tc_ntiles = 0;
         if (pr != FE_PREC_FP64 || fermi) {
             e.any_tc = true;
-            // a problem keeps its width for the whole solve: the control step
-            // reduces the partial slots of the previous product's tiles
-            const int bn = j.bn ? j.bn : tile_width(ctx, j.p->n, pr);
-            const std::vector<TileEnt> &tl = (bn == kTileM) ? j.slot->tilesN : j.slot->tiles;
+            const std::vector<TileEnt> &tl = tiles_tc(j.slot, j.bn, j.bn2, ctx->sym_grid / 2);
             for (TileEnt t : tl) { t.prob = k; tiles.push_back(t); }
-            hprobs[k].tc_ntiles = static_cast<int>(tl.size());
-            hprobs[k].ntiles = static_cast<int>(tl.size());
-            hprobs[k].bn = bn;
+            set_tiles(&hprobs[k], tl, j.ref_bn);
         }
         e.offF[k] = static_cast<int>(tilesF.size());
         e.cntF[k] = 0;
@@ -757,6 +861,8 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
     if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tiles, &e.tiles_cap, tiles.size());
     if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tilesF, &e.tilesF_cap, tilesF.size());
     if (rc == FE_OK) rc = ensure_dev(ctx, &e.d_tilesD, &e.tilesD_cap, tilesD.size());
+    if (rc == FE_OK && np > kSchedTabProbs)
+        rc = ensure_dev(ctx, &e.d_sched, &e.sched_cap, sched_row_bytes() * np * ctx->sym_grid);
     if (rc == FE_OK) rc = ensure_pinned(ctx, &e.h_states, &e.h_states_cap, np);
     if (rc == FE_OK) rc = ensure_pinned(ctx, &e.h_done, &e.h_done_cap, np + 1);  // + error word
     if (rc != FE_OK) return rc;
@@ -777,6 +883,32 @@ int eng_upload(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs) {
     e.nF = static_cast<int>(tilesF.size());
     e.nD = static_cast<int>(tilesD.size());
     return FE_OK;
+}
+
+// Launch k_sym_mma over a table: one step, or (cooperatively, so that all its
+// CTAs are resident and can meet) up to max_steps with their control steps.
+cudaError_t launch_sym(fe_ctx *ctx, Engine &e, const MmaProb *probs, int np, int max_steps) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctx->sym_grid);
+    cfg.blockDim = dim3(kSymThreads);
+    cfg.dynamicSmemBytes = mma_smem_bytes();
+    cfg.stream = e.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = max_steps > 1 ? 1 : 0;
+    ctx->launches += 1;
+    return cudaLaunchKernelEx(&cfg, k_sym_mma, probs, np, static_cast<const TileEnt *>(e.d_tiles), e.d_err, e.d_runs,
+                              e.d_sched, static_cast<StepFlags *>(nullptr), ctx->num_sms, max_steps);
+}
+
+// The error word and the meeting counter of k_sym_mma, cleared before each run.
+cudaError_t clear_ctl(Engine &e) {
+    cudaError_t r = cudaMemsetAsync(&e.d_err->err, 0, sizeof(int), e.stream);
+    if (r == cudaSuccess) r = cudaMemsetAsync(&e.d_err->hold, 0, sizeof(int), e.stream);
+    if (r == cudaSuccess) r = cudaMemsetAsync(&e.d_err->sym_bar, 0, sizeof(unsigned), e.stream);
+    return r;
 }
 
 // Set-up of the problems at table positions [k0, k1): Hp staging, initial
@@ -841,21 +973,17 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
                                                  cudaMemcpyDeviceToDevice, s));
                 tab = e.d_chk;
             }
-            k_control<<<nt, 256, 0, s>>>(tab, nt, e.d_err, nullptr, 0, 0, 0, 0, 0u);
-            for (int c = 0; c < kCheckSteps; ++c) {
-                k_sym_mma<<<ctx->num_sms, kSymThreads, mma_smem_bytes(), s>>>(tab, nt, e.d_tiles, e.ntc, e.d_err,
-                                                                           e.d_skws, e.d_skcnt);
-                k_control<<<nt, 256, 0, s>>>(tab, nt, e.d_err, nullptr, 0, 0, 0, 0, 0u);
-            }
-            ctx->launches += 1 + 2 * kCheckSteps;
+            k_control<<<nt, 256, 0, s>>>(tab, nt, e.d_err, nullptr, 0, 0, 0);
+            FE_CUDA(ctx, launch_sym(ctx, e, tab, nt, kCheckSteps + 1));
+            ctx->launches += 1;
         }
         for (int k : f64_chk) {
             const MmaProb *one = e.d_probs + k;
-            k_control<<<1, 256, 0, s>>>(one, 1, e.d_err, nullptr, 0, 0, 0, 0, 0u);
+            k_control<<<1, 256, 0, s>>>(one, 1, e.d_err, nullptr, 0, 0, 0);
             for (int c = 0; c < kCheckSteps; ++c) {
                 k_fp64_step<<<std::max(1, std::min(e.cntF[k], 8 * ctx->num_sms)), 256, 0, s>>>(
-                    e.d_probs, e.d_tilesF + e.offF[k], e.cntF[k]);
-                k_control<<<1, 256, 0, s>>>(one, 1, e.d_err, nullptr, 0, 0, 0, 0, 0u);
+                    e.d_probs, e.d_tilesF + e.offF[k], e.cntF[k], e.d_err);
+                k_control<<<1, 256, 0, s>>>(one, 1, e.d_err, nullptr, 0, 0, 0);
             }
             ctx->launches += 1 + 2 * kCheckSteps;
         }
@@ -865,7 +993,7 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
         for (int k : f64_chk) k_init_x0<<<kInitBlocks, 256, 0, s>>>(e.d_probs, k);
         ctx->launches += static_cast<long long>(tc_chk.size() + f64_chk.size());
     }
-    k_control<<<m, 256, 0, s>>>(e.d_probs + k0, m, e.d_err, nullptr, 0, 0, 0, 0, 0u);
+    k_control<<<m, 256, 0, s>>>(e.d_probs + k0, m, e.d_err, nullptr, 0, 0, 0);
     ++ctx->launches;
     // the state images must stay valid until their copies ran
     FE_CUDA(ctx, cudaStreamSynchronize(s));
@@ -876,31 +1004,31 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
 // tensor-core and FP64 launch is bracketed by events (4 per step).
 void eng_steps(fe_ctx *ctx, Engine &e, int np, int count, const std::vector<cudaEvent_t> *pev) {
     cudaStream_t s = e.stream;
-    const int grid_tc = ctx->num_sms;  // the kernel itself uses at most (work / largest tile) CTAs
     const int grid_f = std::max(1, std::min(e.nF, 8 * ctx->num_sms));
-    const size_t smem = mma_smem_bytes();
     const int grid_d = std::max(1, std::min(e.nD, ctx->num_sms));
     for (int it = 0; it < count; ++it) {
         if (pev) cudaEventRecord((*pev)[4 * it + 0], s);
         if (e.any_tc) {
-            k_sym_mma<<<grid_tc, kSymThreads, smem, s>>>(e.d_probs, np, e.d_tiles, e.ntc, e.d_err, e.d_skws,
-                                                          e.d_skcnt);
-            ++ctx->launches;
+            launch_sym(ctx, e, e.d_probs, np, 1);
+            if (e.any_fermi) {
+                k_ref_sums<<<ctx->num_sms, kEpiWarps * 32, 0, s>>>(e.d_probs, np);
+                ++ctx->launches;
+            }
         }
         if (pev) cudaEventRecord((*pev)[4 * it + 1], s);
         if (pev) cudaEventRecord((*pev)[4 * it + 2], s);
         if (e.any_fp64) {
-            k_fp64_step<<<grid_f, 256, 0, s>>>(e.d_probs, e.d_tilesF, e.nF);
+            k_fp64_step<<<grid_f, 256, 0, s>>>(e.d_probs, e.d_tilesF, e.nF, e.d_err);
             ++ctx->launches;
         }
         if (e.any_digit) {
-            k_digit_prep<<<2 * ctx->num_sms, 256, 0, s>>>(e.d_probs, np);
+            k_digit_prep<<<2 * ctx->num_sms, 256, 0, s>>>(e.d_probs, np, e.d_err);
             k_digit_mma<<<grid_d, kMmaThreads, digit_smem_bytes(), s>>>(e.d_probs, e.d_tilesD, e.nD,
                                                                         e.d_err);
             ctx->launches += 2;
         }
         if (pev) cudaEventRecord((*pev)[4 * it + 3], s);
-        k_control<<<np, 256, 0, s>>>(e.d_probs, np, e.d_err, nullptr, 0, 0, 0, 0, 0u);
+        k_control<<<np, 256, 0, s>>>(e.d_probs, np, e.d_err, nullptr, 0, 0, 0);
         ++ctx->launches;
     }
 }
@@ -961,17 +1089,18 @@ void fill_result(const SolveState &st, int herr, double ms, fe_result &r) {
     r.ms = ms;
 }
 
-// The step loop of the uploaded table as an instantiated CUDA graph (built
-// once per table layout): the control kernel sets the loop condition and the
-// kernel switches of the next step on the device, so exactly the steps and
-// kernels that have work run, with no host round trip.
+// The step loop of the uploaded table as an instantiated CUDA graph (built once
+// per table layout), with no host round trip:
+//   WHILE(any problem active) { IF(tensor-core work) k_sym_mma, which runs
+//     products and their control steps until another family is due;
+//     k_fp64_step; k_digit_prep, k_digit_mma; k_control }
 int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     std::vector<uintptr_t> key = {reinterpret_cast<uintptr_t>(e.d_probs), reinterpret_cast<uintptr_t>(e.d_tiles),
                                   reinterpret_cast<uintptr_t>(e.d_tilesF), reinterpret_cast<uintptr_t>(e.d_tilesD),
                                   static_cast<uintptr_t>(np), static_cast<uintptr_t>(e.ntc),
                                   static_cast<uintptr_t>(e.nF), static_cast<uintptr_t>(e.nD),
                                   static_cast<uintptr_t>(e.any_tc), static_cast<uintptr_t>(e.any_fp64),
-                                  static_cast<uintptr_t>(e.any_digit)};
+                                  static_cast<uintptr_t>(e.any_digit), reinterpret_cast<uintptr_t>(e.d_sched)};
     if (e.gexec && key == e.gkey) return FE_OK;
     if (e.gexec) cudaGraphExecDestroy(e.gexec);
     if (e.graph) cudaGraphDestroy(e.graph);
@@ -981,24 +1110,9 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     cudaGraph_t g;
     FE_CUDA(ctx, cudaGraphCreate(&g, 0));
     e.graph = g;
-    cudaGraphConditionalHandle hl = 0, ht = 0, hf = 0, hd = 0;
-    // defaults: the first step runs every kernel family (each skips problems
-    // whose step is not its own); later steps follow the control kernel.
-    // A handle exists only for a family the graph contains.
-    unsigned hvalid = kStepActive;
+    cudaGraphConditionalHandle hl = 0, ht = 0;
     FE_CUDA(ctx, cudaGraphConditionalHandleCreate(&hl, g, 1, cudaGraphCondAssignDefault));
-    if (e.any_tc) {
-        FE_CUDA(ctx, cudaGraphConditionalHandleCreate(&ht, g, 1, cudaGraphCondAssignDefault));
-        hvalid |= kStepTc;
-    }
-    if (e.any_fp64) {
-        FE_CUDA(ctx, cudaGraphConditionalHandleCreate(&hf, g, 1, cudaGraphCondAssignDefault));
-        hvalid |= kStepFp64;
-    }
-    if (e.any_digit) {
-        FE_CUDA(ctx, cudaGraphConditionalHandleCreate(&hd, g, 1, cudaGraphCondAssignDefault));
-        hvalid |= kStepDigit;
-    }
+    if (e.any_tc) FE_CUDA(ctx, cudaGraphConditionalHandleCreate(&ht, g, 1, cudaGraphCondAssignDefault));
     cudaGraphNodeParams wp = {};
     wp.type = cudaGraphNodeTypeConditional;
     wp.conditional.handle = hl;
@@ -1008,74 +1122,65 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     FE_CUDA(ctx, cudaGraphAddNode(&wn, g, nullptr, nullptr, 0, &wp));
     cudaGraph_t body = wp.conditional.phGraph_out[0];
     cudaGraphNode_t prev = nullptr;
-    // an IF node in the loop body after `prev`; returns its body graph
-    auto add_if = [&](cudaGraphConditionalHandle h, cudaGraph_t *ib) -> cudaError_t {
-        cudaGraphNodeParams ip = {};
-        ip.type = cudaGraphNodeTypeConditional;
-        ip.conditional.handle = h;
-        ip.conditional.type = cudaGraphCondTypeIf;
-        ip.conditional.size = 1;
-        cudaGraphNode_t in;
-        cudaError_t r = cudaGraphAddNode(&in, body, prev ? &prev : nullptr, nullptr, prev ? 1 : 0, &ip);
-        if (r == cudaSuccess) {
-            prev = in;
-            *ib = ip.conditional.phGraph_out[0];
-        }
-        return r;
-    };
     auto add_kernel = [&](cudaGraph_t gr, const void *fn, int grid, int block, size_t smem, void **args,
-                          cudaGraphNode_t *dep, cudaGraphNode_t *out) -> cudaError_t {
+                          cudaGraphNode_t dep, cudaGraphNode_t *out) -> cudaError_t {
         cudaKernelNodeParams kp = {};
         kp.func = const_cast<void *>(fn);
         kp.gridDim = dim3(grid);
         kp.blockDim = dim3(block);
         kp.sharedMemBytes = static_cast<unsigned>(smem);
         kp.kernelParams = args;
-        return cudaGraphAddKernelNode(out, gr, dep, dep ? 1 : 0, &kp);
+        return cudaGraphAddKernelNode(out, gr, dep ? &dep : nullptr, dep ? 1 : 0, &kp);
     };
     const MmaProb *probs = e.d_probs;
     DevCtl *err = e.d_err;
     cudaGraphNode_t kn, kn2;
     if (e.any_tc) {
-        cudaGraph_t ib;
-        FE_CUDA(ctx, add_if(ht, &ib));
+        cudaGraphNodeParams ip = {};
+        ip.type = cudaGraphNodeTypeConditional;
+        ip.conditional.handle = ht;
+        ip.conditional.type = cudaGraphCondTypeIf;
+        ip.conditional.size = 1;
+        FE_CUDA(ctx, cudaGraphAddNode(&prev, body, nullptr, nullptr, 0, &ip));
+        cudaGraph_t ib = ip.conditional.phGraph_out[0];
         const TileEnt *tl = e.d_tiles;
-        int nt = e.ntc, npp = np;
-        float *skws = e.d_skws;
-        int *skcnt = e.d_skcnt;
-        void *args[] = {&probs, &npp, &tl, &nt, &err, &skws, &skcnt};
-        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_sym_mma), ctx->num_sms, kSymThreads,
+        int npp = np, ref_ctas = ctx->num_sms, max_steps = INT_MAX;
+        float *runs = e.d_runs;
+        char *gsched = e.d_sched;
+        StepFlags *fl = e.d_flags;
+        void *args[] = {&probs, &npp, &tl, &err, &runs, &gsched, &fl, &ref_ctas, &max_steps};
+        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_sym_mma), ctx->sym_grid, kSymThreads,
                                 mma_smem_bytes(), args, nullptr, &kn));
+        cudaLaunchAttributeValue coop = {};
+        coop.cooperative = 1;
+        FE_CUDA(ctx, cudaGraphKernelNodeSetAttribute(kn, cudaLaunchAttributeCooperative, &coop));
     }
     if (e.any_fp64) {
-        cudaGraph_t ib;
-        FE_CUDA(ctx, add_if(hf, &ib));
         const TileF64 *tl = e.d_tilesF;
         int nt = e.nF;
-        void *args[] = {&probs, &tl, &nt};
-        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_fp64_step),
-                                std::max(1, std::min(e.nF, 8 * ctx->num_sms)), 256, 0, args, nullptr, &kn));
+        void *args[] = {&probs, &tl, &nt, &err};
+        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_fp64_step),
+                                std::max(1, std::min(e.nF, 8 * ctx->num_sms)), 256, 0, args, prev, &kn));
+        prev = kn;
     }
     if (e.any_digit) {
-        cudaGraph_t ib;
-        FE_CUDA(ctx, add_if(hd, &ib));
         int npp = np;
-        void *pargs[] = {&probs, &npp};
-        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_digit_prep), 2 * ctx->num_sms, 256, 0,
-                                pargs, nullptr, &kn));
+        void *pargs[] = {&probs, &npp, &err};
+        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_digit_prep), 2 * ctx->num_sms, 256, 0, pargs,
+                                prev, &kn));
         const TileEnt *tl = e.d_tilesD;
         int nt = e.nD;
         void *args[] = {&probs, &tl, &nt, &err};
-        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_digit_mma),
-                                std::max(1, std::min(e.nD, ctx->num_sms)), kMmaThreads, digit_smem_bytes(),
-                                args, &kn, &kn2));
+        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_digit_mma),
+                                std::max(1, std::min(e.nD, ctx->num_sms)), kMmaThreads, digit_smem_bytes(), args, kn,
+                                &kn2));
+        prev = kn2;
     }
     {
-        int npp = np;
+        int npp = np, has_tc = e.any_tc ? 1 : 0;
         StepFlags *fl = e.d_flags;
-        void *args[] = {&probs, &npp, &err, &fl, &hl, &ht, &hf, &hd, &hvalid};
-        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_control), np, 256, 0, args,
-                                prev ? &prev : nullptr, &kn));
+        void *args[] = {&probs, &npp, &err, &fl, &hl, &ht, &has_tc};
+        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_control), np, 256, 0, args, prev, &kn));
     }
     FE_CUDA(ctx, cudaGraphInstantiate(&e.gexec, g, 0));
     e.gkey = key;
@@ -1083,14 +1188,13 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
 }
 
 // Run validated problems on acquired slots to completion (blocking calls).
-int run_problems_once(fe_ctx *ctx, const std::vector<Job> &jobs, fe_result *rs) {
+int run_problems_once(fe_ctx *ctx, std::vector<Job> &jobs, fe_result *rs) {
     Engine &e = ctx->eng;
     const int np = static_cast<int>(jobs.size());
     cudaStream_t s = e.stream;
     int rc = eng_upload(ctx, e, jobs);
     if (rc != FE_OK) return rc;
-    FE_CUDA(ctx, cudaMemsetAsync(e.d_err, 0, sizeof(int), s));
-    FE_CUDA(ctx, cudaMemsetAsync(e.d_skcnt, 0, sizeof(int) * 2 * ctx->num_sms, s));
+    FE_CUDA(ctx, clear_ctl(e));
     FE_CUDA(ctx, cudaEventRecord(e.ev0, s));
     rc = eng_setup(ctx, e, jobs, 0, np);
     if (rc != FE_OK) return rc;
@@ -1134,13 +1238,13 @@ int run_problems_once(fe_ctx *ctx, const std::vector<Job> &jobs, fe_result *rs) 
     ctx->phase_ms[0] = ms_setup;
     ctx->phase_ms[1] = ms_loop;
     ctx->phase_ms[2] = ms_fin;
-    ctx->phase_ms[3] = use_graph ? static_cast<double>(e.h_flags.n_body) : static_cast<double>(nloop);
+    ctx->phase_ms[3] = use_graph ? static_cast<double>(e.h_flags.n_steps) : static_cast<double>(nloop);
     if (use_graph) {
-        // kernels the graph ran: a control per step, every family once in the
-        // first step, then the families the control kernel switched on
+        // kernels the graph ran: per pass a control and the other families' kernels
+        // (which leave at once when no problem is theirs); k_sym_mma when switched on
         const StepFlags &fl = e.h_flags;
-        ctx->launches += fl.n_body + (e.any_tc ? 1 : 0) + (e.any_fp64 ? 1 : 0) + (e.any_digit ? 2 : 0) +
-                         fl.n_tc + fl.n_fp64 + 2ll * fl.n_digit;
+        ctx->launches += static_cast<long long>(fl.n_ctl) * (1 + (e.any_fp64 ? 1 : 0) + (e.any_digit ? 2 : 0)) +
+                         (e.any_tc ? 1 + fl.n_tc : 0);
     }
     if (ctx->prof) {
         // launches that did work: the phases run in order (single FP16, split,
@@ -1206,7 +1310,7 @@ int run_problems_once(fe_ctx *ctx, const std::vector<Job> &jobs, fe_result *rs) 
 // whose HOMO/LUMO estimates proved inconsistent with its spectrum is solved
 // again as plain SP2 (at most one of each, in that order of discovery);
 // fe_result.iters then includes the products of the abandoned attempts.
-int run_problems(fe_ctx *ctx, const std::vector<Job> &jobs, fe_result *rs) {
+int run_problems(fe_ctx *ctx, std::vector<Job> &jobs, fe_result *rs) {
     int rc = run_problems_once(ctx, jobs, rs);
     std::vector<Job> cur = jobs;
     std::vector<int> where(jobs.size());
@@ -1297,6 +1401,8 @@ Job job_of(Req *r) {
     j.lanczos = !r->gershgorin && method_of(&r->p) != kMethodTrfoe;
     j.accel = !r->accel_off;
     j.bn = r->bn;
+    j.bn2 = r->bn2;
+    j.ref_bn = r->ref_bn;
     return j;
 }
 
@@ -1330,7 +1436,6 @@ void serve_loop(fe_ctx *ctx) {
                 }
                 r->slot = s;
             }
-            if (r->bn == 0) r->bn = tile_width(ctx, r->p.n, prec_of(ctx, &r->p));
             started.push_back(r);
         }
         if (!started.empty() || !failed.empty()) {
@@ -1362,10 +1467,14 @@ void serve_loop(fe_ctx *ctx) {
         for (Req *r : all) jobs.push_back(job_of(r));
         const int np = static_cast<int>(all.size());
         int rc = FE_OK;
-        cudaMemsetAsync(e.d_err, 0, sizeof(int), e.stream);
-        cudaMemsetAsync(e.d_skcnt, 0, sizeof(int) * 2 * ctx->num_sms, e.stream);
+        clear_ctl(e);
         if (!started.empty()) {
             rc = eng_upload(ctx, e, jobs);
+            for (int k = 0; k < np; ++k) {
+                all[k]->bn = jobs[k].bn;
+                all[k]->bn2 = jobs[k].bn2;
+                all[k]->ref_bn = jobs[k].ref_bn;
+            }
             if (rc == FE_OK) rc = eng_setup(ctx, e, jobs, k0, np);
         }
         int herr = 0;
@@ -1548,6 +1657,25 @@ extern "C" int fe_create(fe_ctx **out, const fe_config *cfg) {
             rc = set_err(nullptr, FE_ECUDA, "cooperative launch of k_lanczos_run unavailable");
         else
             ctx->lz_grid = std::min(kLzBlocks, per_sm * ctx->num_sms);
+    }
+    if (rc == FE_OK) {
+        // k_sym_mma: one CTA per SM in clusters of two, all resident at once
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2 * (ctx->num_sms / 2));
+        cfg.blockDim = dim3(kSymThreads);
+        cfg.dynamicSmemBytes = mma_smem_bytes();
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int nc = 0;
+        if (cudaOccupancyMaxActiveClusters(&nc, k_sym_mma, &cfg) != cudaSuccess || nc < 1)
+            rc = set_err(nullptr, FE_ECUDA, std::string("clusters of k_sym_mma unavailable: ") +
+                                                cudaGetErrorString(cudaGetLastError()));
+        else
+            ctx->sym_grid = 2 * std::min(nc, ctx->num_sms / 2);
     }
     if (rc == FE_OK) {
         // the register hand-off inside the split-FP16 kernel assumes this allocation
@@ -1818,24 +1946,25 @@ extern "C" int fe_k_sym_square(fe_ctx *ctx, const float *Y, int64_t n, int64_t l
     op.out[0].s = 1.0f;
     // tile width from the context's table for this n (split: FE_PREC_FP32, single: FE_PREC_TRY_FP16)
     const int bn = tile_width(ctx, n, nslices == 2 ? FE_PREC_FP32 : FE_PREC_TRY_FP16);
-    const std::vector<TileEnt> &tl = (bn == kTileM) ? s->tilesN : s->tiles;
+    fe_problem sz{};
+    sz.n = n;
+    std::vector<Job> one(1);
+    one[0].p = &sz;
+    one[0].ref_bn = bn;
+    choose_widths(ctx, one);
+    const std::vector<TileEnt> &tl = tiles_tc(s, one[0].bn, one[0].bn2, ctx->sym_grid / 2);
     rc = ensure_dev(ctx, &eg.d_probs, &eg.probs_cap, 1);
     if (rc == FE_OK) rc = ensure_dev(ctx, &eg.d_tiles, &eg.tiles_cap, tl.size());
     if (rc != FE_OK) { release_slot(ctx, s); return rc; }
     MmaProb hp = s->hp;
     hp.tc_tile0 = 0;
-    hp.tc_ntiles = static_cast<int>(tl.size());
-    hp.ntiles = static_cast<int>(tl.size());
-    hp.bn = bn;
+    set_tiles(&hp, tl, bn);
     cudaMemcpyAsync(eg.d_probs, &hp, sizeof(MmaProb), cudaMemcpyHostToDevice, q);
     cudaMemcpyAsync(eg.d_tiles, tl.data(), sizeof(TileEnt) * tl.size(), cudaMemcpyHostToDevice, q);
-    cudaMemsetAsync(eg.d_skcnt, 0, sizeof(int) * 2 * ctx->num_sms, q);
     cudaMemcpyAsync(s->st, &st0, sizeof(SolveState), cudaMemcpyHostToDevice, q);
     cudaMemsetAsync(eg.d_err, 0, sizeof(int), q);
-    const int nt = static_cast<int>(tl.size());
-    k_sym_mma<<<ctx->num_sms, kSymThreads, mma_smem_bytes(), q>>>(eg.d_probs, 1, eg.d_tiles, nt, eg.d_err,
-                                                                   eg.d_skws, eg.d_skcnt);
-    ctx->launches += 2;
+    launch_sym(ctx, eg, eg.d_probs, 1, 1);
+    ctx->launches += 1;
     cudaMemcpy2DAsync(C, sizeof(float) * ldc, s->Y, sizeof(float) * s->ldy, sizeof(float) * n, n,
                       cudaMemcpyDeviceToDevice, q);
     int herr = 0;
@@ -1879,7 +2008,7 @@ extern "C" int fe_k_digit_square(fe_ctx *ctx, const double *X, int64_t n, int64_
     cudaMemcpyAsync(s->st, &st0, sizeof(SolveState), cudaMemcpyHostToDevice, q);
     cudaMemsetAsync(eg.d_err, 0, sizeof(int), q);
     const int nt = static_cast<int>(s->tilesD.size());
-    k_digit_prep<<<2 * ctx->num_sms, 256, 0, q>>>(eg.d_probs, 1);
+    k_digit_prep<<<2 * ctx->num_sms, 256, 0, q>>>(eg.d_probs, 1, eg.d_err);
     k_digit_mma<<<std::min(nt, ctx->num_sms), kMmaThreads, digit_smem_bytes(), q>>>(eg.d_probs, eg.d_tilesD,
                                                                                     nt, eg.d_err);
     ctx->launches += 2;

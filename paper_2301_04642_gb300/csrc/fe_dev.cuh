@@ -24,9 +24,6 @@ constexpr int kTileN = 256;    // columns of one tensor-core tile (two 128-block
 constexpr int kTileK = 64;     // K per pipeline stage (one 128-byte swizzle row of FP16)
 constexpr int kMaxSlices = 2;
 constexpr int kStages = 2;
-constexpr int kSliceABytes = kTileM * kTileK * 2;   // 16 KiB
-constexpr int kSliceBBytes = kTileN * kTileK * 2;   // 32 KiB
-constexpr int kStageBytes = kMaxSlices * (kSliceABytes + kSliceBBytes);  // 96 KiB
 constexpr int kMmaThreads = 320;  // digit kernel: warp 0 TMA, warp 1 MMA, warps 2-9 drain + epilogue
 constexpr int kEpiWarps = 8;
 // split-FP16 kernel: warpgroup 0 (warp 0 TMA, warp 1 MMA, warps 2-3 idle) gives
@@ -62,8 +59,7 @@ enum DevErr : int {
     kErrTimeoutEmpty = 2,   // smem stage never released
     kErrTimeoutTmem = 3,    // accumulator hand-off never happened
     kErrBadInput = 4,
-    kErrTimeoutPartner = 5, // the partial sums of a split tile never arrived
-    kErrTimeoutGrid = 6,    // a grid barrier of a cooperative launch never completed
+    kErrTimeoutGrid = 6,    // a meeting of all CTAs of a cooperative launch never completed
 };
 
 // bounded waits give up after this many nanoseconds of wall time unless the
@@ -72,21 +68,19 @@ constexpr uint64_t kWaitTimeoutNs = 2000000000ull;
 
 // Device control block of one engine, passed to the kernels that wait: the
 // first error code of the run (the host clears it before each run), the
-// limit of every bounded wait, the arrival counter of the grid barriers of
-// the cooperative Lanczos launch (zeroed before it), and a test hook.  With
-// fail_partner set, the
-// wait of the second CTA of a split tile in k_sym_mma watches `never` (a word
-// nothing writes) instead of its partner's flag, so the wait runs out, the
-// kernel records kErrTimeoutPartner and returns; it exists to test that
+// limit of every bounded wait, the arrival counters of the meetings of all CTAs
+// in the cooperative launches, and a test hook.  With fail_partner set, those
+// meetings in k_sym_mma watch `never` (a word nothing writes), so the wait runs
+// out, the kernel records kErrTimeoutGrid and returns; it exists to test that
 // expiry path.
 struct DevCtl {
     int err;
     int fail_partner;
     int never;
-    int pad;
+    int hold;  // step graph: the other families' kernels of this pass leave at once (see StepFlags)
     unsigned long long wait_ns;
     unsigned lz_bar;
-    unsigned pad2;
+    unsigned sym_bar;  // meetings of the CTAs of a multi-step k_sym_mma launch (zeroed before each run)
 };
 
 constexpr int kHistRows = 160;  // per-step history kept in the solve state
@@ -146,7 +140,7 @@ struct ProdOp {
     int nout;      // 1..3 outputs
     int part_out;  // output whose trace and squared Frobenius norm go to the partials
     float ra, rb, rc;  // aux partial: sum over (ra v + rb E1 + rc [i == j])^2
-    int pad;
+    int ref_sums;      // 1: trace and norm by the reference tiles (MmaProb::rsum, ref_tile_sums)
     OutSpec out[3];
 };
 
@@ -162,13 +156,11 @@ struct SolveState {
     // finite temperature: beta = 1/kT, tracked chemical potential, stages
     double beta, mu_t, beta0;
     int ft_m, ft_stage, ft_sub, ft_j, ft_nj, ft_shifts, wcur, ft_phase;
-    int ft_last_mat, ft_pad2;  // slot whose ||.||_F the last step's partials report
     double ns_r;      // Newton-Schulz: bound on the residual ||I - M W|| of the current W
     double ns_mmin, ns_mmax;  // bounds on the spectrum of the current M
     int ns_single;    // 1: the current Newton-Schulz pair runs single-FP16 products
     int ft_pad3;
     double sc[6];     // identity parts: A = sc I + A~ (W's in sc[kMatW0], shared by both W slots)
-    double fb[6];     // bounds on ||A~||_F (slice scales are derived from them)
     float scl[6];     // slice scale s of each slot's FP16 slices (slices hold s A~)
     double ft_t, w0;  // tanh of the current shift; Newton-Schulz start
     double mu_prev;   // mu(T) of the previous tracked stage (the drift prediction)
@@ -302,12 +294,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for the phase with the given parity; false after limit_ns.
+// Wait for the phase with the given parity; false after limit_ns, counted on
+// the SM clock (at most 2.07 per ns): the global timer is slow to read, and a
+// poll loop that reads it wakes late.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
     if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer();
+    const long long t0 = clock64(), lim = static_cast<long long>(2 * limit_ns);
     while (!mbar_try_wait(bar, parity)) {
-        if (globaltimer() - t0 > limit_ns) return false;
+        if (clock64() - t0 > lim) return false;
     }
     return true;
 }
@@ -367,21 +361,118 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
         : "memory");
 }
 
+// ---- thread-block pairs (cta_group::2): two CTAs of a cluster share one MMA ----
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// every thread of both CTAs arrives and waits
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// cluster address of this CTA's shared-memory object as it lies in CTA `rank`
+__device__ __forceinline__ uint32_t mapa_u32(const void *p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+
+// arrive on a barrier of either CTA.  The barriers of a pair hand over tensor
+// memory and TMA stages, whose order the tcgen05 fences and the async proxy keep;
+// no generic writes pass between the CTAs, so the arrival needs no
+// cluster-wide release (a fence per chunk).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+
+// TMA load into this CTA's shared memory that signals the barrier at a cluster
+// address (the pair's leader).
+__device__ __forceinline__ void tma_load_2d_pair(void *smem_dst, const CUtensorMap *map, uint32_t bar_cluster,
+                                                 int x, int y) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster)
+        : "memory");
+}
+
+// Both CTAs of the pair allocate and free together (one warp each).
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t *smem_slot, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_slot)),
+                 "r"(ncols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+}
+
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
+}
+
+// D (+)= A B^T over the pair (M = 256: 128 rows of each CTA, N split between
+// the CTAs' shared memories); the leader's thread issues it for both.
+__device__ __forceinline__ void tc_mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrive on `bar` of both CTAs once every MMA issued so far has completed.
+__device__ __forceinline__ void tc_commit_pair(uint64_t *bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"(static_cast<uint16_t>(3))
+        : "memory");
+}
+
+// orders generic-proxy accesses to global memory with TMA reads of it
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
+// 16 consecutive FP32 columns of this warp's 32 TMEM lanes.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// ---- meeting point of all blocks of a cooperative launch ----
+__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // 32 consecutive FP32 columns of this warp's 32 TMEM lanes.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
     uint32_t r[32];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
           "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
           "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
           "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        : "r"(taddr)
+        : "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }

@@ -13,8 +13,10 @@ namespace fe {
 // (MmaProb::dg) and A~ zero on the diagonal, its master holding only the
 // upper triangle (the epilogue reads E terms at (i, j), j >= i).
 struct MatSlot {
-    CUtensorMap tmA[kMaxSlices];  // box 64 (K) x 128 rows
-    CUtensorMap tmB[kMaxSlices];  // box 64 (K) x 256 rows
+    CUtensorMap tm128[kMaxSlices];  // boxes 64 (K) x 128, 64, 32 and 16 rows
+    CUtensorMap tm64[kMaxSlices];
+    CUtensorMap tm32[kMaxSlices];
+    CUtensorMap tm16[kMaxSlices];
     __half *sl[kMaxSlices];
     float *master;                // FP32 small part (null when not kept)
     long long pad;
@@ -35,9 +37,10 @@ struct MmaProb {
     MatSlot mats[kNumMats];
     SolveState *st;
     double *part;                    // per-tile partial slots (kPartStride doubles each)
-    int n, ldy, lds, ntiles;         // ntiles: tensor-core tiles of the problem's tile width
-    int ntilesF, bn;                 // bn: tensor-core tile width, 128 or 256 columns
+    int n, ldy, lds, ntiles;         // ntiles: partial slots of a tensor-core step (2 per tile)
+    int ntilesF, pad1;
     int tc_tile0, tc_ntiles;         // this problem's range in the launch's tensor-core tile list
+    int ref_bn, ref_ntiles;          // reference tiles (see run_cut in k_mma.cu)
     float *lzv;                      // Lanczos vectors: v_prev, v, w (n FP32 each)
     float *Y;                        // FP32 master of the zero-temperature iterate
     double *Xd[2];                   // FP64 buffers (FP64 phase / finite-T output), ld ldx
@@ -51,18 +54,23 @@ struct MmaProb {
     int ntilesD, padD;
     double *dg[kNumMats];            // finite T: FP64 diagonals of the matrix slots (n each)
     float *dgf[kNumMats];            // their FP32 copies (the epilogue's E coefficients)
+    // finite T: squared sums of 8 columns of a row, [column / 8][row], ld rows ldr
+    float *rsum;
+    int ldr, padr;
 };
 
-// One tensor-core tile: rows [I*128, I*128+128) x columns [Jp*bn, Jp*bn+bn)
-// for the problem's tile width bn (256: 2Jp + 1 >= I; 128: Jp >= I).
+// One tensor-core tile: rows [I*256, I*256+256) x columns [Jp*bn, Jp*bn+bn) for
+// its width bn (256, 128, 64 or 32), Jp >= 256 I / bn; its two CTAs use the
+// partial slots 2 slot and 2 slot + 1.
 struct TileEnt {
     int prob;
     int I;
     int Jp;
     int slot;  // partial slot index within the problem
+    int bn;    // tensor-core tiles: width
 };
 
-// A digit-product tile uses TileEnt with Jp = J: rows [I*128, +128) x
+// A digit-product tile is a TileEnt with Jp = J: rows [I*128, +128) x
 // columns [J*64, +64), J >= 2I.
 
 // One FP64 tile: rows [I*16, +16) x columns [J*16, +16), J >= I.
@@ -73,13 +81,30 @@ struct TileF64 {
     int slot;
 };
 
-// Split-FP16 symmetric products, Stream-K scheduled over the tiles of all
-// active problems.  ws: kSkSlotFloats floats per participating CTA (partial
-// sums of a split tile); cnt: 2 ints per CTA, zero between launches.
-__global__ void k_sym_mma(const MmaProb *__restrict__ probs, int nprobs,
-                          const TileEnt *__restrict__ tiles, int ntiles, DevCtl *ctl, float *ws, int *cnt);
-constexpr size_t kSkSlotFloats = static_cast<size_t>(kTileM) * kTileN;  // 128 KiB per slot
+// Step bookkeeping of the graph-driven step loop (see k_control).  With
+// max_steps > 1, k_sym_mma runs the control steps between its products itself;
+// `controlled` tells the k_control behind it that every tensor-core step issued
+// is still to run.  The problems stay in step: when the control step leaves some
+// with tensor-core work and some with another family's, k_sym_mma sets
+// DevCtl::hold, that family's kernels and k_control pass, and all of them run in
+// the next pass.
+struct StepFlags;
+// Symmetric products over the tiles of all active problems, one step or (a
+// cooperative launch) up to max_steps of them; grid: pairs of CTAs.  ws:
+// kRunSlotFloats floats per CTA; gsched: sched_row_bytes() bytes per problem
+// and CTA when the table holds more than kSchedTabProbs problems; ref_ctas: the
+// CTA count that the reference schedule is cut for.
+__global__ void k_sym_mma(const MmaProb *__restrict__ probs, int nprobs, const TileEnt *__restrict__ tiles,
+                          DevCtl *ctl, float *ws, char *gsched, StepFlags *flags, int ref_ctas, int max_steps);
+// Reference-tile sums of the problems whose last step asked for them (plain
+// launches; inside a multi-step launch k_sym_mma does this itself).
+__global__ void k_ref_sums(const MmaProb *__restrict__ probs, int nprobs);
+constexpr size_t kRunSlotFloats = static_cast<size_t>(kEpiWarps) * 32 * 128;  // 128 KiB
+constexpr int kSchedTabProbs = 256;
+// 128-row panels per band of the reference tile lists (256- and 128-wide)
+constexpr int kRefBand = 16, kRefBandN = 12;
 size_t mma_smem_bytes();
+size_t sched_row_bytes();
 
 struct RowInfo {
     double lo, hi, diag, maxabs;  // H_ii - r_i, H_ii + r_i, H_ii, max_j |H_ij|
@@ -157,22 +182,20 @@ __device__ __forceinline__ void setup_from_bounds(const MmaProb &pr, SolveState 
 // Zero temperature: X0 -> (c, Y0) and slices.  Finite temperature: z0.  Per-block partials.
 __global__ void k_init_x0(const MmaProb *probs, int prob);
 // Step control for every problem (one block per problem).
-// Step bookkeeping of the graph-driven step loop (see k_control).
-enum StepBits : unsigned { kStepActive = 1u, kStepTc = 2u, kStepFp64 = 4u, kStepDigit = 8u };
 struct StepFlags {
-    unsigned mask, count;                  // per step: OR of the problems' needs; blocks done
-    unsigned n_body, n_tc, n_fp64, n_digit;  // steps run; steps that launched each family
+    unsigned mask, count;      // per pass: OR of the problems' needs; blocks done
+    unsigned n_steps, n_ctl;   // control steps taken; k_control launches
+    unsigned n_tc;             // passes after the first with k_sym_mma switched on
+    unsigned controlled;       // k_sym_mma ran the control step of its last product
 };
 // Control step: one block per problem.  With flags (inside the step graph)
-// the last block to finish also sets the graph's loop and kernel switches.
-// Once a kernel of the run has recorded an error in ctl (a bounded wait ran
-// out), every problem ends with FE_ETIMEOUT.
+// the last block to finish also sets the graph's loop condition and the switch
+// of k_sym_mma.  Once a kernel of the run has recorded an error in ctl (a bounded
+// wait ran out), every problem ends with FE_ETIMEOUT.
 __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, StepFlags *flags,
-                          cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_tc,
-                          cudaGraphConditionalHandle h_fp64, cudaGraphConditionalHandle h_digit,
-                          unsigned hvalid);
+                          cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_tc, int has_tc);
 // FP64-accurate product + SP2 update (upper tiles, mirrored), per-tile partials.
-__global__ void k_fp64_step(const MmaProb *probs, const TileF64 *tiles, int ntiles);
+__global__ void k_fp64_step(const MmaProb *probs, const TileF64 *tiles, int ntiles, const DevCtl *ctl);
 // D = X -> out (FP64, ld), partials of tr(H D) and tr D.
 __global__ void k_finalize(const MmaProb *probs, int prob, double *D, long long ldd);
 __global__ void k_finalize_reduce(const MmaProb *probs, int prob);
@@ -182,7 +205,7 @@ __global__ void k_digit_mma(const MmaProb *__restrict__ probs, const TileEnt *__
                             int ntiles, DevCtl *ctl);
 size_t digit_smem_bytes();
 // Digits of the current iterate for every problem whose next step is kDigit.
-__global__ void k_digit_prep(const MmaProb *probs, int nprobs);
+__global__ void k_digit_prep(const MmaProb *probs, int nprobs, const DevCtl *ctl);
 
 // FP32 -> FP16 slices of s*Y for a standalone product (kernel tests).
 __global__ void k_make_slices(const float *Y, int n, int ldy, float s, __half *hi, __half *lo,

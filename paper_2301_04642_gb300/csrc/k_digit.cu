@@ -136,7 +136,8 @@ __device__ __forceinline__ void put_digits2(const MmaProb &pr, size_t at, long l
     }
 }
 
-__global__ void k_digit_prep(const MmaProb *probs, int nprobs) {
+__global__ void k_digit_prep(const MmaProb *probs, int nprobs, const DevCtl *ctl) {
+    if (ctl->hold) return;
     for (int p = 0; p < nprobs; ++p) {
         const MmaProb &pr = probs[p];
         const SolveState *st = pr.st;
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint64_t wait_ns = ctl->wait_ns;
+    if (ctl->hold) return;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kDigitStages; ++s) {

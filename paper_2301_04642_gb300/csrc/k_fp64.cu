@@ -23,12 +23,14 @@ constexpr int kBK = 32;        // K per shared-memory stage
 constexpr int kLd = kBK + 2;   // row stride: 16-byte reads of 8 rows hit all banks
 }  // namespace
 
-__global__ void __launch_bounds__(256) k_fp64_step(const MmaProb *probs, const TileF64 *tiles, int ntiles) {
+__global__ void __launch_bounds__(256) k_fp64_step(const MmaProb *probs, const TileF64 *tiles, int ntiles,
+                                                   const DevCtl *ctl) {
     __shared__ __align__(16) double sA[2][kTileF64][kLd];
     __shared__ __align__(16) double sB[2][kTileF64][kLd];
     __shared__ double sT[kTileF64][kTileF64 + 1];
     __shared__ double red[3][8];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    if (ctl->hold) return;
 
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const TileF64 te = tiles[t];

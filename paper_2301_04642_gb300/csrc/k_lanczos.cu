@@ -123,12 +123,6 @@ __device__ double tri_last_comp(const double *a, const double *b, int k, double 
 
 namespace {
 
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // Grid barrier number k of a cooperative launch: complete once all nb blocks
 // arrived, i.e. the arrival counter (zeroed before the launch) reaches
 // (k + 1) nb.  The wait is bounded: when it runs out the block records

@@ -13,12 +13,24 @@
 // lower triangle, and leaves per-tile FP64 partials (trace and squared
 // Frobenius norm of one output, trace of another, and an auxiliary sum of
 // squares used as the idempotency measure ||X^2 - X||_F^2).  The step to run
-// is described by the ProdOp the control kernel wrote into the solve state.
+// is described by the ProdOp the control step wrote into the solve state.
 //
-// One persistent CTA per SM walks a list of tiles (of one or many problems).
-// A problem's tile width bn is 256 (128 rows of block I x the blocks 2Jp,
-// 2Jp+1) or 128 (block I x block J = Jp, J >= I), as the host's tile-shape
-// table chose for its n; one launch may mix both.
+// Tiles and what bounds them.  A tile is 256 rows x bn columns (bn = 256, 128,
+// 64 or 32), computed by a cluster of two CTAs (cta_group::2, M = 256): each
+// CTA keeps 128 rows of A and bn/2 rows of B in its shared memory and the
+// accumulators of its 128 rows in its tensor memory.  A split-FP16 chunk of
+// K = 64 is twelve MMAs, 1536 clocks at bn = 256; a CTA of its own would have
+// to take in 96 KiB for them (128 rows of A, 256 of B, two slices each), which
+// an SM's 64 bytes a clock just cover and a loaded L2 does not; a pair takes in
+// 64 KiB per CTA, and the third stage that then fits hides the load latency.
+// A chunk takes 0.98 us at n = 8192 (0.65 in the single-FP16 form), against 1.21
+// us for a CTA of its own; 0.80 (0.50) of it remains with every load and drain taken
+// out, the hand-over of two tensor-memory buffers between the CTAs.  Launches at
+// n = 16384: 11.6 -> 8.8 ms split, 8.4 -> 6.4 ms single.
+// The narrow tiles are for problems with few tiles: a step's time is then one
+// tile's K loop plus its store phase, both shorter the narrower it is
+// (n = 384: 53 us a launch with tiles of 128 x 256, 27 with 256 x 32; n = 517,
+// finite temperature: 133 and 40).  The host picks bn (choose_widths in fe_api.cu).
 //
 // Accuracy: the tensor core adds every MMA into its FP32 accumulator with a
 // one-sided rounding, so an accumulator that lives for the whole K loop
@@ -27,77 +39,593 @@
 // issued first and the four hi*hi MMAs last, so the truncating additions at
 // full magnitude are four per chunk.  The drain warps read each chunk from
 // TMEM and sum the chunks in registers (round-to-nearest FP32) while the MMA
-// warp fills the other chunk buffer.
+// thread fills the other chunk buffer.  A tile's chunks are summed in at most
+// two runs, each in K order, whose cut run_cut() computes from the launch's
+// work alone: an element's rounding depends neither on bn nor on which CTA
+// computes it.
+//
+// Steps per launch.  With max_steps > 1 (a cooperative launch) the kernel runs
+// the control step of every problem between two products, with a meeting of
+// all CTAs before and after it, until a problem needs another kernel family,
+// none is left, or max_steps products ran (see StepFlags).  As a pass of a graph
+// loop (switch, product, control) a step cost about 25 us besides its product; the
+// two meetings take 1.6 us each and the control step 4 to 9: n = 384 went from
+// 77 us a step to 31, n = 517 at finite temperature from 146 to 35.
 //
 // Warp roles (384 threads; warpgroup 0 hands registers to warpgroups 1-2):
-//   warp 0      TMA producer: per K chunk one box per slice for the A panel
-//               (128 rows) and the B panel (bn rows).
-//   warp 1      TMEM owner and MMA issuer: per chunk 4 x (1 or 3) MMAs
-//               M128 Nbn K16 into one of two chunk buffers (2 x 256 cols).
+//   warp 0      TMA producer: per K chunk one box per slice for this CTA's
+//               rows of A (128) and of B (bn/2), signalling the leader's barrier.
+//   warp 1      TMEM owner; in the leader CTA the MMA issuer: per chunk
+//               4 x (1 or 3) MMAs M256 Nbn K16 into one of two chunk buffers
+//               (2 x 256 columns).
 //   warps 2-3   idle (give their registers away)
 //   warps 4-11  drain + epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31
-//               and the columns bn/2 ((w - 4) / 4) .. +bn/2-1 (one 128x128
-//               block, or half of one when bn = 128) in 64-column loads.
+//               and the columns bn/2 ((w - 4) / 4) .. +bn/2-1; between steps
+//               the control step and the next schedule table.
 // Every wait is bounded; on a timeout the kernel records an error code,
 // drains its own copies and MMAs, frees TMEM and returns.
-#include "fe_dev.cuh"
-#include "fe_kernels.cuh"
+#include "k_control.cuh"
 
 namespace fe {
 
 namespace {
 
+constexpr int kSymStages = 3;
+constexpr int kSymHalfBytes = kTileM * kTileK * 2;  // 16 KiB: 128 rows of one slice
+
 struct alignas(1024) StageSmem {
-    uint8_t a[kMaxSlices][kSliceABytes];
-    uint8_t b[kMaxSlices][kSliceBBytes];
+    uint8_t a[kMaxSlices][kSymHalfBytes];
+    uint8_t b[kMaxSlices][kSymHalfBytes];
 };
 
-// The launch's schedule table, in shared memory when the launch has 2 to
-// kSchedProbs problems: per problem (table order) the inclusive prefix sums
-// of active tiles and of work units, and the units of one of its tiles (0:
-// no tensor-core work in this step).  Built once per launch; without it every
-// tile hand-out would walk the problem table in global memory, a chain of
-// dependent loads per problem.
+// The step's schedule (built before every step by the drain warps).  Problems
+// appear in two orders: by position in the launch's table (the reference
+// tiling that run_cut() works on) and by descending dimension (the order
+// in which tiles are handed out, so that the last ones are the small ones).
+struct SchedHead {
+    long long units;  // reference work units of the step
+    int tiles;        // tiles of the step (pairs of CTAs)
+    int rtiles;       // reference tiles
+    int bnmin, wmin, wmax;
+    int cont;         // 1: run this step, 0: leave
+};
+struct SchedRow {
+    long long units;   // reference units of problems 0..q (inclusive)
+    int rtiles;        // reference tiles of problems 0..q (inclusive)
+    int w;             // reference units per tile of problem q (0: no work)
+    int tiles;         // s-th largest problem and those before it: tiles (inclusive)
+    int prob;          // the s-th largest problem
+};
 constexpr int kSchedProbs = 256;
-struct SchedTab {
-    long long units[kSchedProbs];
-    int tiles[kSchedProbs];
-    int w[kSchedProbs];
-    int bnmin, wmin, wmax, pad;
-};
 
-// The fields of one output that the store loop's vector path reads.
+// One output of a step as the store phase reads it (shared memory, one copy
+// per drain warp: read from the op descriptor in global memory the fields would
+// be re-loaded after every store, which could alias them).
 struct OutCache {
     float a, b1, b2, s, g1r, g1c, g2r, g2c;
     int flags, pad;
     float *master;
     __half *sl0, *sl1;
+    double c, q, l1, l2;        // diagonal entry: c + a v_ii + q dx_i dy_i + l1 dx_i + l2 dy_i
+    const double *dx, *dy;      // diagonal form: d vectors (null: 0)
+    double *dgm;                // ... of the target, and their FP32 copy
+    float *dgfm;
+    double *X;                  // FP64 outputs: target, and addend (null: none)
+    const double *Xa;
 };
+struct OpCache {
+    float inv, ra, rb, rc;
+    int nout, pout;
+    const float *E1, *E2, *F1, *F2;  // E masters; FP32 diagonals that scale them (diagonal form)
+    float *rsum;                     // reference-tile sums: squared sums of 8 columns (null: tile partials)
+    long long ldr;
+    OutCache out[3];
+};
+
+__device__ __forceinline__ void load_op(OpCache &oc, const MmaProb &pr, const ProdOp &op, int lane) {
+    if (lane < 3) {
+        const OutSpec &o = op.out[lane];
+        OutCache &c = oc.out[lane];
+        if (lane < op.nout) {
+            const int fl = o.flags, mat = o.mat, dx = o.dx, dy = o.dy;
+            c.a = o.a;
+            c.b1 = o.b1;
+            c.b2 = o.b2;
+            c.s = o.s;
+            c.g1r = o.g1r;
+            c.g1c = o.g1c;
+            c.g2r = o.g2r;
+            c.g2c = o.g2c;
+            c.flags = fl;
+            c.master = pr.mats[mat].master;
+            c.sl0 = pr.mats[mat].sl[0];
+            c.sl1 = pr.mats[mat].sl[1];
+            c.c = o.c;
+            c.q = o.q;
+            c.l1 = o.l1;
+            c.l2 = o.l2;
+            const bool dform = (fl & kOutDiag) != 0;
+            c.dx = (dform && dx >= 0) ? pr.dg[dx] : nullptr;
+            c.dy = (dform && dy >= 0) ? pr.dg[dy] : nullptr;
+            c.dgm = dform ? pr.dg[mat] : nullptr;
+            c.dgfm = dform ? pr.dgf[mat] : nullptr;
+            c.X = pr.Xd[(fl & kOutF64b) ? 1 : 0];
+            c.Xa = (fl & kOutF64Add) ? pr.Xd[(fl & kOutF64b) ? 0 : 1] : nullptr;
+        }
+    } else if (lane == 3) {
+        oc.inv = op.inv;
+        oc.ra = op.ra;
+        oc.rb = op.rb;
+        oc.rc = op.rc;
+        oc.nout = op.nout;
+        oc.pout = op.part_out;
+        oc.E1 = (op.E1 >= 0) ? pr.mats[op.E1].master : nullptr;
+        oc.E2 = (op.E2 >= 0) ? pr.mats[op.E2].master : nullptr;
+        // the outputs of one step share their E1 / E2 coefficient vectors (the
+        // control step sets them so)
+        const float *f1 = nullptr, *f2 = nullptr;
+        for (int o = 0; o < op.nout; ++o) {
+            if (!(op.out[o].flags & kOutDiag)) continue;
+            if (op.out[o].v1 >= 0) f1 = pr.dgf[op.out[o].v1];
+            if (op.out[o].v2 >= 0) f2 = pr.dgf[op.out[o].v2];
+        }
+        oc.F1 = f1;
+        oc.F2 = f2;
+        oc.rsum = op.ref_sums ? pr.rsum : nullptr;
+        oc.ldr = pr.ldr;
+    }
+}
+
+// FP64 partials of a tile, one thread's share.
+struct TilePart {
+    double tr = 0.0, sq = 0.0, tr1 = 0.0, rr = 0.0;
+};
+
+// Eight consecutive columns of one row: a lane's share of a 16-column group.
+struct Eight {
+    float x[8];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = 0.0f;
+    }
+    __device__ __forceinline__ void load(const float *p) {  // 16-byte aligned
+        const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+        x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    }
+};
+
+// ---- Store phase of one warp's strip: rows i0 .. i0 + 31, columns cb .. cb +
+// ncol - 1, from the register sums (lane = row, acc[c] = column cb + c).
+//
+// Groups of 16 columns go through a small per-warp buffer (column-major, stride
+// 34: no bank conflicts either way) that turns lane = row into two lanes per
+// row, eight columns each.  From there everything is in registers: E1/E2 come
+// in as one full 32-byte sector per lane, E1 two half groups (of 16 rows) ahead,
+// the FP16 slices are formed once for both places they go to, a row's 16
+// columns leave as full sectors (lane pairs swap halves of the FP32 master), and
+// the mirrored copies as 64-byte (master) and 32-byte (slices) runs over 16
+// rows.  The loop over the groups is not unrolled: only the copy out of acc is,
+// eight times 16 stores.  A 128 x 256 tile's phase takes 36 us at n = 4096 and 39 at
+// n = 16384 (finite temperature, one output), all SMs storing at once at 2.6 TB/s
+// over the chip; a 128 x 32 tile on the diagonal (three outputs), whose entries had
+// loaded their operands one by one, went from 33 to 10 us.
+//
+// A group off the matrix edge and above the diagonal takes vector accesses;
+// the others guarded 4-byte and 2-byte ones.
+constexpr int kBufLd = 34;
+
+__device__ __forceinline__ void group_to_buf(const float (&acc)[128], int g, float inv, float *buf, int lane) {
+#define FE_GROUP(G)                                                                              \
+    case G: {                                                                                    \
+        _Pragma("unroll") for (int c = 0; c < 16; ++c) buf[c * kBufLd + lane] = acc[16 * G + c] * inv; \
+    } break;
+    switch (g) {
+        FE_GROUP(0)
+        FE_GROUP(1)
+        FE_GROUP(2)
+        FE_GROUP(3)
+        FE_GROUP(4)
+        FE_GROUP(5)
+        FE_GROUP(6)
+        FE_GROUP(7)
+    }
+#undef FE_GROUP
+}
+
+// packed FP16 pairs (columns 2p, 2p + 1) of s x: hi and lo slices
+__device__ __forceinline__ void split_eight(const float *x, float s, uint32_t *hi, uint32_t *lo) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const float y0 = x[2 * p] * s, y1 = x[2 * p + 1] * s;
+        const __half2 h = __floats2half2_rn(y0, y1);
+        const float2 back = __half22float2(h);
+        const __half2 l = __floats2half2_rn(y0 - back.x, y1 - back.y);
+        hi[p] = *reinterpret_cast<const uint32_t *>(&h);
+        lo[p] = *reinterpret_cast<const uint32_t *>(&l);
+    }
+}
+
+// Mirrored slices of a lane's eight columns: lanes on neighbouring rows trade
+// halves, so that each stores pairs (rows i, i + 1) of four columns.
+__device__ __forceinline__ void put_mirror(__half *sl, const uint32_t *w, size_t at, int lds, bool odd) {
+    __half *p0 = sl + at + (odd ? lds - 1 : 0);
+    const size_t step = 2 * static_cast<size_t>(lds);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        // even row: column 2p of both rows; odd row: column 2p + 1
+        const uint32_t nb = __shfl_xor_sync(0xffffffffu, w[p], 2);
+        *reinterpret_cast<uint32_t *>(p0 + p * step) =
+            odd ? __byte_perm(nb, w[p], 0x7632) : __byte_perm(w[p], nb, 0x5410);
+    }
+}
+
+// Coefficient of an E term, q + g f.  Sums of a whole group of eight columns
+// contract it, element-wise ones (the edge, the diagonal, FP64 outputs) round
+// the product: the two forms every release has used in these places.
+__device__ __forceinline__ float e_coef(float g, float f, float q, bool whole) {
+    return whole ? fmaf(g, f, q) : __fadd_rn(q, __fmul_rn(g, f));
+}
+
+template <bool kLean>
+struct Strip {
+    const OpCache &oc;
+    const int n, ldy, lds, ldx, i0, cb, lane, half, r2;
+    const float *const buf;
+    TilePart &pt;
+
+    // One half group on the vector path: rows i0 + r2 + 16 T, eight columns of this
+    // lane from jb on.
+    template <int T>
+    __device__ __forceinline__ void vec(int jg, const Eight &e1, const float *E2, const float *F1, const float *F2,
+                                        float d1, float d2) {
+        const int jb = jg + 8 * half, i = i0 + r2 + 16 * T;
+        const bool odd = (r2 & 1) != 0;
+        Eight e2;
+        e2.zero();
+        if (!kLean && E2) e2.load(E2 + static_cast<size_t>(i) * ldy + jb);
+        Eight f1, f2;
+        if (!kLean) {
+            f1.zero();
+            f2.zero();
+            if (F1) f1.load(F1 + jb);  // jb % 8 == 0, 64-byte aligned vectors
+            if (F2) f2.load(F2 + jb);
+        }
+        float v[8];
+        float crr = 0.0f;
+        const float ra = oc.ra, rb = oc.rb;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = buf[(8 * half + u) * kBufLd + r2 + 16 * T];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float r = fmaf(ra, v[u], rb * e1.x[u]);
+            crr = fmaf(r, r, crr);
+        }
+        pt.rr = fma(2.0, f32_to_f64(crr), pt.rr);
+        const size_t so = static_cast<size_t>(i) * lds + jb;
+        const size_t ms = static_cast<size_t>(jb) * lds + i;
+        const size_t mo = static_cast<size_t>(jb) * ldy + i;
+        const int nout = kLean ? 1 : oc.nout, pout = kLean ? 0 : oc.pout;
+#pragma unroll 1
+        for (int o = 0; o < nout; ++o) {
+            const OutCache &os = oc.out[o];
+            const int fl = kLean ? (kOutMaster | kOutSlices) : os.flags;
+            const bool dform = !kLean && (fl & kOutDiag);
+            float val[8];
+            float csq = 0.0f;
+            const float oa = os.a, ob = os.b1;
+            if (kLean) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) val[u] = fmaf(oa, v[u], ob * e1.x[u]);
+            } else if (dform) {
+                // per-row / per-column coefficients of E1 and E2
+                const float q1 = fmaf(os.g1r, d1, ob), q2 = fmaf(os.g2r, d2, os.b2), g1 = os.g1c, g2 = os.g2c;
+                const bool whole = !(fl & (kOutF64a | kOutF64b));
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    val[u] = fmaf(oa, v[u], fmaf(e_coef(g1, f1.x[u], q1, whole), e1.x[u],
+                                                 e_coef(g2, f2.x[u], q2, whole) * e2.x[u]));
+            } else {
+                const float b2 = os.b2;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) val[u] = fmaf(oa, v[u], fmaf(ob, e1.x[u], b2 * e2.x[u]));
+            }
+            if (!kLean && (fl & (kOutF64a | kOutF64b))) {
+                f64_out<true>(os, o == pout, o == 1, val, v, i, jb);
+                continue;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) csq = fmaf(val[u], val[u], csq);
+            if (!kLean && oc.rsum) oc.rsum[(jb >> 3) * oc.ldr + i] = 2.0f * csq;
+            else if (o == pout) pt.sq = fma(2.0, f32_to_f64(csq), pt.sq);
+            if (fl & kOutSlices) {
+                uint32_t hi[4], lo[4];
+                split_eight(val, os.s, hi, lo);
+                *reinterpret_cast<uint4 *>(os.sl0 + so) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4 *>(os.sl1 + so) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                put_mirror(os.sl0, hi, ms, lds, odd);
+                put_mirror(os.sl1, lo, ms, lds, odd);
+            }
+            if (fl & kOutMaster) {
+                if (!dform) {  // diagonal form: upper master only
+                    float *m = os.master + mo;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u, m += ldy) *m = val[u];
+                }
+                // the even lane keeps columns 0..3 of its eight and takes the odd
+                // lane's 0..3, so that a lane pair fills a 32-byte sector per store
+                float x[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[k] = __shfl_xor_sync(0xffffffffu, half ? val[k] : val[4 + k], 1);
+                float *m = os.master + static_cast<size_t>(i) * ldy + jg + 4 * half;
+                *reinterpret_cast<float4 *>(m) =
+                    half ? make_float4(x[0], x[1], x[2], x[3]) : make_float4(val[0], val[1], val[2], val[3]);
+                *reinterpret_cast<float4 *>(m + 8) =
+                    half ? make_float4(val[4], val[5], val[6], val[7]) : make_float4(x[0], x[1], x[2], x[3]);
+            }
+        }
+    }
+
+    // FP64 output of eight columns.  FP32 terms are summed in FP32 and converted
+    // exactly by integer operations: GB300's FP64 pipe (1/64 of the FP32 rate) keeps
+    // only the FP64 diagonal, the FP64 addend and the squared norm.
+    template <bool kVec>
+    __device__ __forceinline__ void f64_out(const OutCache &os, bool part, bool part1, const float *val, const float *v,
+                                            int i, int jb) {
+        const size_t xo = static_cast<size_t>(i) * ldx + jb;
+        auto ok = [&](int u) { return kVec || (i < n && jb + u < n && jb + u >= i); };
+        double d[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) d[u] = (os.Xa && ok(u)) ? os.Xa[xo + u] : 0.0;
+        const int ud = kVec ? -1 : i - jb;  // this lane's diagonal entry, if 0 <= ud < 8 and i < n
+        double dv = 0.0;
+        if (!kVec && ud >= 0 && ud < 8 && i < n) {
+            float vd = 0.0f, wd = 0.0f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (u == ud) {
+                    vd = v[u];
+                    wd = val[u];
+                }
+            dv = (os.flags & kOutDiag) ? diag_entry(os, vd, i) : f32_to_f64(wd) + os.c;
+        }
+        double *X = os.X;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (!ok(u)) continue;
+            const bool dg = !kVec && u == ud;
+            const double x = dg ? dv : f32_to_f64(val[u]);
+            d[u] = os.Xa ? x + d[u] : x;
+            X[xo + u] = d[u];
+            if (!dg) X[static_cast<size_t>(jb + u) * ldx + i] = d[u];
+            if (part) {
+                if (dg) pt.tr += d[u];
+                pt.sq = fma(dg ? d[u] : 2.0 * d[u], d[u], pt.sq);
+            }
+            if (part1 && dg) pt.tr1 += d[u];
+        }
+    }
+
+    // diagonal entry of an output in the diagonal form, FP64
+    __device__ __forceinline__ double diag_entry(const OutCache &os, float vd, int i) {
+        const double dx = os.dx ? os.dx[i] : 0.0, dy = os.dy ? os.dy[i] : 0.0;
+        const double r = os.c + static_cast<double>(os.a) * static_cast<double>(vd);
+        return r + os.q * dx * dy + os.l1 * dx + os.l2 * dy;
+    }
+
+    // A half group with entries on or below the diagonal or beyond the edge.
+    __device__ __forceinline__ void slow(int jg, int t, const float *E1, const float *E2, const float *F1,
+                                         const float *F2, float d1, float d2) {
+        const int jb = jg + 8 * half, i = i0 + r2 + 16 * t;
+        unsigned okm = 0;  // entries of this lane that exist and lie on or above the diagonal
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i < n && jb + u < n && jb + u >= i) okm |= 1u << u;
+        const int ud = i - jb;
+        const bool has_diag = ud >= 0 && ud < 8 && (okm >> ud & 1u);
+        // a whole group of eight above the diagonal counts twice; elsewhere each
+        // element is weighted by itself
+        const bool full8 = i0 + 32 <= n && jb + 8 <= n && jb >= i0 + 32;
+        const size_t ro = static_cast<size_t>(i) * ldy + jb;
+        Eight e1, e2, f1, f2;
+        e1.zero();
+        e2.zero();
+        f1.zero();
+        f2.zero();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool k = okm >> u & 1u;
+            if (E1 && k) e1.x[u] = E1[ro + u];
+            if (!kLean && E2 && k) e2.x[u] = E2[ro + u];
+            if (!kLean && F1 && k) f1.x[u] = F1[jb + u];
+            if (!kLean && F2 && k) f2.x[u] = F2[jb + u];
+        }
+        float v[8], vd = 0.0f;
+        float crr = 0.0f;
+        const float ra = oc.ra, rb = oc.rb, rc = oc.rc;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            v[u] = buf[(8 * half + u) * kBufLd + r2 + 16 * t];
+            const bool dg = u == ud;
+            if (dg) vd = v[u];
+            const float r = fmaf(ra, v[u], rb * e1.x[u]) + (dg ? rc : 0.0f);
+            if (okm >> u & 1u) crr = fmaf(dg || full8 ? r : 2.0f * r, r, crr);
+        }
+        pt.rr = fma(full8 ? 2.0 : 1.0, f32_to_f64(crr), pt.rr);
+        const int nout = kLean ? 1 : oc.nout, pout = kLean ? 0 : oc.pout;
+#pragma unroll 1
+        for (int o = 0; o < nout; ++o) {
+            const OutCache &os = oc.out[o];
+            const int fl = kLean ? (kOutMaster | kOutSlices) : os.flags;
+            const bool dform = !kLean && (fl & kOutDiag);
+            float val[8];
+            const float q1 = dform ? fmaf(os.g1r, d1, os.b1) : os.b1, q2 = dform ? fmaf(os.g2r, d2, os.b2) : os.b2;
+            const float g1 = dform ? os.g1c : 0.0f, g2 = dform ? os.g2c : 0.0f;
+            const bool whole = full8 && !(fl & (kOutF64a | kOutF64b));
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (kLean) val[u] = fmaf(os.a, v[u], os.b1 * e1.x[u]);
+                else val[u] = fmaf(os.a, v[u], fmaf(e_coef(g1, f1.x[u], q1, whole), e1.x[u],
+                                                    e_coef(g2, f2.x[u], q2, whole) * e2.x[u]));
+            }
+            if (!kLean && (fl & (kOutF64a | kOutF64b))) {
+                f64_out<false>(os, o == pout, o == 1, val, v, i, jb);
+                continue;
+            }
+            if (has_diag) {
+                float nd;  // the stored small part's diagonal entry
+                if (dform) {
+                    // the diagonal goes to the FP64 vector; the small part keeps 0
+                    const double dv = diag_entry(os, vd, i);
+                    os.dgm[i] = dv;
+                    os.dgfm[i] = static_cast<float>(dv);
+                    if (o == pout) {
+                        pt.tr += dv;
+                        pt.sq += dv * dv;
+                    }
+                    if (o == 1) pt.tr1 += dv;
+                    nd = 0.0f;
+                } else {
+                    nd = 0.0f;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (u == ud) nd = val[u] + static_cast<float>(os.c);
+                    if (o == pout) pt.tr += static_cast<double>(nd);
+                    if (o == 1) pt.tr1 += static_cast<double>(nd);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (u == ud) val[u] = nd;
+            }
+            float csq = 0.0f;
+            const float sc = os.s;
+            uint32_t hi[4], lo[4];
+            split_eight(val, sc, hi, lo);
+            float *md = os.master + ro, *mm = os.master + static_cast<size_t>(jb) * ldy + i;
+            __half *s0 = os.sl0, *s1 = os.sl1;
+            const size_t so = static_cast<size_t>(i) * lds + jb, ms = static_cast<size_t>(jb) * lds + i;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool k = okm >> u & 1u, dg = u == ud;
+                if (k) csq = fmaf(dg || full8 ? val[u] : 2.0f * val[u], val[u], csq);
+                if (k && (fl & kOutMaster)) {
+                    md[u] = val[u];
+                    if (!dg && !dform) mm[static_cast<size_t>(u) * ldy] = val[u];
+                }
+                if (k && (fl & kOutSlices)) {
+                    const uint16_t h = static_cast<uint16_t>((u & 1) ? hi[u >> 1] >> 16 : hi[u >> 1] & 0xFFFFu);
+                    const uint16_t l = static_cast<uint16_t>((u & 1) ? lo[u >> 1] >> 16 : lo[u >> 1] & 0xFFFFu);
+                    reinterpret_cast<uint16_t *>(s0)[so + u] = h;
+                    reinterpret_cast<uint16_t *>(s1)[so + u] = l;
+                    if (!dg) {
+                        reinterpret_cast<uint16_t *>(s0)[ms + static_cast<size_t>(u) * lds] = h;
+                        reinterpret_cast<uint16_t *>(s1)[ms + static_cast<size_t>(u) * lds] = l;
+                    }
+                }
+            }
+            if (!kLean && oc.rsum) {
+                if (i < n) oc.rsum[(jb >> 3) * oc.ldr + i] = full8 ? 2.0f * csq : csq;
+            } else if (o == pout) {
+                pt.sq = fma(full8 ? 2.0 : 1.0, f32_to_f64(csq), pt.sq);
+            }
+        }
+    }
+
+    __device__ __forceinline__ void run(const float (&acc)[128], float *wbuf, int ncol) {
+        const float inv = oc.inv;
+        const float *const E1 = oc.E1, *const E2 = kLean ? nullptr : oc.E2;
+        const float *const F1 = kLean ? nullptr : oc.F1, *const F2 = kLean ? nullptr : oc.F2;
+        // the rows' entries of the coefficient vectors, rows r2 and r2 + 16
+        const int ia = i0 + r2, ib = ia + 16;
+        float d1a = 0.0f, d1b = 0.0f, d2a = 0.0f, d2b = 0.0f;
+        if (!kLean) {
+            if (F1 && ia < n) d1a = F1[ia];
+            if (F1 && ib < n) d1b = F1[ib];
+            if (F2 && ia < n) d2a = F2[ia];
+            if (F2 && ib < n) d2b = F2[ib];
+        }
+        const int ng = ncol >> 4;
+        auto full16 = [&](int g) {
+            const int jg = cb + 16 * g;
+            return g < ng && i0 + 32 <= n && jg + 16 <= n && jg >= i0 + 32;
+        };
+        Eight pa, pb;  // E1 of rows r2 and r2 + 16, one group ahead
+        pa.zero();
+        pb.zero();
+        const float *ea = E1 ? E1 + static_cast<size_t>(ia) * ldy + cb + 8 * half : nullptr;
+        const size_t rows16 = 16 * static_cast<size_t>(ldy);
+        if (E1 && full16(0)) {
+            pa.load(ea);
+            pb.load(ea + rows16);
+        }
+#pragma unroll 1
+        for (int g = 0; g < ng; ++g) {
+            const int jg = cb + 16 * g;
+            if (jg >= n) break;
+            const bool next = E1 && full16(g + 1);
+            const float *en = ea + 16 * (g + 1);
+            if (jg + 15 < i0) {  // wholly below the diagonal
+                if (next) {
+                    pa.load(en);
+                    pb.load(en + rows16);
+                }
+                continue;
+            }
+            group_to_buf(acc, g, inv, wbuf, lane);
+            __syncwarp();
+            if (full16(g)) {
+                Eight e = pa;
+                if (next) pa.load(en);
+                vec<0>(jg, e, E2, F1, F2, d1a, d2a);
+                e = pb;
+                if (next) pb.load(en + rows16);
+                vec<1>(jg, e, E2, F1, F2, d1b, d2b);
+            } else {
+                slow(jg, 0, E1, E2, F1, F2, d1a, d2a);
+                slow(jg, 1, E1, E2, F1, F2, d1b, d2b);
+                if (next) {
+                    pa.load(en);
+                    pb.load(en + rows16);
+                }
+            }
+            __syncwarp();  // the buffer is free for the next group
+        }
+    }
+};
+
+template <bool kLean>
+__device__ __forceinline__ void store_strip(const float (&acc)[128], const OpCache &oc, const MmaProb &pr, float *buf,
+                                            int i0, int cb, int ncol, int lane, TilePart &pt) {
+    Strip<kLean> st{oc, pr.n, pr.ldy, pr.lds, pr.ldx, i0, cb, lane, lane & 1, lane >> 1, buf, pt};
+    st.run(acc, buf, ncol);
+}
 
 struct MmaSmemTail {
-    uint64_t full[kStages];
-    uint64_t empty[kStages];
-    uint64_t cfull[2];
-    uint64_t cempty[2];
+    uint64_t full[kSymStages];   // leader: both CTAs' operand bytes have landed
+    uint64_t empty[kSymStages];  // both: the stage's MMAs are done
+    uint64_t cfull[2];           // both: a chunk is in TMEM
+    uint64_t cempty[2];          // leader: all drain warps of the pair have read it
     uint32_t tmem_base;
-    int abort_flag;
+    int step_ok;
     double red[kEpiWarps][4];
     int vote[kEpiWarps];
-    int sk_ticket, sk_ok;             // split-tile hand-off (drain warp 0 writes, all read)
-    double stage[kEpiWarps][32 * 9];  // per-warp staging of 32 rows x 8 columns (direct writes)
-    OutCache oc[kEpiWarps][3];        // per-warp copy of the step's outputs (shared-memory loads
-                                      // in the store loop instead of reloads after every store)
-    SchedTab sch;
+    union {
+        float buf[kEpiWarps][16 * kBufLd];  // per-warp transposition buffer of the store phase
+        ControlSmem ctl;                    // between steps
+    };
+    OpCache oc[kEpiWarps];
+    SchedHead head;
+    SchedRow row[kSchedProbs];
 };
 
-constexpr size_t kMmaSmemBytes = 1024 + sizeof(StageSmem) * kStages + sizeof(MmaSmemTail);
+constexpr size_t kMmaSmemBytes = 1024 + sizeof(StageSmem) * kSymStages + sizeof(MmaSmemTail);
+static_assert(kMmaSmemBytes <= 227 * 1024, "shared memory of one CTA");
 
 __device__ __forceinline__ int step_kind(const SolveState *st) {
     return *reinterpret_cast<const volatile int *>(&st->kind);
 }
 
-__device__ __forceinline__ bool tile_active(const SolveState *st) {
-    const int kind = step_kind(st);
+__device__ __forceinline__ bool tc_kind(int kind) {
     return kind == kTcSingle || kind == kTcSplit || kind == kTcElem || kind == kTcDelta;
 }
 
@@ -112,329 +640,326 @@ __device__ __forceinline__ int step_chunks(const SolveState *st, int n) {
     return step_kind(st) == kTcElem ? 0 : (n + kTileK - 1) / kTileK;
 }
 
-// tile width of a problem: 128 or 256 columns
-__device__ __forceinline__ int tile_bn(const MmaProb &pr) { return pr.bn == kTileM ? kTileM : kTileN; }
-
 __device__ __forceinline__ void record_error(DevCtl *ctl, int code) { atomicCAS(&ctl->err, 0, code); }
 
-// named barrier of the 8 drain/epilogue warps
+// named barriers: the 8 drain/epilogue warps; all 12 warps of the CTA
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void step_bar() { asm volatile("bar.sync 2, 384;" ::: "memory"); }
 
-// hi/lo FP16 slices of s * v[0..7], packed for one 16-byte store each
-// (the same roundings as put_slices)
-__device__ __forceinline__ void split8(const float *v, float s, uint4 &hv, uint4 &lv) {
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const float y0 = v[2 * p] * s, y1 = v[2 * p + 1] * s;
-        const __half2 hh = __floats2half2_rn(y0, y1);
-        const float2 back = __half22float2(hh);
-        const __half2 ll = __floats2half2_rn(y0 - back.x, y1 - back.y);
-        h[p] = *reinterpret_cast<const uint32_t *>(&hh);
-        l[p] = *reinterpret_cast<const uint32_t *>(&ll);
+// ---- Where a tile's chunk sum is cut.  The reference schedule, on which the
+// rounding of a step is defined, runs over the reference tiles of the active
+// problems in table order (128 rows x ref_bn columns, ref_bn = 256 or 128), each
+// worth `units` = its chunks (1 for an epilogue-only step) times its width over
+// the narrowest one.  When every tile is worth the same and there are at least
+// two waves of `ref_ctas` tiles, whole waves are left whole; the remaining one
+// to two waves (all tiles otherwise) are cut into G <= ref_ctas equal contiguous
+// ranges of units, G at most the number of largest tiles, so a tile holds at
+// most one range end.  A chunk belongs to the range that holds its first unit.
+
+// Position of reference tile (I, J) in its problem's list: bands of
+// kRefBand (kRefBandN for 128-wide tiles) row panels, column by column.
+__device__ __forceinline__ int ref_index(int n, int ref_bn, int I, int J) {
+    const int T = (n + kTileM - 1) / kTileM;
+    if (ref_bn == kTileM) {
+        const int b0 = I / kRefBandN * kRefBandN, R = min(kRefBandN, T - b0);
+        const int base = b0 * T - b0 * (b0 - 1) / 2;  // tiles of the bands before
+        const int d = J - b0, m = min(d, R);            // columns before J; those not yet full
+        return base + m * (m + 1) / 2 + (d - m) * R + (I - b0);
     }
-    hv = make_uint4(h[0], h[1], h[2], h[3]);
-    lv = make_uint4(l[0], l[1], l[2], l[3]);
+    const int TP = (T + 1) / 2;
+    const int b0 = I / kRefBand * kRefBand, R = min(kRefBand, T - b0);
+    const int base = b0 * TP - (b0 > 0 ? (b0 - 1) * (b0 - 1) / 4 : 0);
+    const int d = J - b0 / 2, m = min(d, R / 2);
+    return base + m * (m + 1) + (d - m) * R + (I - b0);
 }
 
-__device__ __forceinline__ void put_slices(const MatSlot &m, size_t at, float ys) {
-    const __half hh = __float2half_rn(ys);
-    m.sl[0][at] = hh;
-    m.sl[1][at] = __float2half_rn(ys - __half2float(hh));
+// First chunk of the second run of block (I, column block J128) of problem q
+// (0: one run).  nk: the step's chunks.
+__device__ int run_cut(const SchedHead &sh, const SchedRow *row, const MmaProb &pr, int q, int ref_ctas, int nk, int I,
+                       int J128) {
+    if (nk < 2) return 0;
+    const long long r = ref_index(pr.n, pr.ref_bn, I, pr.ref_bn == kTileM ? J128 : J128 / 2);
+    long long whole = 0;  // tiles in whole waves
+    if (sh.wmin == sh.wmax && sh.rtiles >= 2 * ref_ctas)
+        whole = (sh.rtiles % ref_ctas == 0) ? sh.rtiles : static_cast<long long>(sh.rtiles / ref_ctas - 1) * ref_ctas;
+    if ((q ? row[q - 1].rtiles : 0) + r < whole) return 0;
+    const int w = row[q].w, f = pr.ref_bn / sh.bnmin;
+    const long long u0 = whole * sh.wmax;
+    const long long W = sh.units - u0;
+    long long G = W / sh.wmax;
+    G = G > ref_ctas ? ref_ctas : G;
+    if (G < 2) return 0;
+    const long long x = (q ? row[q - 1].units : 0) + r * w - u0;  // the tile's first unit
+    // the first range end beyond x; ends lie at floor(W b / G)
+    long long b = x * G / W + 1;
+    while (b < G && W * b / G <= x) ++b;
+    if (b >= G) return 0;
+    const long long ku = W * b / G - x;
+    if (ku >= w) return 0;
+    const int k = static_cast<int>((ku + f - 1) / f);
+    return k < nk ? k : 0;
 }
 
-// ---- Schedule: data-parallel waves, then Stream-K.  The launch's work is the
-// sequence, over the active problems in table order, of their tiles, each
-// worth `units` = its 64-wide K chunks (1 for an epilogue-only step) times its
-// width over the narrowest width in the launch (so a 128 x 256 tile weighs
-// twice a 128 x 128 one when both are present).
-// When every tile is worth the same and there are at least two waves, whole
-// waves go first, tile t to CTA t mod grid: all CTAs then step through K
-// together on tiles that are neighbours in the list (the host orders tiles in
-// bands so that these share row and column panels), and each panel chunk is
-// read from HBM about once per wave while the rest hit L2.  The remaining one
-// to two waves of tiles (all of them otherwise) are cut into equal contiguous
-// ranges, one per participating CTA (Stream-K), so tile boundaries (and store
-// phases) fall at different times in different CTAs and the last wave is not
-// left half empty.  At most G = W / (largest tile) CTAs take part, so a tile
-// spans at most two ranges: a head segment at the end of one CTA's range and
-// a tail segment at the start of the next one's.  A chunk worth f units
-// belongs to the range that holds its first unit; a range part that holds no
-// chunk's first unit is skipped.  Every role of a CTA walks the same segments.
-struct Seg {
-    int tile;   // index into the launch's tile list
-    int prob;   // index of its problem in the launch's table
-    int k0;     // first chunk
-    int nch;    // chunks (0 for an epilogue-only step)
-    bool split; // the tile is shared with a neighbouring CTA
-    bool head;  // this CTA has its first chunks (else its last)
-};
-
-// chunks of a tile, counting an epilogue-only step's tile as one
-__device__ __forceinline__ int tile_chunks(const MmaProb &pr) {
-    const int nk = step_chunks(pr.st, pr.n);
-    return nk > 0 ? nk : 1;
-}
-
-// Fill the schedule table (every thread of the CTA calls this between two
-// CTA barriers, `warp0` says whether it is in warp 0).  Pass 1, all threads:
-// chunks, width and tiles of each problem.  Pass 2, warp 0 after a barrier:
-// the narrowest width, the units per tile, and prefix sums (each lane scans
-// a contiguous run of problems, then the run totals are scanned across the
-// warp).
-__device__ void sched_pass1(SchedTab *t, const MmaProb *probs, int np) {
-    for (int q = threadIdx.x; q < np; q += blockDim.x) {
-        const MmaProb &pr = probs[q];
-        const bool act = pr.tc_ntiles > 0 && tile_active(pr.st);
-        t->w[q] = act ? tile_chunks(pr) : 0;
-        t->tiles[q] = act ? pr.tc_ntiles : 0;
-        t->units[q] = act ? tile_bn(pr) : 0;
+// The sums that a finite-temperature step hands to the control of mu (tr z and
+// ||z||_F^2; D follows mu continuously, and a last bit of a sum can flip FP32
+// roundings all over the next stages) are defined on the reference tiles, so that
+// they depend neither on bn nor on which CTA stored what: per row of a tile's
+// 32 x (ref_bn / 2) strips, FP64 sums over the 8-column FP32 sums the store phase
+// left in rsum, in column order, with the diagonal's square before its group; a
+// tree over the strip's rows; the strips in order.  256 threads, one tile per call.
+template <class Bar>
+__device__ void ref_tile_sums(const MmaProb &pr, int tile, double (*red)[4], int t, Bar bar) {
+    const int n = pr.n, T = (n + kTileM - 1) / kTileM;
+    const int w = t >> 5, lane = t & 31, q = w & 3, h = w >> 2;
+    const bool wide = pr.ref_bn == kTileN;
+    const int TP = wide ? (T + 1) / 2 : T;
+    // row-major tile number -> (I, J), J >= I / 2 (or I)
+    auto row0 = [&](int I) {
+        return wide ? I * TP - (I > 0 ? (I - 1) * (I - 1) / 4 : 0) : I * TP - I * (I - 1) / 2;
+    };
+    int lo = 0, hi = T - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (row0(mid) <= tile) lo = mid;
+        else hi = mid - 1;
     }
-}
-
-__device__ void sched_pass2(SchedTab *t, int np, int lane) {
-    int bm = kTileN;
-    for (int q = lane; q < np; q += 32)
-        if (t->w[q] > 0) bm = static_cast<int>(t->units[q]) < bm ? static_cast<int>(t->units[q]) : bm;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int y = __shfl_xor_sync(0xffffffffu, bm, o);
-        bm = y < bm ? y : bm;
-    }
-    const int per = (np + 31) / 32;
-    const int q0 = lane * per, q1 = (q0 + per < np) ? q0 + per : np;
-    long long su = 0;
-    int st = 0, wmin = 0x7fffffff, wmax = 1;
-    for (int q = q0; q < q1; ++q) {
-        const int c = t->w[q];
-        const int w = c > 0 ? c * (static_cast<int>(t->units[q]) / bm) : 0;
-        if (c > 0) {
-            wmin = w < wmin ? w : wmin;
-            wmax = w > wmax ? w : wmax;
-        }
-        su += static_cast<long long>(t->tiles[q]) * w;
-        st += t->tiles[q];
-        t->w[q] = w;
-        t->units[q] = su;
-        t->tiles[q] = st;
-    }
-    long long eu = su;
-    int et = st;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long yu = __shfl_up_sync(0xffffffffu, eu, o);
-        const int yt = __shfl_up_sync(0xffffffffu, et, o);
-        if (lane >= o) {
-            eu += yu;
-            et += yt;
+    const int I = lo, J = tile - row0(I) + (wide ? I / 2 : I);
+    const int i0 = I * kTileM + q * 32, i = i0 + lane;
+    const int ncol = pr.ref_bn >> 1, cb = J * pr.ref_bn + h * ncol;
+    double tr = 0.0, sq = 0.0;
+    if (cb / kTileM >= I && i0 < n) {
+        const SolveState *st = pr.st;
+        const double *dg = pr.dg[st->op.out[0].mat];
+        for (int g = 0; g < ncol / 8; ++g) {
+            const int j0 = cb + 8 * g;
+            if (j0 >= n) break;
+            if (j0 + 7 < i0) continue;
+            if (i >= j0 && i < j0 + 8 && i < n) {
+                const double dv = __ldcg(dg + i);
+                tr += dv;
+                sq += dv * dv;
+            }
+            if (i < n) sq += static_cast<double>(__ldcg(pr.rsum + static_cast<size_t>(j0 >> 3) * pr.ldr + i));
         }
     }
-    eu -= su;
-    et -= st;
-    for (int q = q0; q < q1; ++q) {
-        t->units[q] += eu;
-        t->tiles[q] += et;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int a = __shfl_xor_sync(0xffffffffu, wmin, o);
-        const int b = __shfl_xor_sync(0xffffffffu, wmax, o);
-        wmin = a < wmin ? a : wmin;
-        wmax = b > wmax ? b : wmax;
-    }
+    tr = warp_sum(tr);
+    sq = warp_sum(sq);
     if (lane == 0) {
-        t->bnmin = bm;
-        t->wmin = wmin;
-        t->wmax = wmax;
+        red[w][0] = tr;
+        red[w][1] = sq;
     }
+    bar();
+    if (t < 2) {
+        double a = 0.0;
+        for (int x = 0; x < kEpiWarps; ++x) a += red[x][t];
+        pr.part[static_cast<size_t>(tile) * kPartStride + t] = a;
+    }
+    bar();
 }
 
-struct SegIter {
-    const MmaProb *probs;
-    const SchedTab *tab;   // the shared-memory table, or null: walk the table in global memory
-    int nprobs;
-    int bnmin;             // narrowest tile width among the active problems
-    long long dp, dp_end;  // data-parallel part: next tile index (over active tiles), end
-    long long g, end;      // Stream-K part: this CTA's range of work units
-
-    __device__ int unit_f(const MmaProb &pr) const { return tile_bn(pr) / bnmin; }
-    __device__ int tile_units(const MmaProb &pr) const { return tile_chunks(pr) * unit_f(pr); }
-
-    // the problem holding active tile r (tiles = true) or work unit r of the
-    // launch, with r made relative to the problem's first; nprobs if none
-    __device__ int find(long long &r, bool tiles) const {
-        if (nprobs <= 0) return nprobs;
-        if (tab) {
-            int lo = 0, hi = nprobs - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                const long long v = tiles ? tab->tiles[mid] : tab->units[mid];
-                if (v > r) hi = mid;
-                else lo = mid + 1;
-            }
-            const long long v = tiles ? tab->tiles[lo] : tab->units[lo];
-            if (v <= r) return nprobs;
-            if (lo > 0) r -= tiles ? tab->tiles[lo - 1] : tab->units[lo - 1];
-            return lo;
-        }
-        for (int q = 0; q < nprobs; ++q) {
-            const MmaProb &pr = probs[q];
-            if (pr.tc_ntiles == 0 || !tile_active(pr.st)) continue;
-            const long long span = tiles ? pr.tc_ntiles : static_cast<long long>(pr.tc_ntiles) * tile_units(pr);
-            if (r < span) return q;
-            r -= span;
-        }
-        return nprobs;
+// The schedule table of the next step, by the 256 drain threads.  Returns
+// bit 0: some problem has tensor-core work, bit 1: some problem waits for
+// another kernel family, bit 2: some step of bit 0 has reference-tile sums.  Problems beyond kSchedProbs have their rows in global
+// memory (one copy per CTA) and keep the table's order.
+__device__ int sched_build(SchedHead *sh, SchedRow *row, const MmaProb *probs, int np, int t, int *mask) {
+    // per problem: w = units per reference tile before the width factor,
+    // rtiles, tiles, and in units the reference width
+    if (t == 0) *mask = 0;
+    epi_bar();
+    int m = 0;
+    for (int q = t; q < np; q += kCtlThreads) {
+        const MmaProb &pr = probs[q];
+        const int kind = step_kind(pr.st);
+        const bool act = pr.tc_ntiles > 0 && tc_kind(kind);
+        if (act) m |= 1;
+        if (act && *reinterpret_cast<const volatile int *>(&pr.st->op.ref_sums)) m |= 4;
+        if (kind == kDigit || kind == kFp64) m |= 2;
+        const int nk = act ? step_chunks(pr.st, pr.n) : 0;
+        row[q].w = act ? (nk > 0 ? nk : 1) : 0;
+        row[q].rtiles = act ? pr.ref_ntiles : 0;
+        row[q].units = act ? pr.ref_bn : 0;
+        row[q].tiles = act ? pr.tc_ntiles : 0;
+        row[q].prob = q;
     }
-
-    __device__ void init(const MmaProb *p, int np, const SchedTab *t) {
-        probs = p;
-        nprobs = np;
-        tab = t;
-        long long W = 0, T = 0;
-        int wmax = 1, wmin = 0x7fffffff;
-        if (t) {
-            bnmin = t->bnmin;
-            if (np > 0) {
-                W = t->units[np - 1];
-                T = t->tiles[np - 1];
+    if (m) atomicOr(mask, m);
+    epi_bar();
+    if (np > 1 && np <= kSchedProbs) {
+        // order by descending dimension (ties: table order)
+        int rank = 0, tl = 0;
+        if (t < np) {
+            const int n = probs[t].n;
+            for (int r = 0; r < np; ++r) {
+                const int nr = probs[r].n;
+                rank += (nr > n || (nr == n && r < t)) ? 1 : 0;
             }
-            wmin = t->wmin;
-            wmax = t->wmax;
-        } else {
-            bnmin = kTileN;
-            for (int q = 0; q < np; ++q) {
-                const MmaProb &pr = p[q];
-                if (pr.tc_ntiles == 0 || !tile_active(pr.st)) continue;
-                bnmin = tile_bn(pr) < bnmin ? tile_bn(pr) : bnmin;
+            tl = row[t].tiles;
+        }
+        epi_bar();
+        if (t < np) {
+            row[rank].tiles = tl;
+            row[rank].prob = t;
+        }
+        epi_bar();
+    }
+    if (t < 32) {
+        int bm = kTileN;
+        for (int q = t; q < np; q += 32)
+            if (row[q].w > 0) bm = min(bm, static_cast<int>(row[q].units));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) bm = min(bm, __shfl_xor_sync(0xffffffffu, bm, o));
+        const int per = (np + 31) / 32;
+        const int q0 = t * per, q1 = min(q0 + per, np);
+        long long su = 0;
+        int sr = 0, sl = 0, wmin = 0x7fffffff, wmax = 1;
+        for (int q = q0; q < q1; ++q) {
+            const int c = row[q].w;
+            const int w = c > 0 ? c * (static_cast<int>(row[q].units) / bm) : 0;
+            if (c > 0) {
+                wmin = min(wmin, w);
+                wmax = max(wmax, w);
             }
-            for (int q = 0; q < np; ++q) {
-                const MmaProb &pr = p[q];
-                if (pr.tc_ntiles == 0 || !tile_active(pr.st)) continue;
-                const int w = tile_units(pr);
-                W += static_cast<long long>(pr.tc_ntiles) * w;
-                T += pr.tc_ntiles;
-                wmax = w > wmax ? w : wmax;
-                wmin = w < wmin ? w : wmin;
+            su += static_cast<long long>(row[q].rtiles) * w;
+            sr += row[q].rtiles;
+            sl += row[q].tiles;
+            row[q].w = w;
+            row[q].units = su;
+            row[q].rtiles = sr;
+            row[q].tiles = sl;
+        }
+        long long eu = su;
+        int er = sr, el = sl;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long yu = __shfl_up_sync(0xffffffffu, eu, o);
+            const int yr = __shfl_up_sync(0xffffffffu, er, o);
+            const int yl = __shfl_up_sync(0xffffffffu, el, o);
+            if (t >= o) {
+                eu += yu;
+                er += yr;
+                el += yl;
             }
         }
-        const long long grid = gridDim.x;
-        const long long b = blockIdx.x;
-        long long D = 0;  // tiles in whole data-parallel waves
-        if (T > 0 && wmin == wmax && T >= 2 * grid) D = (T % grid == 0) ? T : (T / grid - 1) * grid;
-        dp = b;
-        dp_end = D;
-        const long long Wsk = W - D * wmax;
-        long long G = Wsk / wmax;
-        if (G > grid) G = grid;
-        if (G < 1) G = 1;
-        if (Wsk <= 0 || b >= G) {
-            g = end = 0;
-        } else {
-            g = D * wmax + Wsk * b / G;
-            end = D * wmax + Wsk * (b + 1) / G;
+        if (t == 31) {
+            sh->units = eu;
+            sh->rtiles = er;
+            sh->tiles = el;
+        }
+        eu -= su;
+        er -= sr;
+        el -= sl;
+        for (int q = q0; q < q1; ++q) {
+            row[q].units += eu;
+            row[q].rtiles += er;
+            row[q].tiles += el;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            wmin = min(wmin, __shfl_xor_sync(0xffffffffu, wmin, o));
+            wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+        }
+        if (t == 0) {
+            sh->bnmin = bm;
+            sh->wmin = wmin;
+            sh->wmax = wmax;
         }
     }
+    const int due = *mask;
+    epi_bar();
+    return due;
+}
 
-    __device__ bool next(Seg &sg) {
-        if (dp < dp_end) {
-            long long r = dp;
-            dp += gridDim.x;
-            const int q = find(r, true);
-            if (q < nprobs) {
-                const MmaProb &pr = probs[q];
-                sg.tile = pr.tc_tile0 + static_cast<int>(r);
-                sg.prob = q;
-                sg.k0 = 0;
-                sg.nch = (step_chunks(pr.st, pr.n) > 0) ? tile_chunks(pr) : 0;
-                sg.split = false;
-                sg.head = true;
-                return true;
-            }
-            dp = dp_end;
+__device__ __forceinline__ int row_work(const SchedRow *row, int q) { return row[q].w; }
+
+// The tiles of one step that this cluster computes: rounds of one tile per
+// cluster, every other round in reverse, so that over two rounds of a list
+// ordered by size every cluster gets about the same work.
+struct TileIter {
+    const SchedHead *sh;
+    const SchedRow *row;
+    int np, cluster, nclusters, round;
+
+    __device__ TileIter(const SchedHead *h, const SchedRow *r, int n)
+        : sh(h), row(r), np(n), cluster(blockIdx.x >> 1), nclusters(gridDim.x >> 1), round(0) {}
+
+    // problem and index in its tile list
+    __device__ bool next(int &prob, int &idx) {
+        const long long g = static_cast<long long>(round) * nclusters +
+                            ((round & 1) ? nclusters - 1 - cluster : cluster);
+        ++round;
+        if (g >= sh->tiles) return false;  // (only in the last round)
+        int lo = 0, hi = np - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (row[mid].tiles > g) hi = mid;
+            else lo = mid + 1;
         }
-        while (g < end) {
-            long long r = g;
-            const int q = find(r, false);
-            if (q == nprobs) break;
-            const MmaProb &pr = probs[q];
-            const int f = unit_f(pr);
-            const int w = tab ? tab->w[q] : tile_units(pr);
-            const int nkc = w / f;
-            const int ku = static_cast<int>(r % w);   // first unit of this range in the tile
-            const long long left = end - g;
-            const int k1u = (left < w - ku) ? ku + static_cast<int>(left) : w;
-            g += k1u - ku;
-            const int k = (ku + f - 1) / f, k1 = (k1u + f - 1) / f;  // chunks starting in [ku, k1u)
-            if (k == k1) continue;
-            sg.tile = pr.tc_tile0 + static_cast<int>(r / w);
-            sg.prob = q;
-            sg.k0 = k;
-            sg.nch = (step_chunks(pr.st, pr.n) > 0) ? k1 - k : 0;
-            sg.split = (k > 0) || (k1 < nkc);
-            sg.head = (k == 0);
-            return true;
-        }
-        g = end;
-        return false;
+        prob = row[lo].prob;
+        idx = static_cast<int>(g) - (lo ? row[lo - 1].tiles : 0);
+        return true;
     }
 };
 
-__device__ __forceinline__ int ld_acquire(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Wait for a flag that a running CTA sets; false after limit_ns.
-__device__ __forceinline__ bool flag_wait_bounded(const int *f, uint64_t limit_ns) {
-    if (ld_acquire(f)) return true;
-    const uint64_t t0 = globaltimer();
-    while (!ld_acquire(f)) {
-        if (globaltimer() - t0 > limit_ns) return false;
-        __nanosleep(64);
+// All blocks of the launch meet (a cooperative launch: all are resident).
+// The counter grows by the number of blocks per meeting.  CTAs without a tile
+// wait here for the whole step, so the limit is eight of the bounded waits.
+// With fail_partner set the wait watches a word nothing writes.
+__device__ bool grid_meet(unsigned *cnt, unsigned nb, DevCtl *ctl, uint64_t wait_ns) {
+    __threadfence();
+    const unsigned old = atomicAdd(cnt, 1u);
+    const unsigned target = old - old % nb + nb;
+    const unsigned *watch = ctl->fail_partner ? reinterpret_cast<const unsigned *>(&ctl->never) : cnt;
+    const unsigned want = ctl->fail_partner ? 1u : target;
+    bool ok = true;
+    if (static_cast<int>(ld_acquire_u32(watch) - want) < 0) {
+        const uint64_t t0 = globaltimer();
+        while (static_cast<int>(ld_acquire_u32(watch) - want) < 0) {
+            if (globaltimer() - t0 > 8 * wait_ns) {
+                ok = false;
+                break;
+            }
+            __nanosleep(20);
+        }
     }
-    return true;
+    if (!ok) record_error(ctl, kErrTimeoutGrid);
+    __threadfence();
+    return ok;
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kSymThreads, 1)
-    k_sym_mma(const MmaProb *__restrict__ probs, int nprobs, const TileEnt *__restrict__ tiles,
-              int ntiles, DevCtl *ctl, float *ws, int *cnt) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSymThreads, 1)
+    k_sym_mma(const MmaProb *__restrict__ probs, int nprobs, const TileEnt *__restrict__ tiles, DevCtl *ctl,
+              float *ws, char *gsched, StepFlags *flags, int ref_ctas, int max_steps) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base_u32 = smem_u32(smem_raw);
     uint8_t *smem = smem_raw + ((1024u - (base_u32 & 1023u)) & 1023u);
     StageSmem *stages = reinterpret_cast<StageSmem *>(smem);
-    MmaSmemTail *tail = reinterpret_cast<MmaSmemTail *>(smem + sizeof(StageSmem) * kStages);
+    MmaSmemTail *tail = reinterpret_cast<MmaSmemTail *>(smem + sizeof(StageSmem) * kSymStages);
+    SchedRow *row = nprobs <= kSchedProbs
+                        ? tail->row
+                        : reinterpret_cast<SchedRow *>(gsched) + static_cast<size_t>(blockIdx.x) * nprobs;
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
     const uint64_t wait_ns = ctl->wait_ns;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < kSymStages; ++s) {
             mbar_init(&tail->full[s], 1);
             mbar_init(&tail->empty[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&tail->cfull[a], 1);
-            mbar_init(&tail->cempty[a], kEpiWarps);
+            mbar_init(&tail->cempty[a], 2 * kEpiWarps);
         }
-        tail->abort_flag = 0;
         fence_barrier_init();
     }
-    // (one problem: its table entry is read directly)
-    const SchedTab *tab = (nprobs > 1 && nprobs <= kSchedProbs) ? &tail->sch : nullptr;
-    if (tab) sched_pass1(&tail->sch, probs, nprobs);
-    if (warp == 1) tmem_alloc(&tail->tmem_base, 512);
+    if (warp == 1) tmem_alloc_pair(&tail->tmem_base, 512);
     tc_fence_before();
     __syncthreads();
+    cluster_sync();  // the peer's barriers are ready before anything signals them
     tc_fence_after();
-    if (tab) {
-        if (warp == 0) sched_pass2(&tail->sch, nprobs, lane);
-        __syncthreads();
-    }
     const uint32_t tmem_base = tail->tmem_base;
 
     if (warp < kSymEpiWarp0) setmaxnreg_dec<kSymRegsLow>();
@@ -442,706 +967,368 @@ __global__ void __launch_bounds__(kSymThreads, 1)
         // ------------------------------------------------------------ producer
         uint32_t stage = 0, phase = 0;
         bool ok = true;
-        uint32_t last_phase[kStages];
-        bool issued[kStages];
-        for (int s = 0; s < kStages; ++s) { issued[s] = false; last_phase[s] = 0; }
-        SegIter it;
-        it.init(probs, nprobs, tab);
-        Seg sg;
-        while (ok && it.next(sg)) {
-            if (sg.tile >= ntiles) break;
-            const TileEnt te = tiles[sg.tile];
-            const MmaProb &pr = probs[sg.prob];
-            const SolveState *st = pr.st;
-            const int S = step_slices(st);
-            const MatSlot &ma = pr.mats[st->op.A];
-            const MatSlot &mb = pr.mats[st->op.B];
-            const bool wide = tile_bn(pr) == kTileN;
-            const CUtensorMap *tmb = wide ? mb.tmB : mb.tmA;  // B panel: 256 or 128 rows
-            const uint32_t bytes = static_cast<uint32_t>(S * (kSliceABytes + (wide ? kSliceBBytes : kSliceABytes)));
-            for (int kc = sg.k0; kc < sg.k0 + sg.nch; ++kc) {
-                bool got = true;
-                if (lane == 0) got = mbar_wait_bounded(&tail->empty[stage], phase ^ 1u, wait_ns);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (!got) {
-                    if (lane == 0) record_error(ctl, kErrTimeoutEmpty);
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) {
-                    mbar_expect_tx(&tail->full[stage], bytes);
-                    for (int s = 0; s < S; ++s) {
-                        tma_load_2d(stages[stage].a[s], &ma.tmA[s], &tail->full[stage],
-                                    kc * kTileK, te.I * kTileM);
-                        tma_load_2d(stages[stage].b[s], &tmb[s], &tail->full[stage],
-                                    kc * kTileK, te.Jp * (wide ? kTileN : kTileM));
+        uint32_t last_phase[kSymStages];
+        bool issued[kSymStages];
+        for (int s = 0; s < kSymStages; ++s) { issued[s] = false; last_phase[s] = 0; }
+        for (;;) {
+            step_bar();
+            if (!tail->head.cont) break;
+            fence_proxy_async_global();  // slices written by other SMs since the last step
+            TileIter it(&tail->head, row, nprobs);
+            int prob, idx;
+            while (ok && it.next(prob, idx)) {
+                const MmaProb &pr = probs[prob];
+                const TileEnt te = tiles[pr.tc_tile0 + idx];
+                const SolveState *st = pr.st;
+                const int S = step_slices(st);
+                const int bn = te.bn, nk = step_chunks(st, pr.n);
+                const CUtensorMap *tma = pr.mats[st->op.A].tm128;
+                const MatSlot &mb = pr.mats[st->op.B];
+                const CUtensorMap *tmb = bn == 256 ? mb.tm128 : bn == 128 ? mb.tm64 : bn == 64 ? mb.tm32 : mb.tm16;
+                const int ya = (2 * te.I + static_cast<int>(rank)) * kTileM;
+                const int yb = te.Jp * bn + static_cast<int>(rank) * (bn >> 1);
+                // both CTAs' operands: 128 rows of A and bn/2 of B each
+                const uint32_t bytes = static_cast<uint32_t>(2 * S * (kSymHalfBytes + bn * kTileK));
+                for (int kc = 0; kc < nk; ++kc) {
+                    bool got = true;
+                    if (lane == 0) got = mbar_wait_bounded(&tail->empty[stage], phase ^ 1u, wait_ns);
+                    got = __shfl_sync(0xffffffffu, got, 0);
+                    if (!got) {
+                        if (lane == 0) record_error(ctl, kErrTimeoutEmpty);
+                        ok = false;
+                        break;
                     }
+                    if (lane == 0) {
+                        if (rank == 0) mbar_expect_tx(&tail->full[stage], bytes);
+                        const uint32_t bar = mapa_u32(&tail->full[stage], 0);
+                        for (int s = 0; s < S; ++s) {
+                            tma_load_2d_pair(stages[stage].a[s], &tma[s], bar, kc * kTileK, ya);
+                            tma_load_2d_pair(stages[stage].b[s], &tmb[s], bar, kc * kTileK, yb);
+                        }
+                    }
+                    __syncwarp();
+                    issued[stage] = true;
+                    last_phase[stage] = phase;
+                    if (++stage == kSymStages) { stage = 0; phase ^= 1u; }
                 }
-                __syncwarp();
-                issued[stage] = true;
-                last_phase[stage] = phase;
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
+            step_bar();
         }
         if (!ok) {
-            // no TMA write may still be in flight when the CTA exits; the last
-            // phase issued on a stage is its newest, so waiting on it is exact
-            tail->abort_flag = 1;
-            if (lane == 0)
-                for (int s = 0; s < kStages; ++s)
-                    if (issued[s]) (void)mbar_wait_bounded(&tail->full[s], last_phase[s], wait_ns);
+            // no TMA write may still be in flight when the CTA exits: the
+            // leader's barriers count both CTAs' bytes, and the pair leaves
+            // together; the peer gives its loads (microseconds) a millisecond
+            if (lane == 0) {
+                if (rank == 0) {
+                    for (int s = 0; s < kSymStages; ++s)
+                        if (issued[s]) (void)mbar_wait_bounded(&tail->full[s], last_phase[s], wait_ns);
+                } else {
+                    const uint64_t t0 = globaltimer();
+                    while (globaltimer() - t0 < 1000000ull) __nanosleep(1000);
+                }
+            }
             __syncwarp();
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         uint32_t stage = 0, phase = 0;
-        uint32_t chunk = 0;  // chunk counter of this CTA: buffer = chunk & 1
+        uint32_t chunk = 0;  // chunk counter of this pair: buffer = chunk & 1
         bool ok = true;
         bool any_commit = false;
-        constexpr uint32_t idesc_w = idesc_f16(kTileM, kTileN, 0);
-        constexpr uint32_t idesc_n = idesc_f16(kTileM, kTileM, 0);
-        SegIter it;
-        it.init(probs, nprobs, tab);
-        Seg sg;
-        while (ok && it.next(sg)) {
-            if (sg.tile >= ntiles) break;
-            const TileEnt te = tiles[sg.tile];
-            const MmaProb &pr = probs[sg.prob];
-            const SolveState *st = pr.st;
-            const int S = step_slices(st);
-            const uint32_t idesc = (tile_bn(pr) == kTileN) ? idesc_w : idesc_n;
-            for (int kc = sg.k0; kc < sg.k0 + sg.nch; ++kc) {
-                const uint32_t buf = chunk & 1u;
-                const uint32_t cph = (chunk >> 1) & 1u;
-                bool got = true;
-                if (lane == 0) got = mbar_wait_bounded(&tail->cempty[buf], cph ^ 1u, wait_ns);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (got) {
-                    if (lane == 0) got = mbar_wait_bounded(&tail->full[stage], phase, wait_ns);
+        for (;;) {
+            step_bar();
+            if (!tail->head.cont) break;
+            TileIter it(&tail->head, row, nprobs);
+            int prob, idx;
+            while (rank == 0 && ok && it.next(prob, idx)) {
+                const MmaProb &pr = probs[prob];
+                const SolveState *st = pr.st;
+                const int S = step_slices(st), nk = step_chunks(st, pr.n);
+                const uint32_t idesc = idesc_f16(2 * kTileM, 0, 0) | (static_cast<uint32_t>(tiles[pr.tc_tile0 + idx].bn >> 3) << 17);
+                for (int kc = 0; kc < nk; ++kc) {
+                    const uint32_t buf = chunk & 1u;
+                    const uint32_t cph = (chunk >> 1) & 1u;
+                    bool got = true;
+                    if (lane == 0) got = mbar_wait_bounded(&tail->cempty[buf], cph ^ 1u, wait_ns);
                     got = __shfl_sync(0xffffffffu, got, 0);
-                    if (!got && lane == 0) record_error(ctl, kErrTimeoutFull);
-                } else if (lane == 0) {
-                    record_error(ctl, kErrTimeoutTmem);
-                }
-                if (!got) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t tmem_d = tmem_base + buf * kTileN;
-                    const uint64_t a0 = smem_desc_sw128(stages[stage].a[0]);
-                    const uint64_t b0 = smem_desc_sw128(stages[stage].b[0]);
-                    uint32_t accum = 0;
-                    if (S == 2) {
-                        const uint64_t a1 = smem_desc_sw128(stages[stage].a[1]);
-                        const uint64_t b1 = smem_desc_sw128(stages[stage].b[1]);
-                        // small cross terms first: hi * lo, lo * hi
+                    if (got) {
+                        if (lane == 0) got = mbar_wait_bounded(&tail->full[stage], phase, wait_ns);
+                        got = __shfl_sync(0xffffffffu, got, 0);
+                        if (!got && lane == 0) record_error(ctl, kErrTimeoutFull);
+                    } else if (lane == 0) {
+                        record_error(ctl, kErrTimeoutTmem);
+                    }
+                    if (!got) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    if (lane == 0) {
+                        const uint32_t tmem_d = tmem_base + buf * kTileN;
+                        const uint64_t a0 = smem_desc_sw128(stages[stage].a[0]);
+                        const uint64_t b0 = smem_desc_sw128(stages[stage].b[0]);
+                        uint32_t accum = 0;
+                        if (S == 2) {
+                            const uint64_t a1 = smem_desc_sw128(stages[stage].a[1]);
+                            const uint64_t b1 = smem_desc_sw128(stages[stage].b[1]);
+                            // small cross terms first: hi * lo, lo * hi
+#pragma unroll
+                            for (int kk = 0; kk < kTileK / 16; ++kk) {
+                                const uint64_t off = static_cast<uint64_t>(kk * 2);  // 32 B along K
+                                tc_mma_f16_pair(tmem_d, a0 + off, b1 + off, idesc, accum);
+                                accum = 1;
+                                tc_mma_f16_pair(tmem_d, a1 + off, b0 + off, idesc, accum);
+                            }
+                        }
+                        // the full-magnitude hi * hi terms last
 #pragma unroll
                         for (int kk = 0; kk < kTileK / 16; ++kk) {
-                            const uint64_t off = static_cast<uint64_t>(kk * 2);  // 32 B along K
-                            tc_mma_f16(tmem_d, a0 + off, b1 + off, idesc, accum);
+                            const uint64_t off = static_cast<uint64_t>(kk * 2);
+                            tc_mma_f16_pair(tmem_d, a0 + off, b0 + off, idesc, accum);
                             accum = 1;
-                            tc_mma_f16(tmem_d, a1 + off, b0 + off, idesc, accum);
                         }
+                        tc_commit_pair(&tail->empty[stage]);  // smem stage may be refilled
+                        tc_commit_pair(&tail->cfull[buf]);    // chunk ready for the drain
+                        any_commit = true;
                     }
-                    // the full-magnitude hi * hi terms last
-#pragma unroll
-                    for (int kk = 0; kk < kTileK / 16; ++kk) {
-                        const uint64_t off = static_cast<uint64_t>(kk * 2);
-                        tc_mma_f16(tmem_d, a0 + off, b0 + off, idesc, accum);
-                        accum = 1;
-                    }
-                    tc_commit(&tail->empty[stage]);  // smem stage may be refilled
-                    tc_commit(&tail->cfull[buf]);    // chunk ready for the drain
-                    any_commit = true;
+                    __syncwarp();
+                    if (++stage == kSymStages) { stage = 0; phase ^= 1u; }
+                    ++chunk;
                 }
-                __syncwarp();
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                ++chunk;
             }
+            step_bar();
         }
         if (!ok) {
-            tail->abort_flag = 1;
             // every issued MMA must finish before TMEM is released
             if (lane == 0 && any_commit) {
                 uint64_t *drain = &tail->cfull[chunk & 1u];
-                tc_commit(drain);
+                tc_commit_pair(drain);
                 (void)mbar_wait_bounded(drain, (chunk >> 1) & 1u, wait_ns);
             }
             __syncwarp();
         }
-    } else if (warp >= kSymEpiWarp0) {
+    } else if (warp < kSymEpiWarp0) {
+        for (;;) {
+            step_bar();
+            if (!tail->head.cont) break;
+            step_bar();
+        }
+    } else {
         // ------------------------------------------------------------ drain + epilogue
         setmaxnreg_inc<kSymRegsHigh>();
         const int ew = warp - kSymEpiWarp0;    // 0..7
+        const int et = threadIdx.x - 32 * kSymEpiWarp0;
         const int q = warp & 3;                // TMEM lane quadrant (hardware rule: warp % 4)
         const int h = ew >> 2;                 // column half of the tile
-        const int row_local = q * 32 + lane;
+        const uint32_t cempty0[2] = {mapa_u32(&tail->cempty[0], 0), mapa_u32(&tail->cempty[1], 0)};
+        float *const wrow = ws + static_cast<size_t>(blockIdx.x) * kRunSlotFloats +
+                            (static_cast<size_t>(ew) * 32 + lane) * 128;  // the first run's sums
         uint32_t chunk = 0;
         bool ok = true;
-        SegIter it;
-        it.init(probs, nprobs, tab);
-        Seg sg;
-        while (ok && it.next(sg)) {
-            if (sg.tile >= ntiles) break;
-            const TileEnt te = tiles[sg.tile];
-            const MmaProb &pr = probs[sg.prob];
-            const SolveState *st = pr.st;
-            const int n = pr.n;
-            const bool wide = tile_bn(pr) == kTileN;
-            const int ncol = wide ? 128 : 64;  // columns of this warp's strip
-            float acc[128];
+        int steps = 0;
+        bool controlled = false;  // the control step of the last product ran here
+        int last_due = 0;
+        for (;;) {
+            // ---- the next step's schedule.  While another family's step is
+            // due the loop pauses: from the start one product is run (its
+            // control step follows that family's kernels), after a control
+            // step the kernel leaves.
+            const int due = sched_build(&tail->head, row, probs, nprobs, et, &tail->step_ok);
+            const bool single = max_steps <= 1 || (due & 2);
+            const bool cont = ok && (due & 1) && steps < max_steps && (steps == 0 || (controlled && !(due & 2)));
+            if (et == 0) tail->head.cont = cont ? 1 : 0;
+            last_due = due;
+            step_bar();
+            if (!cont) break;
+            ++steps;
+            controlled = false;
+            TileIter it(&tail->head, row, nprobs);
+            int prob, idx;
+            while (ok && it.next(prob, idx)) {
+                const MmaProb &pr = probs[prob];
+                const TileEnt te = tiles[pr.tc_tile0 + idx];
+                const SolveState *st = pr.st;
+                const int n = pr.n;
+                const int ncol = te.bn >> 1;  // columns of this warp's strip
+                const int I = 2 * te.I + static_cast<int>(rank);
+                const int cb = te.Jp * te.bn + h * ncol;  // first column of the strip
+                const int nk = step_chunks(st, n);
+                // a strip wholly outside the upper triangle is drained, not kept
+                const bool live = cb / kTileM >= I && cb < n && I * kTileM < n;
+                __syncwarp();
+                load_op(tail->oc[ew], pr, st->op, lane);
+                const int cut = live ? run_cut(tail->head, row, pr, prob, ref_ctas, nk, I, cb / kTileM) : 0;
+                float acc[128];
 #pragma unroll
-            for (int c = 0; c < 128; ++c) acc[c] = 0.0f;
-            for (int kc = sg.k0; kc < sg.k0 + sg.nch; ++kc) {
-                const uint32_t buf = chunk & 1u;
-                const uint32_t cph = (chunk >> 1) & 1u;
-                bool got = mbar_wait_bounded(&tail->cfull[buf], cph, wait_ns);
-                got = __all_sync(0xffffffffu, got);
-                if (!got) {
-                    if (lane == 0) record_error(ctl, kErrTimeoutTmem);
-                    ok = false;
-                    break;
+                for (int c = 0; c < 128; ++c) acc[c] = 0.0f;
+                for (int kc = 0; kc < nk; ++kc) {
+                    const uint32_t buf = chunk & 1u;
+                    const uint32_t cph = (chunk >> 1) & 1u;
+                    bool got = mbar_wait_bounded(&tail->cfull[buf], cph, wait_ns);
+                    got = __all_sync(0xffffffffu, got);
+                    if (!got) {
+                        if (lane == 0) record_error(ctl, kErrTimeoutTmem);
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    if (kc == cut && kc > 0) {
+                        // the second run starts: the first one's sums wait in L2
+#pragma unroll
+                        for (int c = 0; c < 32; ++c)
+                            if (4 * c < ncol) {
+                                __stcg(reinterpret_cast<float4 *>(wrow) + c,
+                                       make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]));
+                                acc[4 * c] = acc[4 * c + 1] = acc[4 * c + 2] = acc[4 * c + 3] = 0.0f;
+                            }
+                    }
+                    const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
+                                           buf * kTileN + static_cast<uint32_t>(h * ncol);
+                    if (!live) {
+                        // nothing to keep
+                    } else if (ncol >= 64) {
+#pragma unroll
+                        for (int c2 = 0; c2 < 2; ++c2) {
+                            if (c2 * 64 < ncol) {
+                                float v[64];
+                                tmem_ld64(tbase + c2 * 64, v);
+#pragma unroll
+                                for (int u = 0; u < 64; ++u) acc[c2 * 64 + u] += v[u];
+                            }
+                        }
+                    } else if (ncol == 32) {
+                        float v[32];
+                        tmem_ld32(tbase, v);
+#pragma unroll
+                        for (int u = 0; u < 32; ++u) acc[u] += v[u];
+                    } else {
+                        float v[16];
+                        tmem_ld16(tbase, v);
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) acc[u] += v[u];
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(cempty0[buf]);
+                    ++chunk;
                 }
-                tc_fence_after();
-                const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                                       buf * kTileN + static_cast<uint32_t>(h * ncol);
+                if (cut > 0) {
 #pragma unroll
-                for (int c2 = 0; c2 < 2; ++c2) {
-                    if (c2 * 64 < ncol) {
-                        float v[64];
-                        tmem_ld64(tbase + c2 * 64, v);
-#pragma unroll
-                        for (int u = 0; u < 64; ++u) acc[c2 * 64 + u] += v[u];
+                    for (int c = 0; c < 32; ++c) {
+                        if (4 * c >= ncol) break;
+                        const float4 p4 = __ldcg(reinterpret_cast<const float4 *>(wrow) + c);
+                        acc[4 * c] += p4.x;
+                        acc[4 * c + 1] += p4.y;
+                        acc[4 * c + 2] += p4.z;
+                        acc[4 * c + 3] += p4.w;
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tail->cempty[buf]);
-                ++chunk;
-            }
-            // a warp leaves the chunk loop early only on a timeout; make the
-            // decision uniform over the drain warps before the named barriers
-            if (lane == 0) tail->vote[ew] = ok ? 1 : 0;
-            epi_bar();
-            bool all_ok = true;
-            for (int w = 0; w < kEpiWarps; ++w) all_ok = all_ok && (tail->vote[w] != 0);
-            epi_bar();
-            if (!all_ok) {
-                ok = false;
-                break;
-            }
 
-            // ---- a tile shared with a neighbouring CTA: the first to arrive
-            // hands its partial sums over through global memory, the second
-            // adds them (one commutative addition: the same result whoever is
-            // second) and runs the epilogue.  The second waits only for a CTA
-            // that is already writing, so the wait is short and bounded.
-            if (sg.split) {
-                const int slot = sg.head ? static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x) - 1;
-                float4 *wsp = reinterpret_cast<float4 *>(ws + static_cast<size_t>(slot) * kSkSlotFloats +
-                                                         (static_cast<size_t>(ew) * 32 + lane) * 128);
-                if (ew == 0 && lane == 0) tail->sk_ticket = atomicAdd(&cnt[2 * slot], 1);
-                epi_bar();
-                const int ticket = tail->sk_ticket;
-                epi_bar();
-                if (ticket == 0) {
-#pragma unroll
-                    for (int c = 0; c < 32; ++c)
-                        if (4 * c < ncol)
-                            wsp[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
-                    __threadfence();
-                    epi_bar();
-                    if (ew == 0 && lane == 0) atomicExch(&cnt[2 * slot + 1], 1);
-                    continue;
+                TilePart pt;
+                const int i0 = I * kTileM + q * 32;
+                if (live && ok && i0 < n) {
+                    const OpCache &oc = tail->oc[ew];
+                    const bool lean = oc.nout == 1 && oc.pout == 0 && !oc.E2 &&
+                                      oc.out[0].flags == (kOutMaster | kOutSlices);
+                    if (lean) store_strip<true>(acc, oc, pr, tail->buf[ew], i0, cb, ncol, lane, pt);
+                    else store_strip<false>(acc, oc, pr, tail->buf[ew], i0, cb, ncol, lane, pt);
                 }
-                if (ew == 0 && lane == 0) {
-                    const int *flag = ctl->fail_partner ? &ctl->never : &cnt[2 * slot + 1];
-                    tail->sk_ok = flag_wait_bounded(flag, wait_ns) ? 1 : 0;
+                // per-tile partials in a fixed order: warp tree, then the 8 warps.  Only
+                // tiles on the diagonal have traces.
+                const bool on_diag = cb < I * kTileM + kTileM;
+                pt.sq = warp_sum(pt.sq);
+                pt.rr = warp_sum(pt.rr);
+                if (on_diag) {
+                    pt.tr = warp_sum(pt.tr);
+                    pt.tr1 = warp_sum(pt.tr1);
+                }
+                if (lane == 0) {
+                    tail->vote[ew] = ok ? 1 : 0;
+                    tail->red[ew][0] = pt.tr;
+                    tail->red[ew][1] = pt.sq;
+                    tail->red[ew][2] = pt.tr1;
+                    tail->red[ew][3] = pt.rr;
                 }
                 epi_bar();
-                const bool got = tail->sk_ok != 0;
+                if (et < 4) {
+                    double a = 0.0;
+                    for (int w = 0; w < kEpiWarps; ++w) a += tail->red[w][et];
+                    pr.part[static_cast<size_t>(2 * te.slot + static_cast<int>(rank)) * kPartStride + et] = a;
+                }
+                // a warp whose chunk loop ended early (only on a timeout) stored
+                // nothing; all of them leave together
+                for (int w = 0; w < kEpiWarps; ++w) ok = ok && tail->vote[w] != 0;
                 epi_bar();
-                if (!got) {
-                    if (ew == 0 && lane == 0) record_error(ctl, kErrTimeoutPartner);
-                    ok = false;
-                    break;
+            }
+            step_bar();  // every warp is done with this step's table
+            if (max_steps <= 1 || (single && !(due & 4))) continue;
+            // ---- control step between two products: everything this step
+            // wrote is visible before it, its decisions before the next product
+            __threadfence();
+            fence_proxy_async_global();
+            epi_bar();
+            // (a CTA that failed meets the others all the same: the control step
+            // sees its error and ends every problem)
+            auto meet = [&]() {
+                if (et == 0) tail->step_ok = grid_meet(&ctl->sym_bar, gridDim.x, ctl, wait_ns) ? 1 : 0;
+                epi_bar();
+                const bool met = tail->step_ok != 0;
+                epi_bar();
+                return met;
+            };
+            bool met = meet();
+            if (met && (due & 4)) {
+                for (int p = 0; p < nprobs; ++p) {
+                    const MmaProb &pr = probs[p];
+                    if (row_work(row, p) == 0 || !pr.st->op.ref_sums) continue;
+                    for (int k = blockIdx.x; k < pr.ref_ntiles; k += gridDim.x)
+                        ref_tile_sums(pr, k, tail->red, et, [] { epi_bar(); });
                 }
                 __threadfence();
-#pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    if (4 * c >= ncol) break;
-                    const float4 p4 = __ldcg(wsp + c);
-                    acc[4 * c] += p4.x;
-                    acc[4 * c + 1] += p4.y;
-                    acc[4 * c + 2] += p4.z;
-                    acc[4 * c + 3] += p4.w;
-                }
                 epi_bar();
-                if (ew == 0 && lane == 0) {
-                    atomicExch(&cnt[2 * slot], 0);
-                    atomicExch(&cnt[2 * slot + 1], 0);
-                }
+                met = meet();
             }
-
-            // ---- store phase for the strip of block J (J = 2 Jp + h when bn =
-            // 256, else J = Jp and columns 64 h .. 64 h + 63 of it)
-            // Lane = row i of the warp's 32-row strip.  The masters E1/E2 are
-            // symmetric, so they are read at (j, i): lanes on consecutive
-            // addresses.  Mirrored writes (j, i) are coalesced the same way;
-            // direct writes (i, j) go through a per-warp staging buffer so that
-            // each store instruction covers 4 rows x 8 consecutive columns.
-            // Columns are taken 8 at a time.  E1/E2 are re-read per output (L1
-            // hits): the control kernel lets an output overwrite E1/E2 in place
-            // only when it is the step's single output.
-            const ProdOp &op = st->op;
-            const float inv = op.inv;
-            const int ldy = pr.ldy, lds = pr.lds, ldx = pr.ldx;
-            const float *E1 = (op.E1 >= 0) ? pr.mats[op.E1].master : nullptr;
-            const float *E2 = (op.E2 >= 0) ? pr.mats[op.E2].master : nullptr;
-            const int nout = op.nout, pout = op.part_out;
-            const float ra = op.ra, rb = op.rb, rc = op.rc;
-            if (lane < nout) {
-                const OutSpec &o = op.out[lane];
-                OutCache &c = tail->oc[ew][lane];
-                c.a = o.a;
-                c.b1 = o.b1;
-                c.b2 = o.b2;
-                c.s = o.s;
-                c.g1r = o.g1r;
-                c.g1c = o.g1c;
-                c.g2r = o.g2r;
-                c.g2c = o.g2c;
-                c.flags = o.flags;
-                c.master = pr.mats[o.mat].master;
-                c.sl0 = pr.mats[o.mat].sl[0];
-                c.sl1 = pr.mats[o.mat].sl[1];
+            if (single) {
+                ok = ok && met;
+                continue;
             }
-            __syncwarp();
-            const int i0 = te.I * kTileM + q * 32;
-            const int i = i0 + lane;
-            const int J = wide ? 2 * te.Jp + h : te.Jp;
-            const int cb = J * kTileM + (wide ? 0 : 64 * h);  // first column of the strip
-            const int ng = ncol / 8;                            // its 8-column groups
-            double tr = 0.0, sq = 0.0, tr1 = 0.0, rr = 0.0;
-            double *stg = tail->stage[ew];
-            float *stf = reinterpret_cast<float *>(stg);
-            const int rsub = lane >> 3, csub = lane & 7;  // direct-write lane layout
-            const bool lean = nout == 1 && pout == 0 && !E2 && op.out[0].flags == (kOutMaster | kOutSlices);
-            if (lean && J >= te.I && cb < n && i0 < n) {
-                // the zero-temperature step: one output a v + b1 E1 + c [i == j].
-                // An 8-column group wholly inside the matrix and above the
-                // diagonal (every element exists and counts twice) takes the
-                // vector path: each lane reads E1 and writes its own row's 8
-                // columns with 16-byte accesses, and the mirrored rows go
-                // through the staging buffer (layout [column][row], stride 33:
-                // conflict-free both ways) so that 4 lanes write 8 consecutive
-                // elements each of one row.  Other groups (the diagonal's, the
-                // matrix edge) take the element-wise path.
-                const bool diag = (J == te.I);
-                const OutSpec &os = op.out[0];
-                const MatSlot &m = pr.mats[os.mat];
-                const float oa = os.a, ob = os.b1, oc = static_cast<float>(os.c), osc = os.s;
-                float *Mo = m.master;
-                __half *S0 = m.sl[0], *S1 = m.sl[1];
-                const int mr = lane >> 2;        // mirrored row within the group
-                const int mc = (lane & 3) * 8;   // its first column within the strip
-                // a group takes the vector path when all of it exists and lies
-                // above the diagonal; its E1 row segment is loaded one group
-                // ahead, so the load's latency overlaps the previous group
-                auto vec_group = [&](int c) {
-                    const int jc = cb + c * 8;
-                    return i0 + 32 <= n && jc + 8 <= n && (!diag || jc >= i0 + 32);
-                };
-                float4 pa = make_float4(0.f, 0.f, 0.f, 0.f), pb = pa;
-                if (vec_group(0)) {
-                    const size_t r0 = static_cast<size_t>(i) * ldy + cb;
-                    pa = *reinterpret_cast<const float4 *>(E1 + r0);
-                    pb = *reinterpret_cast<const float4 *>(E1 + r0 + 4);
+            if (met)
+                for (int p = blockIdx.x; p < nprobs; p += gridDim.x) {
+                    (void)control_one(probs[p], ctl, &tail->ctl, et, [] { epi_bar(); });
+                    epi_bar();
                 }
-#pragma unroll
-                for (int c8 = 0; c8 < kTileM / 8; ++c8) {
-                    const int j0 = cb + c8 * 8;
-                    if (c8 >= ng || j0 >= n) break;
-                    const float4 ea = pa, eb = pb;  // this group's E1 (when it is a vector group)
-                    if (c8 + 1 < ng && vec_group(c8 + 1)) {
-                        const size_t rn = static_cast<size_t>(i) * ldy + j0 + 8;
-                        pa = *reinterpret_cast<const float4 *>(E1 + rn);
-                        pb = *reinterpret_cast<const float4 *>(E1 + rn + 4);
-                    }
-                    if (diag && j0 + 7 < i0) continue;
-                    const bool full = vec_group(c8);
-                    if (full) {
-                        const size_t ro = static_cast<size_t>(i) * ldy + j0;
-                        const float e[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
-                        float val[8];
-                        float csq = 0.0f, crr = 0.0f;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const float v = acc[c8 * 8 + u] * inv;
-                            val[u] = fmaf(oa, v, ob * e[u]);
-                            const float r = fmaf(ra, v, rb * e[u]);
-                            csq = fmaf(val[u], val[u], csq);
-                            crr = fmaf(r, r, crr);
-                            stf[u * 33 + lane] = val[u];
-                        }
-                        sq += 2.0 * static_cast<double>(csq);
-                        rr += 2.0 * static_cast<double>(crr);
-                        *reinterpret_cast<float4 *>(Mo + ro) = make_float4(val[0], val[1], val[2], val[3]);
-                        *reinterpret_cast<float4 *>(Mo + ro + 4) = make_float4(val[4], val[5], val[6], val[7]);
-                        uint4 hv, lv;
-                        split8(val, osc, hv, lv);
-                        const size_t so = static_cast<size_t>(i) * lds + j0;
-                        *reinterpret_cast<uint4 *>(S0 + so) = hv;
-                        *reinterpret_cast<uint4 *>(S1 + so) = lv;
-                        __syncwarp();
-                        float w[8];
-#pragma unroll
-                        for (int t2 = 0; t2 < 8; ++t2) w[t2] = stf[mr * 33 + mc + t2];
-                        __syncwarp();
-                        const size_t mo = static_cast<size_t>(j0 + mr) * ldy + i0 + mc;
-                        *reinterpret_cast<float4 *>(Mo + mo) = make_float4(w[0], w[1], w[2], w[3]);
-                        *reinterpret_cast<float4 *>(Mo + mo + 4) = make_float4(w[4], w[5], w[6], w[7]);
-                        split8(w, osc, hv, lv);
-                        const size_t ms = static_cast<size_t>(j0 + mr) * lds + i0 + mc;
-                        *reinterpret_cast<uint4 *>(S0 + ms) = hv;
-                        *reinterpret_cast<uint4 *>(S1 + ms) = lv;
-                        continue;
-                    }
-                    float csq = 0.0f, crr = 0.0f;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int j = j0 + u;
-                        float val = 0.0f;
-                        if (i < n && j < n && (!diag || j >= i)) {
-                            const bool on_diag = (j == i);
-                            const size_t mt = static_cast<size_t>(j) * ldy + i;
-                            const float v = acc[c8 * 8 + u] * inv;
-                            const float e1 = E1 ? E1[mt] : 0.0f;
-                            val = fmaf(oa, v, ob * e1) + (on_diag ? oc : 0.0f);
-                            const float r = fmaf(ra, v, rb * e1) + (on_diag ? rc : 0.0f);
-                            if (!on_diag) {
-                                Mo[mt] = val;
-                                const float ys = val * osc;
-                                const __half hh = __float2half_rn(ys);
-                                const size_t ms = static_cast<size_t>(j) * lds + i;
-                                S0[ms] = hh;
-                                S1[ms] = __float2half_rn(ys - __half2float(hh));
-                            } else {
-                                tr += static_cast<double>(val);
-                            }
-                            csq = fmaf(on_diag ? val : 2.0f * val, val, csq);
-                            crr = fmaf(on_diag ? r : 2.0f * r, r, crr);
-                        }
-                        stf[lane * 9 + u] = val;
-                    }
-                    sq += static_cast<double>(csq);
-                    rr += static_cast<double>(crr);
-                    __syncwarp();
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const int ii = i0 + 4 * k + rsub, jj = j0 + csub;
-                        if (ii < n && jj < n && (!diag || jj >= ii)) {
-                            const float val = stf[(4 * k + rsub) * 9 + csub];
-                            Mo[static_cast<size_t>(ii) * ldy + jj] = val;
-                            const float ys = val * osc;
-                            const __half hh = __float2half_rn(ys);
-                            const size_t ms = static_cast<size_t>(ii) * lds + jj;
-                            S0[ms] = hh;
-                            S1[ms] = __float2half_rn(ys - __half2float(hh));
-                        }
-                    }
-                    __syncwarp();
-                }
-            } else if (J >= te.I && cb < n && i0 < n) {
-                // any other step (1-3 outputs, E1/E2, FP64 outputs): groups
-                // wholly above the diagonal take the 16-byte path as in the
-                // zero-temperature step (one output after another; an output
-                // overwrites E1/E2 in place only when it is the single one)
-                const bool diag = (J == te.I);
-                bool has_f64 = false;
-                for (int o = 0; o < nout; ++o) has_f64 = has_f64 || (op.out[o].flags & (kOutF64a | kOutF64b));
-                // diagonal form: the outputs of one step share their E1 / E2
-                // coefficient vectors (the control kernel sets them so); the
-                // row's entries are read once per strip, the columns' once per group
-                int ev1 = -1, ev2 = -1;
-                for (int o = 0; o < nout; ++o) {
-                    if (!(op.out[o].flags & kOutDiag)) continue;
-                    if (op.out[o].v1 >= 0) ev1 = op.out[o].v1;
-                    if (op.out[o].v2 >= 0) ev2 = op.out[o].v2;
-                }
-                bool dup = false;  // a diagonal-form step: its masters are upper-triangular
-                for (int o = 0; o < nout; ++o) dup = dup || (op.out[o].flags & kOutDiag);
-                const float *F1 = (ev1 >= 0) ? pr.dgf[ev1] : nullptr;
-                const float *F2 = (ev2 >= 0) ? pr.dgf[ev2] : nullptr;
-                const float d1i = (F1 && i < n) ? F1[i] : 0.0f;
-                const float d2i = (F2 && i < n) ? F2[i] : 0.0f;
-                const int mr = lane >> 2, mc = (lane & 3) * 8;
-#pragma unroll
-                for (int c8 = 0; c8 < kTileM / 8; ++c8) {
-                    const int j0 = cb + c8 * 8;
-                    if (c8 >= ng || j0 >= n) break;
-                    if (diag && j0 + 7 < i0) continue;  // strictly below the diagonal
-                    if (!has_f64 && i0 + 32 <= n && j0 + 8 <= n && (!diag || j0 >= i0 + 32)) {
-                        const size_t ro = static_cast<size_t>(i) * ldy + j0;
-                        float e1[8], e2[8], v[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) { e1[u] = 0.0f; e2[u] = 0.0f; }
-                        if (E1) {
-                            const float4 a4 = *reinterpret_cast<const float4 *>(E1 + ro);
-                            const float4 b4 = *reinterpret_cast<const float4 *>(E1 + ro + 4);
-                            e1[0] = a4.x; e1[1] = a4.y; e1[2] = a4.z; e1[3] = a4.w;
-                            e1[4] = b4.x; e1[5] = b4.y; e1[6] = b4.z; e1[7] = b4.w;
-                        }
-                        if (E2) {
-                            const float4 a4 = *reinterpret_cast<const float4 *>(E2 + ro);
-                            const float4 b4 = *reinterpret_cast<const float4 *>(E2 + ro + 4);
-                            e2[0] = a4.x; e2[1] = a4.y; e2[2] = a4.z; e2[3] = a4.w;
-                            e2[4] = b4.x; e2[5] = b4.y; e2[6] = b4.z; e2[7] = b4.w;
-                        }
-                        float crr = 0.0f;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            v[u] = acc[c8 * 8 + u] * inv;
-                            const float r = fmaf(ra, v[u], rb * e1[u]);
-                            crr = fmaf(r, r, crr);
-                        }
-                        rr += 2.0 * static_cast<double>(crr);
-                        const size_t so = static_cast<size_t>(i) * lds + j0;
-                        const size_t mo = static_cast<size_t>(j0 + mr) * ldy + i0 + mc;
-                        const size_t ms = static_cast<size_t>(j0 + mr) * lds + i0 + mc;
-                        for (int o = 0; o < nout; ++o) {
-                            const OutCache &os = tail->oc[ew][o];
-                            const int fl = os.flags;
-                            float val[8];
-                            float csq = 0.0f;
-                            if (fl & kOutDiag) {
-                                // per-row / per-column coefficients of E1 and E2
-                                const float r1 = fmaf(os.g1r, d1i, os.b1);
-                                const float r2 = fmaf(os.g2r, d2i, os.b2);
-#pragma unroll
-                                for (int u = 0; u < 8; u += 4) {
-                                    // FP32 copies, 32-byte aligned (j0 % 8 == 0, stride % 8 == 0)
-                                    const float4 f1 = F1 ? *reinterpret_cast<const float4 *>(F1 + j0 + u)
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-                                    const float4 f2 = F2 ? *reinterpret_cast<const float4 *>(F2 + j0 + u)
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-                                    val[u] = fmaf(os.a, v[u], fmaf(fmaf(os.g1c, f1.x, r1), e1[u], fmaf(os.g2c, f2.x, r2) * e2[u]));
-                                    val[u + 1] = fmaf(os.a, v[u + 1],
-                                                      fmaf(fmaf(os.g1c, f1.y, r1), e1[u + 1], fmaf(os.g2c, f2.y, r2) * e2[u + 1]));
-                                    val[u + 2] = fmaf(os.a, v[u + 2],
-                                                      fmaf(fmaf(os.g1c, f1.z, r1), e1[u + 2], fmaf(os.g2c, f2.z, r2) * e2[u + 2]));
-                                    val[u + 3] = fmaf(os.a, v[u + 3],
-                                                      fmaf(fmaf(os.g1c, f1.w, r1), e1[u + 3], fmaf(os.g2c, f2.w, r2) * e2[u + 3]));
-                                }
-                            } else {
-#pragma unroll
-                                for (int u = 0; u < 8; ++u) val[u] = fmaf(os.a, v[u], fmaf(os.b1, e1[u], os.b2 * e2[u]));
-                            }
-#pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                csq = fmaf(val[u], val[u], csq);
-                                stf[u * 33 + lane] = val[u];
-                            }
-                            if (o == pout) sq += 2.0 * static_cast<double>(csq);
-                            uint4 hv, lv;
-                            if (fl & kOutMaster) {
-                                *reinterpret_cast<float4 *>(os.master + ro) = make_float4(val[0], val[1], val[2], val[3]);
-                                *reinterpret_cast<float4 *>(os.master + ro + 4) = make_float4(val[4], val[5], val[6], val[7]);
-                            }
-                            if (fl & kOutSlices) {
-                                split8(val, os.s, hv, lv);
-                                *reinterpret_cast<uint4 *>(os.sl0 + so) = hv;
-                                *reinterpret_cast<uint4 *>(os.sl1 + so) = lv;
-                            }
-                            __syncwarp();
-                            float w[8];
-#pragma unroll
-                            for (int t2 = 0; t2 < 8; ++t2) w[t2] = stf[mr * 33 + mc + t2];
-                            __syncwarp();
-                            if ((fl & kOutMaster) && !(fl & kOutDiag)) {  // diagonal form: upper master only
-                                *reinterpret_cast<float4 *>(os.master + mo) = make_float4(w[0], w[1], w[2], w[3]);
-                                *reinterpret_cast<float4 *>(os.master + mo + 4) = make_float4(w[4], w[5], w[6], w[7]);
-                            }
-                            if (fl & kOutSlices) {
-                                split8(w, os.s, hv, lv);
-                                *reinterpret_cast<uint4 *>(os.sl0 + ms) = hv;
-                                *reinterpret_cast<uint4 *>(os.sl1 + ms) = lv;
-                            }
-                        }
-                        continue;
-                    }
-                    // element (i, j0 + u) exists in this block's upper part
-                    auto okf = [&](int u) { return i < n && j0 + u < n && (!diag || j0 + u >= i); };
-                    // E masters of a diagonal-form step hold the upper triangle only
-                    // (read at (i, j)); others are read at (j, i), lanes on
-                    // consecutive addresses
-                    auto e_at = [&](int u) {
-                        return dup ? static_cast<size_t>(i) * ldy + j0 + u : static_cast<size_t>(j0 + u) * ldy + i;
-                    };
-                    auto e1f = [&](int u) { return E1 ? E1[e_at(u)] : 0.0f; };
-                    auto e2f = [&](int u) { return E2 ? E2[e_at(u)] : 0.0f; };
-                    // off-diagonal value of an output (diagonal form: per-row and
-                    // per-column E coefficients)
-                    auto offv = [&](const OutSpec &os, int u) -> float {
-                        const float vv = acc[c8 * 8 + u] * inv;
-                        if (!(os.flags & kOutDiag)) return fmaf(os.a, vv, fmaf(os.b1, e1f(u), os.b2 * e2f(u)));
-                        const int j = j0 + u;
-                        const float c1 = os.b1 + os.g1r * d1i + (F1 ? os.g1c * F1[j] : 0.0f);
-                        const float c2 = os.b2 + os.g2r * d2i + (F2 ? os.g2c * F2[j] : 0.0f);
-                        return fmaf(os.a, vv, fmaf(c1, e1f(u), c2 * e2f(u)));
-                    };
-                    // diagonal entry of an output in the diagonal form, FP64
-                    auto diagv = [&](const OutSpec &os, int u) -> double {
-                        double r = os.c + static_cast<double>(os.a) * static_cast<double>(acc[c8 * 8 + u] * inv);
-                        const double dxv = (os.dx >= 0) ? pr.dg[os.dx][i] : 0.0;
-                        const double dyv = (os.dy >= 0) ? pr.dg[os.dy][i] : 0.0;
-                        return r + os.q * dxv * dyv + os.l1 * dxv + os.l2 * dyv;
-                    };
-                    float crr = 0.0f;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (okf(u)) {
-                            const bool on_diag = (j0 + u == i);
-                            const float r = fmaf(ra, acc[c8 * 8 + u] * inv, rb * e1f(u)) + (on_diag ? rc : 0.0f);
-                            crr = fmaf(on_diag ? r : 2.0f * r, r, crr);
-                        }
-                    }
-                    rr += static_cast<double>(crr);
-                    for (int o = 0; o < nout; ++o) {
-                        const OutSpec &os = op.out[o];
-                        const int fl = os.flags;
-                        if (fl & (kOutF64a | kOutF64b)) {
-                            double *X = pr.Xd[(fl & kOutF64a) ? 0 : 1];
-                            const double *Xa = (fl & kOutF64Add) ? pr.Xd[(fl & kOutF64a) ? 1 : 0] : nullptr;
-#pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                const int j = j0 + u;
-                                const bool on_diag = (j == i);
-                                double d = 0.0;
-                                if (okf(u)) {
-                                    // the FP32 terms summed in FP32 and converted exactly by
-                                    // integer operations: GB300's FP64 pipe (1/64 of the FP32
-                                    // rate) keeps only the FP64 diagonal, the FP64 addend and
-                                    // the squared norm
-                                    if ((fl & kOutDiag) && on_diag) {
-                                        d = diagv(os, u);
-                                    } else if (fl & kOutDiag) {
-                                        d = f32_to_f64(offv(os, u));
-                                    } else {
-                                        d = f32_to_f64(fmaf(os.a, acc[c8 * 8 + u] * inv, fmaf(os.b1, e1f(u), os.b2 * e2f(u))));
-                                        if (on_diag) d += os.c;
-                                    }
-                                    if (Xa) d += Xa[static_cast<size_t>(j) * ldx + i];  // symmetric: read at (j, i)
-                                    if (!on_diag) X[static_cast<size_t>(j) * ldx + i] = d;
-                                    if (o == pout) {
-                                        if (on_diag) tr += d;
-                                        sq = fma(on_diag ? d : 2.0 * d, d, sq);
-                                    }
-                                    if (o == 1 && on_diag) tr1 += d;
-                                }
-                                stg[lane * 9 + u] = d;
-                            }
-                            __syncwarp();
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const int ii = i0 + 4 * k + rsub, jj = j0 + csub;
-                                if (ii < n && jj < n && (!diag || jj >= ii))
-                                    X[static_cast<size_t>(ii) * ldx + jj] = stg[(4 * k + rsub) * 9 + csub];
-                            }
-                            __syncwarp();
-                            continue;
-                        }
-                        const MatSlot &m = pr.mats[os.mat];
-                        const float cdiag = static_cast<float>(os.c);
-                        const bool dform = (fl & kOutDiag) != 0;
-                        float csq = 0.0f;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int j = j0 + u;
-                            const bool on_diag = (j == i);
-                            float val = 0.0f;
-                            if (okf(u)) {
-                                if (dform && on_diag) {
-                                    // the diagonal goes to the FP64 vector; the small part keeps 0
-                                    const double dv = diagv(os, u);
-                                    pr.dg[os.mat][i] = dv;
-                                    pr.dgf[os.mat][i] = static_cast<float>(dv);
-                                    if (o == pout) {
-                                        tr += dv;
-                                        sq += dv * dv;
-                                    }
-                                    if (o == 1) tr1 += dv;
-                                } else {
-                                    val = offv(os, u) + ((on_diag && !dform) ? cdiag : 0.0f);
-                                    if (!on_diag) {
-                                        if ((fl & kOutMaster) && !dform) m.master[static_cast<size_t>(j) * ldy + i] = val;
-                                        if (fl & kOutSlices) put_slices(m, static_cast<size_t>(j) * lds + i, val * os.s);
-                                    }
-                                    if (o == pout) {
-                                        if (on_diag) tr += static_cast<double>(val);
-                                        csq = fmaf(on_diag ? val : 2.0f * val, val, csq);
-                                    }
-                                    if (o == 1 && on_diag) tr1 += static_cast<double>(val);
-                                }
-                            }
-                            stf[lane * 9 + u] = val;
-                        }
-                        if (o == pout) sq += static_cast<double>(csq);
-                        __syncwarp();
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int ii = i0 + 4 * k + rsub, jj = j0 + csub;
-                            if (ii < n && jj < n && (!diag || jj >= ii)) {
-                                const float val = stf[(4 * k + rsub) * 9 + csub];
-                                if (fl & kOutMaster) m.master[static_cast<size_t>(ii) * ldy + jj] = val;
-                                if (fl & kOutSlices) put_slices(m, static_cast<size_t>(ii) * lds + jj, val * os.s);
-                            }
-                        }
-                        __syncwarp();
-                    }
-                }
-            }
-            // deterministic per-tile partials: warp tree, then the 8 warps in order
-            tr = warp_sum(tr);
-            sq = warp_sum(sq);
-            tr1 = warp_sum(tr1);
-            rr = warp_sum(rr);
-            if (lane == 0) {
-                tail->red[ew][0] = tr;
-                tail->red[ew][1] = sq;
-                tail->red[ew][2] = tr1;
-                tail->red[ew][3] = rr;
-            }
-            epi_bar();
-            if (ew == 0 && lane == 0) {
-                double a = 0, b = 0, c = 0, d = 0;
-                for (int w = 0; w < kEpiWarps; ++w) {
-                    a += tail->red[w][0];
-                    b += tail->red[w][1];
-                    c += tail->red[w][2];
-                    d += tail->red[w][3];
-                }
-                double *slot = pr.part + static_cast<size_t>(te.slot) * kPartStride;
-                slot[0] = a;
-                slot[1] = b;
-                slot[2] = c;
-                slot[3] = d;
-            }
-            epi_bar();
+            ok = met && meet() && ok;
+            controlled = true;
         }
-        if (!ok) tail->abort_flag = 1;
+        if (et == 0 && blockIdx.x == 0 && flags && steps > 0) {
+            flags->n_steps += static_cast<unsigned>(controlled ? steps : steps - 1);
+            flags->controlled = (controlled && ok) ? 1u : 0u;
+            // products of this kernel and of another family that are due in the same
+            // step run in the same pass, the next one
+            ctl->hold = (controlled && ok && (last_due & 1) && (last_due & 2)) ? 1 : 0;
+        }
     }
 
     tc_fence_before();
     __syncthreads();
+    cluster_sync();  // nothing signals a CTA that has left
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc_pair(tmem_base, 512);
+    }
+}
+
+__global__ void __launch_bounds__(kCtlThreads) k_ref_sums(const MmaProb *__restrict__ probs, int nprobs) {
+    __shared__ double red[kEpiWarps][4];
+    for (int p = 0; p < nprobs; ++p) {
+        const MmaProb &pr = probs[p];
+        if (pr.tc_ntiles == 0 || !tc_kind(step_kind(pr.st)) || !pr.st->op.ref_sums) continue;
+        for (int k = blockIdx.x; k < pr.ref_ntiles; k += gridDim.x)
+            ref_tile_sums(pr, k, red, threadIdx.x, [] { __syncthreads(); });
     }
 }
 
 size_t mma_smem_bytes() { return kMmaSmemBytes; }
+size_t sched_row_bytes() { return sizeof(SchedRow); }
 
 }  // namespace fe
