@@ -185,12 +185,9 @@ struct fe_ctx {
     long long n_submitted = 0, n_deferred = 0;
     long long peak_waiting = 0, peak_running = 0;
     // fe_project / fe_rotate: FP16 slices of both operands and split-K
-    // partial tiles (one arena, grown on demand), argument block, tile list
+    // partial tiles (one arena, grown on demand)
     char *gws = nullptr;
     size_t gws_cap = 0;
-    GemmArgs *d_gargs = nullptr;
-    TileEnt *d_gtiles = nullptr;
-    size_t gtiles_cap = 0;
     unsigned long long *d_amax = nullptr;
 };
 
@@ -578,6 +575,7 @@ constexpr double kCostChunkMin = 1200.0;  // ... at least: the hand-over's laten
 constexpr double kCostChunkCol = 1.5;     // ... growing a little with the columns
 constexpr double kCostTile = 10000.0;     // fill, hand-offs, partials
 constexpr double kCostStore = 230.0;      // store phase, per column
+constexpr double kCostGemmStore = 60.0;   // ... of a k_gemm_split tile
 
 int validate(fe_ctx *ctx, const fe_problem *p) {
     if (!p) return set_err(ctx, FE_EINVAL, "problem is NULL");
@@ -1718,8 +1716,6 @@ extern "C" int fe_destroy(fe_ctx *ctx) {
     ctx->slots.clear();
     for (cudaEvent_t ev : ctx->pev) cudaEventDestroy(ev);
     if (ctx->gws) cudaFree(ctx->gws);
-    if (ctx->d_gargs) cudaFree(ctx->d_gargs);
-    if (ctx->d_gtiles) cudaFree(ctx->d_gtiles);
     if (ctx->d_amax) cudaFree(ctx->d_amax);
     delete ctx;
     return FE_OK;
@@ -2029,22 +2025,17 @@ namespace {
 
 // Run C = A B^T (k_gemm_split, + k_gemm_reduce in split mode) on the
 // context's stream with the slices already in the workspace; blocking.
-int run_gemm(fe_ctx *ctx, const GemmArgs &ga, const std::vector<TileEnt> &tl, const char *what) {
+int run_gemm(fe_ctx *ctx, const GemmArgs &ga, const char *what) {
     Engine &eg = ctx->eng;
     cudaStream_t q = eg.stream;
-    int rc = ensure_dev(ctx, &ctx->d_gtiles, &ctx->gtiles_cap, tl.size());
-    if (rc != FE_OK) return rc;
-    FE_CUDA(ctx, cudaMemcpyAsync(ctx->d_gargs, &ga, sizeof(GemmArgs), cudaMemcpyHostToDevice, q));
-    FE_CUDA(ctx, cudaMemcpyAsync(ctx->d_gtiles, tl.data(), sizeof(TileEnt) * tl.size(), cudaMemcpyHostToDevice, q));
     FE_CUDA(ctx, cudaMemsetAsync(eg.d_err, 0, sizeof(int), q));
     const int units = ga.ntiles * (ga.nsplit > 0 ? ga.nsplit : 1);
     FE_CUDA(ctx, cudaEventRecord(eg.ev_setup, q));
-    k_gemm_split<<<std::min(units, ctx->num_sms), kGemmThreads, gemm_smem_bytes(), q>>>(ctx->d_gargs, ctx->d_gtiles,
-                                                                                        eg.d_err);
+    k_gemm_split<<<std::min(2 * units, ctx->sym_grid), kSymThreads, gemm_smem_bytes(), q>>>(ga, eg.d_err);
     ctx->launches += 1;
     FE_CUDA(ctx, cudaEventRecord(eg.ev_loop, q));
     if (ga.nsplit > 0) {
-        k_gemm_reduce<<<dim3(ga.ntiles, kGemmN / 16), 256, 0, q>>>(ctx->d_gargs, ctx->d_gtiles);
+        k_gemm_reduce<<<dim3(2 * ga.ntiles, ga.bn / 16), 256, 0, q>>>(ga);
         ctx->launches += 1;
     }
     FE_CUDA(ctx, cudaEventRecord(eg.ev1, q));
@@ -2069,7 +2060,6 @@ int run_gemm(fe_ctx *ctx, const GemmArgs &ga, const std::vector<TileEnt> &tl, co
 
 // Workspace of `bytes` and the small device blocks of the GEMM path.
 int gemm_workspace(fe_ctx *ctx, size_t bytes) {
-    if (!ctx->d_gargs) FE_CUDA(ctx, cudaMalloc(&ctx->d_gargs, sizeof(GemmArgs)));
     if (!ctx->d_amax) FE_CUDA(ctx, cudaMalloc(&ctx->d_amax, 2 * sizeof(unsigned long long)));
     if (bytes <= ctx->gws_cap) return FE_OK;
     if (ctx->gws) cudaFree(ctx->gws);
@@ -2085,11 +2075,38 @@ int gemm_workspace(fe_ctx *ctx, size_t bytes) {
     return FE_OK;
 }
 
-// Blocks of k_split_rows: one per row (direct) or per 64 x 64 tile
-// (transposed), at most 8 per SM (the kernel loops).
-int split_grid(fe_ctx *ctx, int64_t rows, int64_t cols, bool transpose) {
-    const int64_t t = transpose ? ((rows + 63) / 64) * ((cols + 63) / 64) : rows;
-    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(t, 8LL * ctx->num_sms)));
+// Tile width of a product with K parts of `chunks` 64-wide chunks: the one whose
+// rounds of tiles over the CTA pairs take least, by the cost of a tile as in
+// choose_widths (count(bn): work units at that width).
+template <class Count>
+int gemm_width(fe_ctx *ctx, int chunks, Count count) {
+    int best = kWidths[0];
+    double best_cost = DBL_MAX;
+    for (int bn : kWidths) {
+        const double t = chunks * std::max(kCostChunkMin + kCostChunkCol * bn, kCostChunkMma * bn) + kCostTile +
+                         kCostGemmStore * bn;
+        const double cost = std::ceil(static_cast<double>(count(bn)) / (0.5 * ctx->sym_grid)) * t;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = bn;
+        }
+    }
+    return best;
+}
+
+int64_t blocks64(int64_t x) { return (x + 63) / 64; }
+
+// Largest magnitudes and slices of both operands; a block of k_split per 64 x 64
+// tile, at most 6 per SM and operand (the kernels loop).
+cudaError_t launch_split(fe_ctx *ctx, const SplitArgs &sa) {
+    int64_t t = 1;
+    for (const SplitArgs::Op &o : sa.op) t = std::max(t, blocks64(o.rows) * blocks64(o.cols));
+    const int64_t rows = std::max(sa.op[0].rows, sa.op[1].rows);
+    k_absmax<<<dim3(static_cast<unsigned>(std::min<int64_t>(rows, 4LL * ctx->num_sms)), 2), 256, 0,
+               ctx->eng.stream>>>(sa);
+    k_split<<<dim3(static_cast<unsigned>(std::min<int64_t>(t, 6LL * ctx->num_sms)), 2), 256, 0, ctx->eng.stream>>>(sa);
+    ctx->launches += 2;
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -2104,23 +2121,22 @@ extern "C" int fe_project(fe_ctx *ctx, const double *Psi, const double *HPsi, in
     cudaStream_t q = ctx->eng.stream;
     const int64_t lds = static_cast<int64_t>(align_up(static_cast<size_t>(m), 8));  // slices of Psi^T: n rows of m
     const int nk = static_cast<int>((m + kTileK - 1) / kTileK);
-    // upper-triangle tiles: 128-row block I, 192-column panel J holding some j >= i
-    std::vector<TileEnt> tl;
-    const int TI = static_cast<int>((n + kTileM - 1) / kTileM), TJ = static_cast<int>((n + kGemmN - 1) / kGemmN);
-    for (int J = 0; J < TJ; ++J)
-        for (int I = 0; I < TI; ++I)
-            if (static_cast<int64_t>(J) * kGemmN + kGemmN - 1 >= static_cast<int64_t>(I) * kTileM)
-                tl.push_back(TileEnt{0, I, J, 0});
-    const int ntiles = static_cast<int>(tl.size());
-    // K parts: at most 128 chunks (K = 8192) summed in FP32 per part, and
-    // enough work units for about six waves over the SMs; at least 8 chunks a part
-    int S = std::max((nk + 127) / 128, (6 * ctx->num_sms + ntiles - 1) / ntiles);
+    // K parts: at most 128 chunks (K = 8192) summed in FP32 per part, at least 8
+    // chunks a part, and about 912 parts of 128 x 192 blocks over the upper
+    // triangle (six for each of 152 SMs).  The cut decides the rounding, so it does
+    // not follow the tiles.
+    const int TI = static_cast<int>((n + kTileM - 1) / kTileM), TJ = static_cast<int>((n + 191) / 192);
+    int64_t blocks = 0;
+    for (int J = 0; J < TJ; ++J) blocks += std::min<int64_t>(TI, (static_cast<int64_t>(J) * 192 + 191) / kTileM + 1);
+    int S = std::max((nk + 127) / 128, static_cast<int>((6 * ctx->num_sms + blocks - 1) / blocks));
     S = std::max(1, std::min(S, std::max(1, nk / 8)));
     const int cs = (nk + S - 1) / S;
     S = (nk + cs - 1) / cs;  // every part non-empty
+    const int bn = gemm_width(ctx, cs, [&](int w) { return num_tiles_tc(n, w) * S; });
+    const int ntiles = static_cast<int>(num_tiles_tc(n, bn));
     const size_t slice = 2 * static_cast<size_t>(n) * static_cast<size_t>(lds);
-    const size_t tsz = static_cast<size_t>(kTileM) * kGemmN * sizeof(float);
-    const size_t bytes = align_up(4 * slice, 1024) + static_cast<size_t>(ntiles) * S * tsz;
+    const size_t tsz = 2 * static_cast<size_t>(kTileM) * bn * sizeof(float);
+    const size_t o_ws = align_up(4 * slice, 1024), bytes = o_ws + static_cast<size_t>(ntiles) * S * tsz;
     int rc = gemm_workspace(ctx, bytes);
     if (rc != FE_OK) return rc;
     __half *sl[4];
@@ -2129,26 +2145,26 @@ extern "C" int fe_project(fe_ctx *ctx, const double *Psi, const double *HPsi, in
     memset(&ga, 0, sizeof(ga));
     for (int k = 0; k < 2 && rc == FE_OK; ++k) {
         rc = encode_map_rect(ctx, &ga.tA[k], sl[k], m, n, lds, kTileM);
-        if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tB[k], sl[2 + k], m, n, lds, kGemmN);
+        if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tB[k], sl[2 + k], m, n, lds, bn / 2);
     }
     if (rc != FE_OK) return rc;
     ga.C = Hp;
     ga.ldc = ldh;
-    ga.ws = reinterpret_cast<float *>(ctx->gws + align_up(4 * slice, 1024));
+    ga.ws = reinterpret_cast<float *>(ctx->gws + o_ws);
     ga.amax = ctx->d_amax;
     ga.rows_a = ga.rows_b = static_cast<int>(n);
     ga.kdim = static_cast<int>(m);
     ga.nsplit = S;
     ga.ntiles = ntiles;
+    ga.bn = bn;
     FE_CUDA(ctx, cudaEventRecord(ctx->eng.ev0, q));
     FE_CUDA(ctx, cudaMemsetAsync(ctx->d_amax, 0, 2 * sizeof(unsigned long long), q));
-    k_absmax<<<4 * ctx->num_sms, 256, 0, q>>>(Psi, m, n, ld, ctx->d_amax);
-    k_absmax<<<4 * ctx->num_sms, 256, 0, q>>>(HPsi, m, n, ld, ctx->d_amax + 1);
-    const int gs = split_grid(ctx, m, n, true);
-    k_split_rows<<<gs, 256, 0, q>>>(Psi, m, n, ld, ctx->d_amax, sl[0], sl[1], lds, 1);
-    k_split_rows<<<gs, 256, 0, q>>>(HPsi, m, n, ld, ctx->d_amax + 1, sl[2], sl[3], lds, 1);
-    ctx->launches += 4;
-    return run_gemm(ctx, ga, tl, "fe_project");
+    SplitArgs sa;
+    sa.op[0] = {Psi, m, n, ld, sl[0], sl[1], lds, ctx->d_amax};
+    sa.op[1] = {HPsi, m, n, ld, sl[2], sl[3], lds, ctx->d_amax + 1};
+    sa.transpose = 1;
+    FE_CUDA(ctx, launch_split(ctx, sa));
+    return run_gemm(ctx, ga, "fe_project");
 }
 
 extern "C" int fe_rotate(fe_ctx *ctx, const double *Psi, int64_t m, int64_t n, int64_t ldpsi, const double *D,
@@ -2160,13 +2176,12 @@ extern "C" int fe_rotate(fe_ctx *ctx, const double *Psi, int64_t m, int64_t n, i
     cudaSetDevice(ctx->device);
     cudaStream_t q = ctx->eng.stream;
     const int64_t lds = static_cast<int64_t>(align_up(static_cast<size_t>(n), 8));  // K = n
-    std::vector<TileEnt> tl;
-    const int TI = static_cast<int>((m + kTileM - 1) / kTileM), TJ = static_cast<int>((n + kGemmN - 1) / kGemmN);
-    for (int I = 0; I < TI; ++I)
-        for (int J = 0; J < TJ; ++J) tl.push_back(TileEnt{0, I, J, 0});
-    const size_t sa = 2 * static_cast<size_t>(m) * static_cast<size_t>(lds);
-    const size_t sb = 2 * static_cast<size_t>(n) * static_cast<size_t>(lds);
-    const size_t oa = align_up(sa, 1024), ob = align_up(sb, 1024);
+    const int P = static_cast<int>((m + 255) / 256);
+    const int nk = static_cast<int>(blocks64(n));
+    const int bn = gemm_width(ctx, nk, [&](int w) { return static_cast<int64_t>(P) * ((n + w - 1) / w); });
+    const int CJ = static_cast<int>((n + bn - 1) / bn);
+    const size_t oa = align_up(2 * static_cast<size_t>(m) * static_cast<size_t>(lds), 1024);
+    const size_t ob = align_up(2 * static_cast<size_t>(n) * static_cast<size_t>(lds), 1024);
     int rc = gemm_workspace(ctx, 2 * oa + 2 * ob);
     if (rc != FE_OK) return rc;
     __half *ah = reinterpret_cast<__half *>(ctx->gws), *al = reinterpret_cast<__half *>(ctx->gws + oa);
@@ -2175,8 +2190,8 @@ extern "C" int fe_rotate(fe_ctx *ctx, const double *Psi, int64_t m, int64_t n, i
     memset(&ga, 0, sizeof(ga));
     rc = encode_map_rect(ctx, &ga.tA[0], ah, n, m, lds, kTileM);
     if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tA[1], al, n, m, lds, kTileM);
-    if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tB[0], bh, n, n, lds, kGemmN);
-    if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tB[1], bl, n, n, lds, kGemmN);
+    if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tB[0], bh, n, n, lds, bn / 2);
+    if (rc == FE_OK) rc = encode_map_rect(ctx, &ga.tB[1], bl, n, n, lds, bn / 2);
     if (rc != FE_OK) return rc;
     ga.C = Out;
     ga.ldc = ldo;
@@ -2185,15 +2200,17 @@ extern "C" int fe_rotate(fe_ctx *ctx, const double *Psi, int64_t m, int64_t n, i
     ga.rows_b = static_cast<int>(n);
     ga.kdim = static_cast<int>(n);
     ga.nsplit = 0;
-    ga.ntiles = static_cast<int>(tl.size());
+    ga.ntiles = P * CJ;
+    ga.ntj = CJ;
+    ga.bn = bn;
     FE_CUDA(ctx, cudaEventRecord(ctx->eng.ev0, q));
     FE_CUDA(ctx, cudaMemsetAsync(ctx->d_amax, 0, 2 * sizeof(unsigned long long), q));
-    k_absmax<<<4 * ctx->num_sms, 256, 0, q>>>(Psi, m, n, ldpsi, ctx->d_amax);
-    k_absmax<<<4 * ctx->num_sms, 256, 0, q>>>(D, n, n, ldd, ctx->d_amax + 1);
-    k_split_rows<<<split_grid(ctx, m, n, false), 256, 0, q>>>(Psi, m, n, ldpsi, ctx->d_amax, ah, al, lds, 0);
-    k_split_rows<<<split_grid(ctx, n, n, false), 256, 0, q>>>(D, n, n, ldd, ctx->d_amax + 1, bh, bl, lds, 0);
-    ctx->launches += 4;
-    return run_gemm(ctx, ga, tl, "fe_rotate");
+    SplitArgs sa;
+    sa.op[0] = {Psi, m, n, ldpsi, ah, al, lds, ctx->d_amax};
+    sa.op[1] = {D, n, n, ldd, bh, bl, lds, ctx->d_amax + 1};
+    sa.transpose = 0;
+    FE_CUDA(ctx, launch_split(ctx, sa));
+    return run_gemm(ctx, ga, "fe_rotate");
 }
 
 extern "C" int fe_k_profile(fe_ctx *ctx, int enable) {
