@@ -1890,7 +1890,7 @@ extern "C" int fe_k_gershgorin(fe_ctx *ctx, const double *H, int64_t n, int64_t 
     cudaMemcpyAsync(eg.d_probs, &hp, sizeof(MmaProb), cudaMemcpyHostToDevice, q);
     cudaMemcpyAsync(s->st, &st0, sizeof(SolveState), cudaMemcpyHostToDevice, q);
     cudaMemsetAsync(s->bad, 0, sizeof(int), q);
-    k_bounds_rows<<<ceil_div(static_cast<int>(n), 8), 256, 0, q>>>(eg.d_probs, 0, s->rowinfo, s->bad);
+    k_bounds_only<<<ceil_div(static_cast<int>(n), 8), 256, 0, q>>>(H, static_cast<int>(n), ld, s->rowinfo, s->bad);
     k_bounds_reduce<<<1, 1024, 0, q>>>(eg.d_probs, 0, s->rowinfo, s->bad);
     ctx->launches += 2;
     cudaMemcpyAsync(&res, s->st, sizeof(SolveState), cudaMemcpyDeviceToHost, q);

@@ -112,6 +112,8 @@ struct RowInfo {
 
 // Gershgorin row pass: one warp per row.
 __global__ void k_bounds_rows(const MmaProb *probs, int prob, RowInfo *rowinfo, int *bad);
+// The same from Hp alone, without the FP32 copy and the largest magnitudes.
+__global__ void k_bounds_only(const double *H, int n, long long ldh, RowInfo *rowinfo, int *bad);
 // Deterministic reduction of the row info into the state (one block); with
 // the Lanczos estimate off it also prepares X0 from the Gershgorin bounds.
 __global__ void k_bounds_reduce(const MmaProb *probs, int prob, const RowInfo *rowinfo,

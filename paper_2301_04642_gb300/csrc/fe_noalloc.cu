@@ -51,15 +51,8 @@ __global__ void __launch_bounds__(256) k_gershgorin_oneshot(const double *H, int
     const int row = blockIdx.x * kNaRowsPerBlock + (threadIdx.x >> 5);
     if (row < n) {
         const double *h = H + static_cast<long long>(row) * ld;
-        double s = 0.0;
-        int nonfinite = 0;
-        for (int j = lane; j < n; j += 32) {
-            const double v = h[j];
-            if (!isfinite(v)) nonfinite = 1;
-            s += fabs(v);
-        }
-        s = warp_sum(s);
-        nonfinite = __any_sync(0xffffffffu, nonfinite);
+        bool nonfinite;
+        const double s = row_abs_sum(h, n, lane, &nonfinite);
         if (lane == 0) {
             const double d = h[row];
             const double r = s - fabs(d);
