@@ -23,7 +23,7 @@
 // B and the accumulators of its 128 rows, so that a chunk costs a CTA 64 KiB from L2
 // for twice the products of a 128 x 192 tile (80 KiB).  A projection of 131072 x
 // 4096 takes 4.0 ms here (5.5 ms with 128 x 192 tiles of one CTA), the rotation
-// 11.4 ms (12.5 ms); narrow tiles fill the chip for small n (n = 517 from m = 9001:
+// 9.2 ms (12.5 ms); narrow tiles fill the chip for small n (n = 517 from m = 9001:
 // 27 us of 143).  Bound: the tensor cores at large n (6.6 and 13.2 TFLOP in those,
 // 3.5 and 6.9 ms at 1.9 PFLOP/s) and, in the rotation, the 4.3 GB of FP64 output.
 // The width is the one of the least modelled time (gemm_width).
@@ -100,15 +100,33 @@ __device__ __forceinline__ void group_out(const float (&acc)[128], int gr, float
 #undef FE_GROUP
 }
 
-// x 2^e in FP64 by integer operations on the encodings (exact; zero, subnormal,
-// infinite and NaN x and results beyond the normal range take FP64 arithmetic)
+// x 2^e in FP64, rounded to nearest, by integer operations alone: a branch to FP64
+// arithmetic for the rare encodings (which the compiler turned into selects) cost the
+// rotation of 131072 x 4096 2.2 of 11.4 ms, of 20000 x 300 43 of 110 us
 __device__ __forceinline__ double f32_to_f64_scaled(float x, int e) {
     const unsigned b = __float_as_uint(x);
-    const int f = static_cast<int>((b >> 23) & 0xFFu);
-    const int r = f + 896 + e;
-    if (f == 0 || f == 255 || r <= 0 || r >= 2047) return scalbn(static_cast<double>(x), e);
-    return __hiloint2double(static_cast<int>((b & 0x80000000u) | (static_cast<unsigned>(r) << 20) | ((b >> 3) & 0xFFFFFu)),
-                            static_cast<int>(b << 29));
+    unsigned m = b & 0x7FFFFFu;
+    int f = static_cast<int>((b >> 23) & 0xFFu);
+    if (f == 0) {  // zero, or m 2^-149: leading bit to position 23
+        const int z = __clz(static_cast<int>(m)) - 8;
+        f = m ? 1 - z : -100000;
+        m = (m << (z & 31)) & 0x7FFFFFu;
+    }
+    int r = f + 896 + e;
+    unsigned long long v = (static_cast<unsigned long long>(m) << 29);
+    if (f == 255) {
+        r = 2047;  // Inf, NaN
+    } else if (r >= 2047) {
+        r = 2047;
+        v = 0;
+    } else if (r <= 0) {  // subnormal: the 53 bits shifted down, ties to even
+        const int sh = min(1 - r, 60);
+        const unsigned long long w = v | (1ull << 52), half = 1ull << (sh - 1);
+        v = (w + (half - 1) + ((w >> sh) & 1)) >> sh;
+        r = 0;  // a carry to 2^52 is the least normal number
+    }
+    v += (static_cast<unsigned long long>(r) << 52) | (static_cast<unsigned long long>(b >> 31) << 63);
+    return __longlong_as_double(static_cast<long long>(v));
 }
 
 // Work unit u: part u / ntiles of tile u % ntiles.  The parts go outermost, so
@@ -369,7 +387,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSymThreads, 1)
             // an FP64 product with its conversion it took GB300's FP64 pipe (2 lanes a
             // clock and SM) 32 clocks per element and lane.  The loop over the groups
             // stays rolled (only the copy out of acc is unrolled): unrolled sixteen
-            // times with an FP64 buffer the rotation of 131072 x 4096 took 20 ms, 11.4 with
+            // times with an FP64 buffer the rotation of 131072 x 4096 took 20 ms, 9.2 with
             // this.
             const bool pair = (g.ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15u) == 0;
             const int c2 = 2 * (lane & 7), rr = lane >> 3;
@@ -416,8 +434,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSymThreads, 1)
 // chip: the projection from m = 9001 took 397 us with one block per tile (234 us
 // of it here), 191 us with these.  Bound at large n by the FP64 additions (2 per
 // clock and SM); the FP32 terms are widened by integer operations to keep the
-// conversions off that pipe (n = 4096 from m = 131072, 16 parts: 10.87 -> 10.76
-// ms for the projection).  The upper rows go out through shared memory,
+// conversions off that pipe (n = 4096 from m = 131072, 16 parts: 0.56 ms with a
+// branch to the conversion for the rare encodings, 0.31 ms without one).  The upper rows go out through shared memory,
 // 128 bytes at a time; the mirrored ones are written as they are read.
 __global__ void __launch_bounds__(256) k_gemm_reduce(const __grid_constant__ GemmArgs g) {
     constexpr int kCols = 16;
@@ -446,7 +464,7 @@ __global__ void __launch_bounds__(256) k_gemm_reduce(const __grid_constant__ Gem
 #pragma unroll
         for (int q = 0; q < kCols / 2; ++q) v[q] = b[2 * q * kTileM];
 #pragma unroll
-        for (int q = 0; q < kCols / 2; ++q) sum[q] += f32_to_f64(v[q]);
+        for (int q = 0; q < kCols / 2; ++q) sum[q] += f32_to_f64_scaled(v[q], 0);
     }
 #pragma unroll
     for (int q = 0; q < kCols / 2; ++q) {
