@@ -66,7 +66,7 @@ struct Slot {
     float *Y = nullptr;
     double *Xd[2] = {};
     double *Dtmp = nullptr;
-    float *lzv = nullptr;   // Lanczos vectors (3 n FP32)
+    float *lzv = nullptr;   // Lanczos vectors (6 n FP32)
     double *part = nullptr;
     SolveState *st = nullptr;
     RowInfo *rowinfo = nullptr;
@@ -435,7 +435,7 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
     s->Xd[0] = reinterpret_cast<double *>(take(8 * nn * ldx));
     s->Xd[1] = reinterpret_cast<double *>(take(8 * nn * ldx));
     s->Dtmp = reinterpret_cast<double *>(take(8 * nn * nn));
-    s->lzv = reinterpret_cast<float *>(take(4 * 3 * nn));
+    s->lzv = reinterpret_cast<float *>(take(4 * 6 * nn));
     __half *digs[kDigits] = {};
     if (method == kMethodSp2)
         for (int a = 0; a < kDigits; ++a) digs[a] = reinterpret_cast<__half *>(take(2 * nn * lds));
@@ -938,6 +938,8 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
     if (any_lz) {
         // the estimate of every problem that takes one, all at once in one
         // cooperative launch (the kernel skips problems without lz_on)
+        const bool one = tc_chk.size() + f64_chk.size() == 1;
+        const int k1st = tc_chk.empty() ? f64_chk[0] : tc_chk[0];
         int vmax = 0;
         for (int k : tc_chk) vmax = std::max(vmax, static_cast<int>(jobs[k].p->n));
         for (int k : f64_chk) vmax = std::max(vmax, static_cast<int>(jobs[k].p->n));
@@ -947,10 +949,20 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
         DevCtl *ctl = e.d_err;
         unsigned *bar = &e.d_err->lz_bar;
         int kk0 = k0, mm = m;
-        void *args[] = {&probs, &kk0, &mm, &vcap, &narrow, &ctl, &bar};
         FE_CUDA(ctx, cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
-        FE_CUDA(ctx, cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_lanczos_run), dim3(ctx->lz_grid),
-                                                 dim3(kLzThreads), args, sizeof(float) * vcap, s));
+        if (one && vmax <= kLzWarps * ctx->lz_grid) {
+            // a single problem with a row per warp of k_lanczos_run, whose sums
+            // k_lanczos_one repeats; a block per 8 rows, at most one per SM
+            int kk = k1st;
+            void *args[] = {&probs, &kk, &narrow, &ctl, &bar};
+            FE_CUDA(ctx, cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_lanczos_one),
+                                                     dim3(std::min(ceil_div(vmax, 8), ctx->num_sms)), dim3(kLzThreads),
+                                                     args, lz_one_smem(vmax), s));
+        } else {
+            void *args[] = {&probs, &kk0, &mm, &vcap, &narrow, &ctl, &bar};
+            FE_CUDA(ctx, cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_lanczos_run), dim3(ctx->lz_grid),
+                                                     dim3(kLzThreads), args, sizeof(float) * vcap, s));
+        }
         ctx->launches += 1;
     }
     for (int k = k0; k < k1; ++k) k_init_x0<<<kInitBlocks, 256, 0, s>>>(e.d_probs, k);
@@ -1641,7 +1653,9 @@ extern "C" int fe_create(fe_ctx **out, const fe_config *cfg) {
                         cudaFuncSetAttribute(k_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(gemm_smem_bytes())) != cudaSuccess ||
                         cudaFuncSetAttribute(k_lanczos_run, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(sizeof(float) * kLzVcap)) != cudaSuccess))
+                                             static_cast<int>(sizeof(float) * kLzVcap)) != cudaSuccess ||
+                        cudaFuncSetAttribute(k_lanczos_one, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(lz_one_smem(kLzWarps * kLzBlocks))) != cudaSuccess))
         rc = set_err(nullptr, FE_ECUDA, std::string("context setup: ") + cudaGetErrorString(cudaGetLastError()));
     if (rc == FE_OK) {
         // the Lanczos launch waits at grid barriers, so all its blocks must be

@@ -41,7 +41,8 @@ struct MmaProb {
     int ntilesF, pad1;
     int tc_tile0, tc_ntiles;         // this problem's range in the launch's tensor-core tile list
     int ref_bn, ref_ntiles;          // reference tiles (see run_cut in k_mma.cu)
-    float *lzv;                      // Lanczos vectors: v_prev, v, w (n FP32 each)
+    float *lzv;                      // Lanczos vectors: v_prev, v, w (n FP32 each), or in k_lanczos_one two
+                                     // copies of w (n FP32) and of the rows' products (n FP64)
     float *Y;                        // FP32 master of the zero-temperature iterate
     double *Xd[2];                   // FP64 buffers (FP64 phase / finite-T output), ld ldx
     int ldx, pad0;
@@ -131,9 +132,14 @@ __global__ void k_bounds_reduce(const MmaProb *probs, int prob, const RowInfo *r
 // factor (a test hook that forces the too-tight case).
 constexpr int kLzBlocks = 304;
 constexpr int kLzThreads = 512;
+constexpr int kLzWarps = kLzThreads / 32;
 constexpr int kLzVcap = 24576;  // largest v staged in shared memory (96 KiB)
 __global__ void k_lanczos_run(const MmaProb *probs, int k0, int m, int vcap, double narrow, DevCtl *ctl,
                               unsigned *bar);
+// The same for the one problem at table position k, n <= kLzWarps kLzBlocks
+// (dynamic shared memory lz_one_smem(n)); any grid that is resident at once.
+__global__ void k_lanczos_one(const MmaProb *probs, int k, double narrow, DevCtl *ctl, unsigned *bar);
+constexpr size_t lz_one_smem(int n) { return 2 * sizeof(float) * static_cast<size_t>((n + 3) & ~3); }
 // Certified bounds from the certificate steps (kCheckSteps products issued by
 // k_control after k_lanczos_run), then the X0 preparation; one block per
 // problem from k0.

@@ -44,18 +44,43 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     return z ^ (z >> 31);
 }
 
-__device__ __forceinline__ double block_sum_1024(double v, double *sh) {
+// Sum over the block's threads, of which those from `cnt` on hold zero, as a
+// binary tree (t + t + 256, t + t + 128, ...; the zero levels left out); thread 0
+// hands it to `done`, and what that writes to shared memory is visible to all
+// when the call returns.  The scalar arithmetic belongs in `done`: run by every
+// thread, an FP64 square root and a division took the 16 warps of a block 4 us.
+template <class F>
+__device__ __forceinline__ void block_sum(double v, double *sh, int cnt, F done) {
     const int t = threadIdx.x;
-    sh[t] = v;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (t < o) sh[t] += sh[t + o];
+    if (cnt > 32) {
+        int o = kLzThreads / 2;
+        while (o >= cnt) o >>= 1;
+        sh[t] = v;
+        __syncthreads();
+        for (; o >= 32; o >>= 1) {
+            if (t < o) {
+                v += sh[t + o];
+                sh[t] = v;
+            }
+            __syncthreads();
+        }
+    } else {
         __syncthreads();
     }
-    const double r = sh[0];
+    if (t < 32) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (t == 0) done(v);
+    }
     __syncthreads();
-    return r;
 }
+
+// scalars of a step, from thread 0 to its block
+struct LzScalars {
+    float alpha, beta, inv;
+    int stop;
+    double bn;
+};
 
 // number of eigenvalues of the tridiagonal (a, b) below x (Sturm sequence),
 // in FP32 with the squared couplings b2[i] = b[i]^2 (GB300 runs FP64 at 1/64
@@ -86,10 +111,10 @@ __device__ double tri_eig(const float *a, const float *b2, int k, int idx, doubl
         const double x = lo + w * static_cast<double>(lane + 1) / 33.0;
         const unsigned above = __ballot_sync(0xffffffffu, sturm_count_f(a, b2, k, static_cast<float>(x)) > idx);
         const int f = above ? __ffs(above) - 1 : 32;  // first point above the eigenvalue
-        const double nlo = lo + w * static_cast<double>(f) / 33.0;
-        const double nhi = (f < 32) ? lo + w * static_cast<double>(f + 1) / 33.0 : hi;
-        lo = nlo;
-        hi = nhi;
+        // the points either side of it, from the lanes that hold them
+        const double below = __shfl_sync(0xffffffffu, x, (f + 31) & 31), over = __shfl_sync(0xffffffffu, x, f & 31);
+        if (f > 0) lo = below;
+        if (f < 32) hi = over;
     }
     return 0.5 * (lo + hi);
 }
@@ -136,13 +161,13 @@ __device__ bool grid_barrier(unsigned *cnt, unsigned k, unsigned nb, DevCtl *ctl
         const unsigned target = (k + 1u) * nb;
         bool ok = true;
         if (ld_acquire_u32(cnt) < target) {
+            // the timer is slow to read: every 64 polls
             const uint64_t lim = ctl->wait_ns, t0 = globaltimer();
-            while (ld_acquire_u32(cnt) < target) {
-                if (globaltimer() - t0 > lim) {
+            for (unsigned it = 1; ld_acquire_u32(cnt) < target; ++it) {
+                if ((it & 63u) == 0 && globaltimer() - t0 > lim) {
                     ok = false;
                     break;
                 }
-                __nanosleep(32);
             }
         }
         if (!ok) atomicCAS(&ctl->err, 0, kErrTimeoutGrid);
@@ -153,67 +178,88 @@ __device__ bool grid_barrier(unsigned *cnt, unsigned k, unsigned nb, DevCtl *ctl
     return *flag != 0;
 }
 
-// v = fixed pseudo-random unit vector, v_prev = 0 (the whole block)
-__device__ void lz_start(const MmaProb &pr, double *sh) {
-    SolveState *st = pr.st;
-    if (!st->lz_on) return;
-    const int n = pr.n;
-    float *vp = pr.lzv, *v = pr.lzv + n;
+// entry i of the fixed start vector, uniform in [-1, 1)
+__device__ __forceinline__ float lz_entry(int i) {
+    return static_cast<float>(static_cast<double>(mix64(0xF00Dull + static_cast<uint64_t>(i)) >> 11) *
+                              (2.0 / 9007199254740992.0) - 1.0);
+}
+
+// v = the start vector at unit length, vp = 0 (the whole block; either array may
+// be shared or global memory)
+__device__ void lz_unit(float *vp, float *v, int n, double *sh, LzScalars *sc) {
     double ss = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float x = static_cast<float>(static_cast<double>(mix64(0xF00Dull + static_cast<uint64_t>(i)) >> 11) *
-                                           (2.0 / 9007199254740992.0) - 1.0);  // uniform in [-1, 1)
+        const float x = lz_entry(i);
         v[i] = x;
         vp[i] = 0.0f;
         ss += static_cast<double>(x) * x;
     }
-    const double nrm = sqrt(block_sum_1024(ss, sh));
-    const float inv = nrm > 0.0 ? static_cast<float>(1.0 / nrm) : 0.0f;
+    block_sum(ss, sh, n, [&](double sum) {
+        const double nrm = sqrt(sum);
+        sc->inv = nrm > 0.0 ? static_cast<float>(1.0 / nrm) : 0.0f;
+    });
+    const float inv = sc->inv;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] *= inv;
+}
+
+__device__ void lz_start(const MmaProb &pr, double *sh, LzScalars *sc) {
+    SolveState *st = pr.st;
+    if (!st->lz_on) return;
+    lz_unit(pr.lzv, pr.lzv + pr.n, pr.n, sh, sc);
     if (threadIdx.x == 0) {
         st->lz_k = 0;
         st->lz_b[0] = 0.0;
     }
 }
 
-// This block's share of w = H v: rows blockIdx.x * kWarps + warp, stepping
-// by the grid's warps, one warp per row.  H is read from its FP32 copy in the
-// problem's FP32 master (written by k_bounds_rows; rows 16-byte aligned, ld a
-// multiple of 4) as 16-byte quadruples, four per lane in flight.  v comes
-// from shared memory when `vs` holds it, else from L2 (ld.cg: another block
-// wrote it since this launch began, so L1 may hold a stale copy).  The
-// block's partial of w . v goes to its partial slot.
+// sum_j H_row,j v_j by a warp: H from its FP32 copy in the problem's FP32 master
+// (written by k_bounds_rows; rows 16-byte aligned, ld a multiple of 4) as 16-byte
+// quadruples, four per lane in flight
+template <class V4, class V1>
+__device__ __forceinline__ double lz_row(const float *h, int n, int lane, V4 v4, V1 v1) {
+    const int m = n >> 2;
+    const float4 *h4 = reinterpret_cast<const float4 *>(h);
+    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+    int k = lane;
+    auto dot4 = [&](const float4 a, int q, float acc) {
+        const float4 x = v4(q);
+        return fmaf(a.x, x.x, fmaf(a.y, x.y, fmaf(a.z, x.z, fmaf(a.w, x.w, acc))));
+    };
+    for (; k + 96 < m; k += 128) {
+        const float4 a0 = h4[k], a1 = h4[k + 32], a2 = h4[k + 64], a3 = h4[k + 96];
+        s0 = dot4(a0, k, s0);
+        s1 = dot4(a1, k + 32, s1);
+        s2 = dot4(a2, k + 64, s2);
+        s3 = dot4(a3, k + 96, s3);
+    }
+    for (; k < m; k += 32) s0 = dot4(h4[k], k, s0);
+    for (int jj = 4 * m + lane; jj < n; jj += 32) s1 = fmaf(h[jj], v1(jj), s1);
+    return warp_sum(static_cast<double>((s0 + s1) + (s2 + s3)));
+}
+
+// This block's share of w = H v: rows blockIdx.x * kLzWarps + warp, stepping
+// by the grid's warps, one warp per row.  v comes from shared memory when `vs`
+// holds it, else from L2 (ld.cg: another block wrote it since this launch
+// began, so L1 may hold a stale copy).  The block's partial of w . v goes to its
+// partial slot.
 template <bool kStaged>
 __device__ void lz_matvec(const MmaProb &pr, const float *vs, double *red) {
-    constexpr int kWarps = kLzThreads / 32;
+    constexpr int kWarps = kLzWarps;
     const int n = pr.n;
     const float *v = kStaged ? vs : pr.lzv + n;
     float *w = pr.lzv + 2 * static_cast<size_t>(n);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    auto vat = [&](int i) { return kStaged ? v[i] : __ldcg(v + i); };
+    auto v1 = [&](int i) { return kStaged ? v[i] : __ldcg(v + i); };
+    auto v4 = [&](int q) {
+        if (kStaged) return reinterpret_cast<const float4 *>(v)[q];
+        return make_float4(v1(4 * q), v1(4 * q + 1), v1(4 * q + 2), v1(4 * q + 3));  // v at an odd offset
+    };
     double part = 0.0;
     for (int row = blockIdx.x * kWarps + wid; row < n; row += gridDim.x * kWarps) {
-        const float *h = pr.Y + static_cast<size_t>(row) * pr.ldy;
-        const int m = n >> 2;  // 16-byte quadruples
-        const float4 *h4 = reinterpret_cast<const float4 *>(h);
-        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
-        int k = lane;
-        auto dot4 = [&](const float4 a, int q, float acc) {
-            return fmaf(a.x, vat(4 * q), fmaf(a.y, vat(4 * q + 1), fmaf(a.z, vat(4 * q + 2), fmaf(a.w, vat(4 * q + 3), acc))));
-        };
-        for (; k + 96 < m; k += 128) {
-            const float4 a0 = h4[k], a1 = h4[k + 32], a2 = h4[k + 64], a3 = h4[k + 96];
-            s0 = dot4(a0, k, s0);
-            s1 = dot4(a1, k + 32, s1);
-            s2 = dot4(a2, k + 64, s2);
-            s3 = dot4(a3, k + 96, s3);
-        }
-        for (; k < m; k += 32) s0 = dot4(h4[k], k, s0);
-        for (int jj = 4 * m + lane; jj < n; jj += 32) s1 = fmaf(h[jj], vat(jj), s1);
-        const double s = warp_sum(static_cast<double>((s0 + s1) + (s2 + s3)));
+        const double s = lz_row(pr.Y + static_cast<size_t>(row) * pr.ldy, n, lane, v4, v1);
         if (lane == 0) {
             w[row] = static_cast<float>(s);
-            part += s * static_cast<double>(vat(row));
+            part += s * static_cast<double>(v1(row));
         }
     }
     if (lane == 0) red[wid] = part;
@@ -226,71 +272,85 @@ __device__ void lz_matvec(const MmaProb &pr, const float *vs, double *red) {
     __syncthreads();
 }
 
+// beta_{j+1} = ||w'|| from its square, whether the subspace is invariant (to
+// FP32 accuracy), and 1 / beta_{j+1}
+__device__ __forceinline__ void lz_norm(double sum, double alpha, LzScalars *sc) {
+    sc->bn = sqrt(sum);
+    sc->stop = !(sc->bn > 1e-6 * fmax(fabs(alpha), 1e-300));
+    sc->inv = sc->stop ? 0.0f : static_cast<float>(1.0 / sc->bn);
+}
+
 // alpha_j = w . v (the blocks' partials, in block order); w' = w - alpha_j v
 // - beta_j v_prev; beta_{j+1} = ||w'||; v_prev <- v, v <- w' / beta_{j+1}
 // (the whole block; everything another block wrote is read through L2)
-__device__ void lz_update(const MmaProb &pr, int j, double *sh) {
+__device__ void lz_update(const MmaProb &pr, int j, double *sh, LzScalars *sc) {
     SolveState *st = pr.st;
     const int n = pr.n;
     float *vp = pr.lzv, *v = pr.lzv + n, *w = pr.lzv + 2 * static_cast<size_t>(n);
-    double a = 0.0;
+    double a = 0.0, alpha = 0.0;
     for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += blockDim.x)
         a += __ldcg(pr.part + static_cast<size_t>(b) * kPartStride);
-    const double alpha = block_sum_1024(a, sh);
-    const double beta = st->lz_b[j];
-    const float af = static_cast<float>(alpha), bf = static_cast<float>(beta);
+    block_sum(a, sh, static_cast<int>(gridDim.x), [&](double sum) {
+        alpha = sum;
+        sc->alpha = static_cast<float>(sum);
+        sc->beta = static_cast<float>(st->lz_b[j]);
+    });
+    const float af = sc->alpha, bf = sc->beta;
     float ssf = 0.0f;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const float x = fmaf(-af, v[i], fmaf(-bf, vp[i], __ldcg(w + i)));
         w[i] = x;
         ssf = fmaf(x, x, ssf);
     }
-    const double bn = sqrt(block_sum_1024(static_cast<double>(ssf), sh));
-    const bool stop = !(bn > 1e-6 * fmax(fabs(alpha), 1e-300));  // invariant subspace (to FP32 accuracy)
-    const float inv = stop ? 0.0f : static_cast<float>(1.0 / bn);
+    block_sum(static_cast<double>(ssf), sh, n, [&](double sum) { lz_norm(sum, alpha, sc); });
+    const float inv = sc->inv;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         vp[i] = v[i];
         v[i] = w[i] * inv;
     }
     if (threadIdx.x == 0) {
         st->lz_a[j] = alpha;
-        st->lz_b[j + 1] = stop ? 0.0 : bn;
-        st->lz_k = stop ? -(j + 1) : j + 1;  // negative: stopped after |lz_k| steps
+        st->lz_b[j + 1] = sc->stop ? 0.0 : sc->bn;
+        st->lz_k = sc->stop ? -(j + 1) : j + 1;  // negative: stopped after |lz_k| steps
     }
 }
 
-// bounds from the tridiagonal, then the X0 preparation (warp 0 of the block)
+// bounds from the tridiagonal, then the X0 preparation (the whole block; warp 0
+// takes the lowest Ritz pair, warp 1 the highest)
 __device__ void lz_finish(const MmaProb &pr, double narrow) {
     SolveState *st = pr.st;
-    const int lane = threadIdx.x & 31;
+    const int t = threadIdx.x;
     const int k = st->lz_k < 0 ? -st->lz_k : st->lz_k;
     const double glo = st->gersh_lo, ghi = st->gersh_hi;
     __shared__ double a[kLanczosSteps], b[kLanczosSteps + 1];  // b[i] couples i-1 and i, b[k] the residual
     __shared__ float af[kLanczosSteps], b2f[kLanczosSteps + 1];
-    if (lane < kLanczosSteps) {
-        a[lane] = st->lz_a[lane];
-        af[lane] = static_cast<float>(a[lane]);
+    __shared__ double end[2];
+    if (t < kLanczosSteps) {
+        a[t] = st->lz_a[t];
+        af[t] = static_cast<float>(a[t]);
     }
-    if (lane <= kLanczosSteps) {
-        b[lane] = st->lz_b[lane];
-        b2f[lane] = static_cast<float>(b[lane] * b[lane]);
+    if (t <= kLanczosSteps) {
+        b[t] = st->lz_b[t];
+        b2f[t] = static_cast<float>(b[t] * b[t]);
     }
-    __syncwarp();
+    __syncthreads();
+    if (k >= 2 && t < 64) {
+        const bool top = t >= 32;
+        const double th = tri_eig(af, b2f, k, top ? k - 1 : 0, glo, ghi);
+        const double r = b[k] * tri_last_comp(a, b, k, th);
+        if ((t & 31) == 0) end[top] = top ? fmin(ghi, th + r) : fmax(glo, th - r);
+    }
+    __syncthreads();
+    if (t != 0) return;
     double lo = glo, hi = ghi;
     if (k >= 2) {
-        const double tmin = tri_eig(af, b2f, k, 0, glo, ghi);
-        const double tmax = tri_eig(af, b2f, k, k - 1, glo, ghi);
-        const double rmin = b[k] * tri_last_comp(a, b, k, tmin);
-        const double rmax = b[k] * tri_last_comp(a, b, k, tmax);
-        lo = fmax(glo, tmin - rmin);
-        hi = fmin(ghi, tmax + rmax);
+        lo = end[0];
+        hi = end[1];
         if (!(hi > lo)) {
             lo = glo;
             hi = ghi;
         }
     }
-    __syncwarp();
-    if (lane != 0) return;
     if (narrow < 1.0) {
         const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo) * narrow;
         lo = mid - half;
@@ -312,12 +372,13 @@ __device__ void lz_finish(const MmaProb &pr, double narrow) {
 // updating block before the barrier) is skipped from then on.
 __global__ void __launch_bounds__(kLzThreads, 2)
     k_lanczos_run(const MmaProb *probs, int k0, int m, int vcap, double narrow, DevCtl *ctl, unsigned *bar) {
-    extern __shared__ float vs[];  // v of the problem in hand, when n <= vcap
+    extern __shared__ __align__(16) float vs[];  // v of the problem in hand, when n <= vcap
     __shared__ double sh[kLzThreads];
     __shared__ int flag;
+    __shared__ LzScalars sc;
     const unsigned nb = gridDim.x;
     unsigned nbar = 0;
-    for (int q = blockIdx.x; q < m; q += nb) lz_start(probs[k0 + q], sh);
+    for (int q = blockIdx.x; q < m; q += nb) lz_start(probs[k0 + q], sh, &sc);
     if (!grid_barrier(bar, nbar++, nb, ctl, &flag)) return;
     for (int j = 0; j < kLanczosSteps; ++j) {
         for (int q = 0; q < m; ++q) {
@@ -336,14 +397,102 @@ __global__ void __launch_bounds__(kLzThreads, 2)
         if (!grid_barrier(bar, nbar++, nb, ctl, &flag)) return;
         for (int q = blockIdx.x; q < m; q += nb) {
             const MmaProb &pr = probs[k0 + q];
-            if (pr.st->lz_on && pr.st->lz_k >= 0) lz_update(pr, j, sh);
+            if (pr.st->lz_on && pr.st->lz_k >= 0) lz_update(pr, j, sh, &sc);
             __syncthreads();
         }
         if (!grid_barrier(bar, nbar++, nb, ctl, &flag)) return;
     }
-    if (threadIdx.x < 32)
-        for (int q = blockIdx.x; q < m; q += nb)
-            if (probs[k0 + q].st->lz_on) lz_finish(probs[k0 + q], narrow);
+    for (int q = blockIdx.x; q < m; q += nb) {
+        if (probs[k0 + q].st->lz_on) lz_finish(probs[k0 + q], narrow);
+        __syncthreads();
+    }
+}
+
+// The estimate of one problem with at most kLzWarps `parts` rows, every block
+// keeping v and v_prev in shared memory and making the update itself (the same
+// arithmetic in each): a step has one grid barrier, and no block waits for
+// another's update.  Row r is a warp of block r % grid; w and the rows'
+// products w_r v_r go through L2, in two copies that alternate, so that a step
+// may write while a slower block still reads the step before.  The products
+// are added as k_lanczos_run adds them (16 rows in order, then a tree over
+// those groups), so both kernels give the same bounds.
+// All 12 steps and the end: n = 384 in 261 us with two barriers a step and the
+// scalar arithmetic in every thread, 102 us here; n = 4096 in 376 and 212 us.  A
+// step is bound by the latencies of the barrier and of the two sums, at n = 4096
+// also by the 67 MB of H from L2.
+__global__ void __launch_bounds__(kLzThreads, 1)
+    k_lanczos_one(const MmaProb *probs, int k, double narrow, DevCtl *ctl, unsigned *bar) {
+    extern __shared__ float4 dyn[];
+    __shared__ double sh[kLzThreads];
+    __shared__ int flag;
+    __shared__ LzScalars sc;
+    const MmaProb &pr = probs[k];
+    SolveState *st = pr.st;
+    const int n = pr.n, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const unsigned nb = gridDim.x;
+    float *v = reinterpret_cast<float *>(dyn), *vp = v + ((n + 3) & ~3);
+    const bool first = blockIdx.x == 0 && t == 0;
+    double alpha = 0.0, beta = 0.0;  // thread 0
+    lz_unit(vp, v, n, sh, &sc);
+    if (first) {
+        st->lz_k = 0;
+        st->lz_b[0] = 0.0;
+    }
+    __syncthreads();
+    const int groups = (n + kLzWarps - 1) / kLzWarps;
+    for (int j = 0; j < kLanczosSteps; ++j) {
+        float *w = pr.lzv + static_cast<size_t>(j & 1) * n;
+        double *rp = reinterpret_cast<double *>(pr.lzv + 2 * static_cast<size_t>(n)) + static_cast<size_t>(j & 1) * n;
+        for (int row = wid * static_cast<int>(nb) + static_cast<int>(blockIdx.x); row < n; row += kLzWarps * static_cast<int>(nb)) {
+            const double s = lz_row(pr.Y + static_cast<size_t>(row) * pr.ldy, n, lane,
+                                    [&](int q) { return reinterpret_cast<const float4 *>(v)[q]; },
+                                    [&](int i) { return v[i]; });
+            if (lane == 0) {
+                w[row] = static_cast<float>(s);
+                rp[row] = s * static_cast<double>(v[row]);
+            }
+        }
+        if (!grid_barrier(bar, static_cast<unsigned>(j), nb, ctl, &flag)) return;
+        double a = 0.0;
+        if (t < groups) {
+            double p[kLzWarps];
+#pragma unroll
+            for (int q = 0; q < kLzWarps; ++q) {
+                const int r = t * kLzWarps + q;
+                p[q] = r < n ? __ldcg(rp + r) : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < kLzWarps; ++q) a += p[q];
+        }
+        block_sum(a, sh, groups, [&](double sum) {
+            alpha = sum;
+            sc.alpha = static_cast<float>(sum);
+            sc.beta = static_cast<float>(beta);
+        });
+        const float af = sc.alpha, bf = sc.beta;
+        float ssf = 0.0f;
+        for (int i = t; i < n; i += kLzThreads) {
+            const float x = fmaf(-af, v[i], fmaf(-bf, vp[i], __ldcg(w + i)));
+            vp[i] = v[i];
+            v[i] = x;
+            ssf = fmaf(x, x, ssf);
+        }
+        block_sum(static_cast<double>(ssf), sh, n, [&](double sum) {
+            lz_norm(sum, alpha, &sc);
+            beta = sc.stop ? 0.0 : sc.bn;
+        });
+        const float inv = sc.inv;
+        const bool stop = sc.stop;
+        for (int i = t; i < n; i += kLzThreads) v[i] *= inv;
+        if (first) {
+            st->lz_a[j] = alpha;
+            st->lz_b[j + 1] = beta;
+            st->lz_k = stop ? -(j + 1) : j + 1;  // negative: stopped after |lz_k| steps
+        }
+        __syncthreads();
+        if (stop) break;
+    }
+    if (blockIdx.x == 0) lz_finish(pr, narrow);
 }
 
 // Certified bounds from the check steps, then the X0 preparation (one thread
