@@ -1165,32 +1165,41 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
         coop.cooperative = 1;
         FE_CUDA(ctx, cudaGraphKernelNodeSetAttribute(kn, cudaLaunchAttributeCooperative, &coop));
     }
-    if (e.any_fp64) {
-        const TileF64 *tl = e.d_tilesF;
-        int nt = e.nF;
-        void *args[] = {&probs, &tl, &nt, &err};
-        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_fp64_step),
-                                std::max(1, std::min(e.nF, 8 * ctx->num_sms)), 256, 0, args, prev, &kn));
-        prev = kn;
-    }
-    if (e.any_digit) {
-        int npp = np;
-        void *pargs[] = {&probs, &npp, &err};
-        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_digit_prep), 2 * ctx->num_sms, 256, 0, pargs,
-                                prev, &kn));
-        const TileEnt *tl = e.d_tilesD;
-        int nt = e.nD;
-        void *args[] = {&probs, &tl, &nt, &err};
-        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_digit_mma),
-                                std::max(1, std::min(e.nD, ctx->num_sms)), kMmaThreads, digit_smem_bytes(), args, kn,
-                                &kn2));
-        prev = kn2;
-    }
-    {
-        int npp = np, has_tc = e.any_tc ? 1 : 0;
-        StepFlags *fl = e.d_flags;
-        void *args[] = {&probs, &npp, &err, &fl, &hl, &ht, &has_tc};
-        FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_control), np, 256, 0, args, prev, &kn));
+    // A table of FP64 problems alone takes four products and controls a pass: a pass
+    // of the while node costs 3.4 us besides its kernels, and kernels that find the
+    // problems done leave at once (n = 256, 25 steps: 1.363 ms a solve with one,
+    // 1.325 with two, 1.303 with four, 1.316 with eight).
+    constexpr int kFp64Unroll = 4;
+    const bool fp64_only = e.any_fp64 && !e.any_tc && !e.any_digit;
+    for (int u = 0; u < (fp64_only ? kFp64Unroll : 1); ++u) {
+        if (e.any_fp64) {
+            const TileF64 *tl = e.d_tilesF;
+            int nt = e.nF;
+            void *args[] = {&probs, &tl, &nt, &err};
+            FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_fp64_step),
+                                    std::max(1, std::min(e.nF, 8 * ctx->num_sms)), 256, 0, args, prev, &kn));
+            prev = kn;
+        }
+        if (e.any_digit) {
+            int npp = np;
+            void *pargs[] = {&probs, &npp, &err};
+            FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_digit_prep), 2 * ctx->num_sms, 256, 0, pargs,
+                                    prev, &kn));
+            const TileEnt *tl = e.d_tilesD;
+            int nt = e.nD;
+            void *args[] = {&probs, &tl, &nt, &err};
+            FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_digit_mma),
+                                    std::max(1, std::min(e.nD, ctx->num_sms)), kMmaThreads, digit_smem_bytes(), args, kn,
+                                    &kn2));
+            prev = kn2;
+        }
+        {
+            int npp = np, has_tc = e.any_tc ? 1 : 0;
+            StepFlags *fl = e.d_flags;
+            void *args[] = {&probs, &npp, &err, &fl, &hl, &ht, &has_tc};
+            FE_CUDA(ctx, add_kernel(body, reinterpret_cast<const void *>(k_control), np, 256, 0, args, prev, &kn));
+            prev = kn;
+        }
     }
     FE_CUDA(ctx, cudaGraphInstantiate(&e.gexec, g, 0));
     e.gkey = key;
@@ -2370,7 +2379,7 @@ extern "C" int fe_autotune(fe_ctx *ctx, int count, const int64_t *ns, uint32_t p
         p.n_e = static_cast<double>(ne);
         p.flags = FE_PTR_DEVICE | FE_METHOD_SP2 | prec;
         // throughput, not latency: enough copies of the problem in one batch
-        // for two waves of 128 x 256 tiles over the SMs (at most 16 copies;
+        // for two waves of 128 x 256 blocks over the SMs (at most 16 copies;
         // they share the read-only Hp)
         const int wide_tiles = T * ((T + 1) / 2);
         const int copies = std::max(1, std::min(16, (2 * ctx->num_sms + wide_tiles - 1) / wide_tiles));
