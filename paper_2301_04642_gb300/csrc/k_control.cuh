@@ -1080,16 +1080,29 @@ __device__ __forceinline__ bool control_one(const MmaProb &pr, const DevCtl *ctl
         sh->s[0][t] = a;
         sh->s[1][t] = b;
         bar();
-        for (int o = kCtlThreads / 2; o > 0; o >>= 1) {
+        int o = kCtlThreads / 2;
+        while (o >= 32 && o >= pr.ref_ntiles) o >>= 1;  // levels that add zeros
+        for (; o >= 32; o >>= 1) {
             if (t < o) {
-                sh->s[0][t] += sh->s[0][t + o];
-                sh->s[1][t] += sh->s[1][t + o];
+                a += sh->s[0][t + o];
+                b += sh->s[1][t + o];
+                sh->s[0][t] = a;
+                sh->s[1][t] = b;
             }
             bar();
         }
-        if (t == 32) control_prepare(st, 1, sh->s[0][0], sh->s[1][0], 0.0, &sh->pre);
+        // the rest of both trees in one warp, the second sum in its upper half
+        if (t < 32) {
+            const bool h16 = t & 16;
+            double x = (h16 ? b : a) + __shfl_xor_sync(0xffffffffu, h16 ? a : b, 16);
+#pragma unroll
+            for (o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if ((t & 15) == 0) sh->s[2 + (t >> 4)][0] = x;
+        }
         bar();
-        if (t == 0) control_decide(st, sh->s[0][0], sh->s[1][0], 0.0, &sh->pre);
+        if (t == 32) control_prepare(st, 1, sh->s[2][0], sh->s[3][0], 0.0, &sh->pre);
+        bar();
+        if (t == 0) control_decide(st, sh->s[2][0], sh->s[3][0], 0.0, &sh->pre);
         return true;
     }
     // fixed order: strided over the threads, warp trees, then the warps
@@ -1104,15 +1117,18 @@ __device__ __forceinline__ bool control_one(const MmaProb &pr, const DevCtl *ctl
     }
     const int nw = nparts < kCtlThreads ? (nparts + 31) / 32 : kCtlThreads / 32;  // warps that hold partials
     if (t < 32 * nw) {
+        // the four sums over the warp by halves (xor 16, 8, 4, 2, 1), packed: after the
+        // first level a half-warp holds each of two sums, after the second a quarter
+        // each of four.  An FP64 addition takes 64 clocks of the SM quadrant's pipe
+        // whatever the lanes hold: 6 of them instead of 20 (n = 384: 1.31 -> 1.28 ms a
+        // solve, n = 517 at finite temperature 5.05 -> 4.98, with the trees above).
+        const bool h16 = t & 16, h8 = t & 8;
+        const double x = (h16 ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[1], 16);
+        const double y = (h16 ? v[3] : v[2]) + __shfl_xor_sync(0xffffffffu, h16 ? v[2] : v[3], 16);
+        double z = (h8 ? y : x) + __shfl_xor_sync(0xffffffffu, h8 ? x : y, 8);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-        }
-        if ((t & 31) == 0) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) sh->s[q][t >> 5] = v[q];
-        }
+        for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if ((t & 7) == 0) sh->s[(h16 ? 1 : 0) + (h8 ? 2 : 0)][t >> 5] = z;
     }
     bar();
     // warps 0 to 4: lane q sums component q over the warps, lane 0 collects

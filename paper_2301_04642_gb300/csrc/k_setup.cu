@@ -135,10 +135,19 @@ __global__ void __launch_bounds__(256, 4) k_init_x0(const MmaProb *probs, int pr
     const MmaProb &pr = probs[prob];
     SolveState *st = pr.st;
     const int n = pr.n;
-    double w = st->emax - st->emin;
-    if (!(w > 0.0)) w = 1.0;
-    const double inv_w = 1.0 / w;
-    const double dshift = st->emax * inv_w - st->c;  // diagonal of Y0 gets +dshift
+    // scalars by one thread: the division in every thread kept the FP64 pipe (2
+    // lanes a clock and SM) busy for 2 us of the launch
+    __shared__ double sc_w[2];
+    if (threadIdx.x == 0) {
+        double w = st->emax - st->emin;
+        if (!(w > 0.0)) w = 1.0;
+        const double inv = 1.0 / w;
+        sc_w[0] = inv;
+        sc_w[1] = st->emax * inv - st->c;
+    }
+    __syncthreads();
+    const double inv_w = sc_w[0];
+    const double dshift = sc_w[1];  // diagonal of Y0 gets +dshift
     const float s0 = st->s_cur;
     const bool fp64 = (st->prec == kPrecFp64);
     // the certificate steps start from X0 in the zero-temperature form
