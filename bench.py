@@ -595,7 +595,7 @@ def main():
 
 def profile_solve(args, torch, fe, wl):
     """One solve of the workload (or of its recipe at --n) with the step loop
-    as plain launches (per-launch CUDA events), fixed 128 x 256 tiles unless
+    as plain launches (per-launch CUDA events), tiles up to 256 columns unless
     --tiles says otherwise; prints the per-kernel times.  In a k_sym_mma
     launch list the first three launches are the bound certificate."""
     # the workload's spectrum recipe at --n (or the workload's own n), Q from

@@ -154,10 +154,10 @@ typedef uint64_t fe_ticket;
 /* One tile-shape table entry as fe_autotune reports it. */
 typedef struct {
     int64_t n;       /* problem dimension                                          */
-    int bn;          /* tensor-core tile width chosen: 256 (128 x 256 tiles) or 128 */
+    int bn;          /* largest tensor-core tile width chosen: 256 or 128            */
     double ms_256;   /* best device time (ms) per solve of a synthetic batch of this
-                        size with 128 x 256 tiles                                  */
-    double ms_128;   /* the same with 128 x 128 tiles                               */
+                        size with tiles up to 256 columns wide                    */
+    double ms_128;   /* the same with tiles up to 128 columns wide                  */
 } fe_tune;
 
 /* Create a context on cfg->device.  cfg may be NULL (defaults).
@@ -212,7 +212,7 @@ FE_API int fe_poll(fe_ctx *ctx, fe_ticket t, fe_result *r);
  * fe_autotune fills the table for the panel counts of ns[0..count): for each
  * it times `reps` batches of synthetic gapped solves of that size (N_e =
  * 0.85 n, device Hp, no output; enough copies per batch, at most 16, for two
- * waves of 128 x 256 tiles over the SMs, so that the time per solve measures
+ * waves of 128 x 256 blocks over the SMs, so that the time per solve measures
  * throughput as in a busy batch or server) with each width under precision
  * policy `prec` (0 = the context's default; FE_PREC_FP64 has no tiles), keeps
  * the width with the lower time per solve, and writes the table to the
@@ -226,13 +226,13 @@ FE_API int fe_autotune(fe_ctx *ctx, int count, const int64_t *ns, uint32_t prec,
  * (copies of one problem); in a mixed batch the widths interact (one launch
  * holds every problem's tiles), so this tunes on the batch itself: it times
  * fe_solve_batch on ps[0..count) (outputs not written: every D is ignored)
- * with 128 x 256 tiles for every problem, then makes the problems of the
- * smallest panel count narrow (128 x 128), then those of the next one, and so
+ * with up to 256 columns for every problem, then makes the problems of the
+ * smallest panel count narrow (128), then those of the next one, and so
  * on while each step lowers the batch's device time by more than 0.5%; the
  * first step that does not is undone and ends the search.  The result is left
  * in the context's table (and its autotune_path file).  Each trial is one
  * untimed batch then the best of `reps` (< 1: 2).  trial_ms[0..max_trials)
- * receives the trials' batch times (ms; [0] = all 128 x 256), *ntrials their
+ * receives the trials' batch times (ms; [0] = 256 for all), *ntrials their
  * number (both may be NULL / 0).
  * Errors: FE_EINVAL (count < 1, an invalid problem), any fe_solve_batch
  * status (the table is then left as it was). */

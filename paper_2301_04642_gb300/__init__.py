@@ -354,8 +354,8 @@ class Context:
 
     # ---- tile-shape autotuner ---------------------------------------------------
     def autotune(self, ns, precision="mixed", reps=2):
-        """Time synthetic solves of each size in `ns` with 128 x 256 and
-        128 x 128 tensor-core tiles and keep the faster width per size
+        """Time synthetic solves of each size in `ns` with tensor-core tiles up
+        to 256 and up to 128 columns wide and keep the faster width per size
         (fe_autotune); returns one dict per size."""
         ns = [int(x) for x in ns]
         arr = (ctypes.c_int64 * max(1, len(ns)))(*ns)
@@ -368,7 +368,7 @@ class Context:
     def autotune_batch(self, items, reps=2, max_trials=64):
         """Tune the tile widths on a batch (fe_autotune_batch; items as for
         solve_batch, outputs not written).  Returns the trials' batch times
-        (ms; the first with 128 x 256 tiles everywhere)."""
+        (ms; the first with tiles up to 256 columns everywhere)."""
         probs = (FeProblem * len(items))()
         keep = []
         for k, it in enumerate(items):
