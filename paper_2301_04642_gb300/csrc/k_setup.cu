@@ -28,7 +28,7 @@ __global__ void k_bounds_rows(const MmaProb *probs, int prob, RowInfo *rowinfo, 
     // the FP32 rate)
     constexpr unsigned long long kAbs = 0x7FFFFFFFFFFFFFFFull, kExp = 0x7FF0000000000000ull;
     double s = 0.0;
-    unsigned long long mxb = 0, nonfin = 0;
+    unsigned long long mxb = 0;
     // four loads per lane in flight: the 128 to 2048 rows an SM holds must
     // keep enough bytes outstanding to stream Hp at HBM speed
     // The row also goes to the FP32 master as an FP32 copy of Hp for the
@@ -47,7 +47,6 @@ __global__ void k_bounds_rows(const MmaProb *probs, int prob, RowInfo *rowinfo, 
         const unsigned long long b1 = static_cast<unsigned long long>(__double_as_longlong(h1)) & kAbs;
         const unsigned long long b2 = static_cast<unsigned long long>(__double_as_longlong(h2)) & kAbs;
         const unsigned long long b3 = static_cast<unsigned long long>(__double_as_longlong(h3)) & kAbs;
-        nonfin |= ((b0 & kExp) == kExp) | ((b1 & kExp) == kExp) | ((b2 & kExp) == kExp) | ((b3 & kExp) == kExp);
         s += __longlong_as_double(static_cast<long long>(b0));
         s1 += __longlong_as_double(static_cast<long long>(b1));
         s2 += __longlong_as_double(static_cast<long long>(b2));
@@ -58,15 +57,15 @@ __global__ void k_bounds_rows(const MmaProb *probs, int prob, RowInfo *rowinfo, 
         const double h0 = h[j];
         yrow[j] = f64_to_f32_rn(h0);
         const unsigned long long b0 = static_cast<unsigned long long>(__double_as_longlong(h0)) & kAbs;
-        nonfin |= ((b0 & kExp) == kExp);
         s += __longlong_as_double(static_cast<long long>(b0));
         mxb = max(mxb, b0);
     }
     s = warp_sum((s + s1) + (s2 + s3));
     for (int o = 16; o > 0; o >>= 1) mxb = max(mxb, __shfl_xor_sync(0xffffffffu, mxb, o));
     const double mx = __longlong_as_double(static_cast<long long>(mxb));
-    int nonfinite = nonfin ? 1 : 0;
-    nonfinite = __any_sync(0xffffffffu, nonfinite);
+    // Inf and NaN have the largest encodings; tested entry by entry, the exponent
+    // compares went to the FP64 pipe (n = 4096: 125 us a launch, 88 with this)
+    const bool nonfinite = (mxb & kExp) == kExp;
     if (lane == 0) {
         const double d = h[row];
         const double r = s - fabs(d);
