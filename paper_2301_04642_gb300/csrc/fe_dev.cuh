@@ -231,19 +231,17 @@ struct SolveState {
 // small fraction of its FP32 rate, enough to make an HBM-bound pass over FP64
 // data arithmetic bound.  Values below FP32's normal range become 0, values
 // above it infinity (callers pass finite data of moderate range).
-// f64_to_f32_scaled: of x 2^e, the exponent moved before the conversion.  Free of
-// branches: the dropped 29 bits round by an addition that carries into the result.
-__device__ __forceinline__ float f64_to_f32_scaled(double x, int e) {
+// Free of branches: the dropped 29 bits round by an addition that carries into the result.
+__device__ __forceinline__ float f64_to_f32_rn(double x) {
     const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
     const int ex = static_cast<int>((hi >> 20) & 0x7FFu);
-    const int fe = ex - 896 + e;  // FP32 exponent field
+    const int fe = ex - 896;  // FP32 exponent field
     unsigned r = (__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | (static_cast<unsigned>(fe) << 23);
     r += ((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (r & 1u)) >> 29;  // a carry may raise the exponent
     r = (ex == 0 || fe <= 0) ? 0u : r;
     r = (ex == 0x7FF || fe >= 255) ? 0x7F800000u : r;
     return __uint_as_float(r | (hi & 0x80000000u));
 }
-__device__ __forceinline__ float f64_to_f32_rn(double x) { return f64_to_f32_scaled(x, 0); }
 
 // Exact FP32 -> FP64 conversion by integer operations on the encodings: the
 // conversion instruction runs on the FP64 pipe, which GB300 executes at 1/64
