@@ -13,13 +13,19 @@ __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, S
         return kind == kTcSingle || kind == kTcSplit || kind == kTcElem || kind == kTcDelta;
     };
     // after a k_sym_mma that controlled its own products, only the steps of the
-    // other families (their kernels ran behind it) have been taken
-    const bool ran = flags && *reinterpret_cast<const volatile unsigned *>(&flags->controlled) != 0 &&
-                     *reinterpret_cast<const volatile int *>(&ctl->err) == 0;
-    const bool hold = ran && *reinterpret_cast<const volatile int *>(&ctl->hold) != 0;
+    // other families (their kernels ran behind it) have been taken.  One thread
+    // decides for the block: the block that finishes last clears both words, and a
+    // late warp of a block with nothing to do would read them cleared.
+    __shared__ int sh_step;
+    if (threadIdx.x == 0) {
+        const bool ran = flags && *reinterpret_cast<const volatile unsigned *>(&flags->controlled) != 0 &&
+                         *reinterpret_cast<const volatile int *>(&ctl->err) == 0;
+        const bool hold = ran && *reinterpret_cast<const volatile int *>(&ctl->hold) != 0;
+        sh_step = p < nprobs && !hold && !(ran && tc_pending(probs[p].st));
+    }
+    __syncthreads();
     bool stepped = false;
-    if (p < nprobs && !hold && !(ran && tc_pending(probs[p].st)))
-        stepped = control_one(probs[p], ctl, &sh, threadIdx.x, [] { __syncthreads(); });
+    if (sh_step) stepped = control_one(probs[p], ctl, &sh, threadIdx.x, [] { __syncthreads(); });
     if (!flags || threadIdx.x != 0) return;
     // Inside the step graph: collect what the next pass needs over all problems;
     // the block that finishes last sets the graph's conditions (loop on while any

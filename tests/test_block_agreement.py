@@ -1,0 +1,76 @@
+"""Threads of a block must agree before they meet at a barrier, and see what
+another thread wrote only after one.  Device code runs here on the host, thread by thread, in
+the order that shows a disagreement."""
+import os
+import re
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2301_04642_gb300", "csrc")
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+pytestmark = pytest.mark.skipif(
+    not (shutil.which("g++") and os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h"))),
+    reason="needs g++ and the CUDA headers")
+
+
+def _host(name):
+    """A source file with its inline PTX taken out."""
+    s = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"\basm volatile\(.*?\);", ";", s, flags=re.S)
+
+
+def _run(tmp_path, main, files=(), snippet=""):
+    for f in ("fe_dev.cuh", "fe_kernels.cuh") + tuple(files):
+        (tmp_path / f).write_text(_host(f))
+    (tmp_path / "main.cpp").write_text('#include "cuda_emu.h"\n' + snippet + main)
+    exe = str(tmp_path / "main")
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-I", str(tmp_path), "-I", os.path.join(ROOT, "tests", "emu"),
+                        "-I", os.path.join(ROOT, "include"), "-I", os.path.join(CUDA, "include"),
+                        str(tmp_path / "main.cpp"), "-o", exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+SETUP = r"""
+#include "k_control.cuh"
+#include "k_control.cu"
+static std::vector<int> reversed_warps(int n) {  // warp by warp, a warp's last lane first
+    std::vector<int> o;
+    for (int w = 0; w < n; w += 32)
+        for (int t = w + 31; t >= w; --t) o.push_back(t);
+    return o;
+}
+"""
+
+CONTROL_KERNEL = SETUP + r"""
+int main() {
+    static fe::SolveState st, before;
+    static double part[4 * 608];
+    fe::MmaProb pr;
+    memset(&pr, 0, sizeof pr);
+    pr.st = &st;
+    pr.part = part;
+    pr.ntiles = 2;
+    st.kind = fe::kTcSplit;  // a product that is still to run: k_control passes
+    before = st;
+    fe::StepFlags fl{};
+    fl.controlled = 1;
+    fe::DevCtl ctl{};
+    gridDim.x = 1;
+    const int stuck = emu::run(256, reversed_warps(256),
+                               [&](int) { fe::k_control(&pr, 1, &ctl, &fl, 0, 0, 1); });
+    const int changed = memcmp(&st, &before, sizeof st) != 0;
+    printf("stuck %d, state changed %d, steps %u, controls %u\n", stuck, changed, fl.n_steps, fl.n_ctl);
+    return stuck || changed || fl.n_steps != 0 || fl.n_ctl != 1 || fl.controlled != 0;
+}
+"""
+
+
+def test_control_kernel_takes_one_decision_per_block(tmp_path):
+    """k_control clears the flags it acts on; a late warp must not act on the cleared ones."""
+    _run(tmp_path, CONTROL_KERNEL, files=("k_control.cuh", "k_control.cu"))
