@@ -1031,6 +1031,7 @@ constexpr int kCtlThreads = 256;
 struct ControlSmem {
     double s[4][kCtlThreads];
     Prep pre;
+    int verdict;  // 0: the problem is done, 1: end it (a bounded wait ran out), 2: take the step
 };
 
 // Control step of one problem by kCtlThreads threads (t: 0 .. kCtlThreads - 1;
@@ -1048,8 +1049,20 @@ __device__ __forceinline__ bool control_one(const MmaProb &pr, const DevCtl *ctl
         int x;
         asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(reinterpret_cast<const char *>(st) + 128 * t) : "memory");
     }
-    if (*reinterpret_cast<const volatile int *>(&st->done)) return false;
-    if (ctl && *reinterpret_cast<const volatile int *>(&ctl->err) != 0) {
+    // number of partial slots written by the previous producer
+    const int kind = *reinterpret_cast<const volatile int *>(&st->kind);
+    // One thread decides whether there is a step to take: inside k_sym_mma another
+    // CTA's wait may run out between two threads' reads of the error word, and
+    // threads that disagreed would meet at different barriers.
+    if (t == 0) {
+        const bool done = *reinterpret_cast<const volatile int *>(&st->done) != 0;
+        const bool err = ctl && *reinterpret_cast<const volatile int *>(&ctl->err) != 0;
+        sh->verdict = done ? 0 : err ? 1 : 2;
+    }
+    bar();
+    const int verdict = sh->verdict;
+    if (verdict == 0) return false;
+    if (verdict == 1) {
         // a kernel of this run gave up a bounded wait: its outputs are not
         // trustworthy, so the expansion stops here
         if (t == 0) {
@@ -1060,8 +1073,6 @@ __device__ __forceinline__ bool control_one(const MmaProb &pr, const DevCtl *ctl
         return true;
     }
 
-    // number of partial slots written by the previous producer
-    const int kind = *reinterpret_cast<const volatile int *>(&st->kind);
     int nparts;
     if (kind == kNone) nparts = kInitBlocks;
     else if (kind == kFp64) nparts = pr.ntilesF;

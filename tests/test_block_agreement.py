@@ -74,3 +74,39 @@ int main() {
 def test_control_kernel_takes_one_decision_per_block(tmp_path):
     """k_control clears the flags it acts on; a late warp must not act on the cleared ones."""
     _run(tmp_path, CONTROL_KERNEL, files=("k_control.cuh", "k_control.cu"))
+
+
+CONTROL_STEP = SETUP + r"""
+int main(int argc, char **argv) {
+    int bad = 0;
+    // a bounded wait of another block runs out after the k-th thread had its turn
+    for (int k : {0, 31, 127, 254}) {
+        static fe::SolveState st;
+        static double part[4 * 608];
+        memset(&st, 0, sizeof st);
+        fe::MmaProb pr;
+        memset(&pr, 0, sizeof pr);
+        pr.st = &st;
+        pr.part = part;
+        st.n = 2;
+        st.bad_input = 1;  // ends the problem with FE_EINVAL when the step is taken
+        fe::DevCtl ctl{};
+        fe::ControlSmem sh;
+        int taken = 0;
+        std::vector<int> order;
+        for (int t = 0; t < 256; ++t) order.push_back(t);
+        const int stuck = emu::run(256, order,
+                                   [&](int t) { taken += fe::control_one(pr, &ctl, &sh, t, [] { emu::meet(0); }); },
+                                   [&](int done) { if (done == k) ctl.err = fe::kErrTimeoutGrid; });
+        printf("after thread %d: stuck %d, taken by %d, status %d\n", k, stuck, taken, st.status);
+        bad += stuck || taken != 256 || !st.done || (st.status != -1 && st.status != -4);
+    }
+    return bad;
+}
+"""
+
+
+def test_control_step_takes_one_decision_per_block(tmp_path):
+    """control_one inside a launch whose other blocks still run: an error recorded
+    between two threads' reads must not leave some of them at a barrier."""
+    _run(tmp_path, CONTROL_STEP, files=("k_control.cuh", "k_control.cu"))
