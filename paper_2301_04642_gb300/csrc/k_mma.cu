@@ -122,6 +122,7 @@ struct OpCache {
     OutCache out[3];
 };
 
+// Copies what the store phase needs of the step's operands; whole warp.
 __device__ __forceinline__ void load_op(OpCache &oc, const MmaProb &pr, const ProdOp &op, int lane) {
     if (lane < 3) {
         const OutSpec &o = op.out[lane];
@@ -174,6 +175,9 @@ __device__ __forceinline__ void load_op(OpCache &oc, const MmaProb &pr, const Pr
         oc.rsum = op.ref_sums ? pr.rsum : nullptr;
         oc.ldr = pr.ldr;
     }
+    // every lane reads the copy, and an epilogue-only step has no chunk loop whose
+    // barriers would stand between
+    __syncwarp();
 }
 
 // FP64 partials of a tile, one thread's share.

@@ -36,6 +36,41 @@ def _run(tmp_path, main, files=(), snippet=""):
     assert r.returncode == 0, r.stdout + r.stderr
 
 
+LOAD_OP = r"""
+int main() {
+    fe::MmaProb pr;
+    memset(&pr, 0, sizeof pr);
+    pr.mats[2].master = reinterpret_cast<float *>(64);
+    fe::ProdOp op;
+    memset(&op, 0, sizeof op);
+    op.nout = 2;
+    op.part_out = 1;
+    op.E1 = op.E2 = -1;
+    op.inv = 0.5f;
+    for (int o = 0; o < 3; ++o) op.out[o].a = 1.0f + o, op.out[o].mat = 2, op.out[o].flags = 3;
+    fe::OpCache oc;
+    memset(&oc, 0xee, sizeof oc);
+    std::vector<int> order;
+    for (int t = 31; t >= 0; --t) order.push_back(t);  // the lanes that write come last
+    int bad = 0;
+    const int stuck = emu::run(32, order, [&](int lane) {
+        fe::load_op(oc, pr, op, lane);
+        bad += !(oc.nout == 2 && oc.pout == 1 && oc.inv == 0.5f && oc.E2 == nullptr && oc.out[0].a == 1.0f &&
+                 oc.out[1].a == 2.0f && oc.out[1].master == pr.mats[2].master);
+    });
+    printf("stuck %d, lanes with stale operands %d\n", stuck, bad);
+    return stuck || bad;
+}
+"""
+
+
+def test_operand_copy_is_seen_by_every_lane(tmp_path):
+    """load_op: four lanes write the warp's copy of the step's operands, all read it."""
+    s = _host("k_mma.cu")
+    part = s[s.index("struct OutCache {"):s.index("// FP64 partials of a tile")]
+    _run(tmp_path, LOAD_OP, snippet='#include "fe_dev.cuh"\n#include "fe_kernels.cuh"\nnamespace fe {\n' + part + "}\n")
+
+
 SETUP = r"""
 #include "k_control.cuh"
 #include "k_control.cu"
