@@ -68,6 +68,7 @@ struct Slot {
     double *Dtmp = nullptr;
     float *lzv = nullptr;   // Lanczos vectors (6 n FP32)
     double *part = nullptr;
+    size_t nparts = 0;
     SolveState *st = nullptr;
     RowInfo *rowinfo = nullptr;
     int *bad = nullptr;
@@ -302,11 +303,10 @@ size_t slot_bytes(int n, int method, int *ldy, int *lds, int *ldx, size_t *npart
     *ldx = n;
     const int T = ceil_div(n, kTileM);
     const size_t ntiles = 2 * static_cast<size_t>(num_tiles_tc(n, 32));  // the narrowest width has most
-    const size_t ntF = method == kMethodSp2 ? static_cast<size_t>(num_tiles_f64(n)) : 0;
     const size_t TD = static_cast<size_t>(ceil_div(n, kDigitN));
     size_t ntD = 0;
     for (size_t I = 0; I < static_cast<size_t>(T); ++I) ntD += (TD > 2 * I) ? TD - 2 * I : 0;
-    *nparts = std::max<size_t>({static_cast<size_t>(kInitBlocks), ntiles, ntF, ntD,
+    *nparts = std::max<size_t>({static_cast<size_t>(kInitBlocks), ntiles, ntD,
                                 static_cast<size_t>(kFinBlocks)});
     const size_t nn = static_cast<size_t>(n);
     size_t b = 0;
@@ -320,10 +320,7 @@ size_t slot_bytes(int n, int method, int *ldy, int *lds, int *ldx, size_t *npart
     add(8 * 3 * nn);                                 // Lanczos vectors
     if (method == kMethodSp2)
         for (int a = 0; a < kDigits; ++a) add(2 * nn * (*lds));  // digits of X/4
-    if (method == kMethodFermi) {
-        add(12 * kNumMats * align_up(nn, 8));             // FP64 diagonals + FP32 copies
-        add(4 * ((nn + 7) / 8) * align_up(nn, 32));       // 8-column sums (MmaProb::rsum)
-    }
+    if (method == kMethodFermi) add(12 * kNumMats * align_up(nn, 8));  // FP64 diagonals + FP32 copies
     add(8 * kPartStride * (*nparts));                // partials
     add(sizeof(SolveState));
     add(sizeof(RowInfo) * nn);
@@ -441,8 +438,10 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
         for (int a = 0; a < kDigits; ++a) digs[a] = reinterpret_cast<__half *>(take(2 * nn * lds));
     const size_t dstride = align_up(nn, 8);  // 64-byte aligned vectors
     double *diags = (method == kMethodFermi) ? reinterpret_cast<double *>(take(12 * kNumMats * dstride)) : nullptr;
+    // the 8-column sums of a step (n/8 x ldr FP32) lie in Dtmp, which only the output needs
     const size_t ldr = align_up(nn, 32);
-    float *rsum = (method == kMethodFermi) ? reinterpret_cast<float *>(take(4 * ((nn + 7) / 8) * ldr)) : nullptr;
+    float *rsum = (method == kMethodFermi) ? reinterpret_cast<float *>(s->Dtmp) : nullptr;
+    s->nparts = nparts;
     s->part = reinterpret_cast<double *>(take(8 * kPartStride * nparts));
     s->st = reinterpret_cast<SolveState *>(take(sizeof(SolveState)));
     s->rowinfo = reinterpret_cast<RowInfo *>(take(sizeof(RowInfo) * nn));
@@ -847,6 +846,10 @@ int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
         if (pr == FE_PREC_FP64 && !fermi && !trfoe) {
             e.any_fp64 = true;
             build_tiles_f64(j.slot);
+            // a partial per 16 x 16 tile: where they outnumber the slot's, they take
+            // the first digit array (n x lds FP16), which this schedule leaves unused
+            if (j.slot->tilesF.size() > j.slot->nparts)
+                hprobs[k].part = reinterpret_cast<double *>(hprobs[k].dig[0]);
             for (TileF64 t : j.slot->tilesF) { t.prob = k; tilesF.push_back(t); }
             e.cntF[k] = static_cast<int>(j.slot->tilesF.size());
         }
