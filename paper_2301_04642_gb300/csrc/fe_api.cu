@@ -2103,12 +2103,14 @@ int gemm_workspace(fe_ctx *ctx, size_t bytes) {
 
 // Tile width of a product with K parts of `chunks` 64-wide chunks: the one whose
 // rounds of tiles over the CTA pairs take least, by the cost of a tile as in
-// choose_widths (count(bn): work units at that width).
-template <class Count>
-int gemm_width(fe_ctx *ctx, int chunks, Count count) {
-    int best = kWidths[0];
+// choose_widths (count(bn): work units at that width), among those whose workspace
+// (bytes(bn): narrow tiles leave less of it beyond the matrix edge) the budget holds.
+template <class Count, class Bytes>
+int gemm_width(fe_ctx *ctx, int chunks, Count count, Bytes bytes) {
+    int best = kWidths[3];
     double best_cost = DBL_MAX;
     for (int bn : kWidths) {
+        if (bytes(bn) > ctx->budget) continue;
         const double t = chunks * std::max(kCostChunkMin + kCostChunkCol * bn, kCostChunkMma * bn) + kCostTile +
                          kCostGemmStore * bn;
         const double cost = std::ceil(static_cast<double>(count(bn)) / (0.5 * ctx->sym_grid)) * t;
@@ -2158,12 +2160,14 @@ extern "C" int fe_project(fe_ctx *ctx, const double *Psi, const double *HPsi, in
     S = std::max(1, std::min(S, std::max(1, nk / 8)));
     const int cs = (nk + S - 1) / S;
     S = (nk + cs - 1) / cs;  // every part non-empty
-    const int bn = gemm_width(ctx, cs, [&](int w) { return num_tiles_tc(n, w) * S; });
-    const int ntiles = static_cast<int>(num_tiles_tc(n, bn));
     const size_t slice = 2 * static_cast<size_t>(n) * static_cast<size_t>(lds);
-    const size_t tsz = 2 * static_cast<size_t>(kTileM) * bn * sizeof(float);
-    const size_t o_ws = align_up(4 * slice, 1024), bytes = o_ws + static_cast<size_t>(ntiles) * S * tsz;
-    int rc = gemm_workspace(ctx, bytes);
+    const size_t o_ws = align_up(4 * slice, 1024);
+    auto bytes = [&](int w) {
+        return o_ws + static_cast<size_t>(num_tiles_tc(n, w)) * S * 2 * static_cast<size_t>(kTileM) * w * sizeof(float);
+    };
+    const int bn = gemm_width(ctx, cs, [&](int w) { return num_tiles_tc(n, w) * S; }, bytes);
+    const int ntiles = static_cast<int>(num_tiles_tc(n, bn));
+    int rc = gemm_workspace(ctx, bytes(bn));
     if (rc != FE_OK) return rc;
     __half *sl[4];
     for (int k = 0; k < 4; ++k) sl[k] = reinterpret_cast<__half *>(ctx->gws + k * slice);
@@ -2204,7 +2208,8 @@ extern "C" int fe_rotate(fe_ctx *ctx, const double *Psi, int64_t m, int64_t n, i
     const int64_t lds = static_cast<int64_t>(align_up(static_cast<size_t>(n), 8));  // K = n
     const int P = static_cast<int>((m + 255) / 256);
     const int nk = static_cast<int>(blocks64(n));
-    const int bn = gemm_width(ctx, nk, [&](int w) { return static_cast<int64_t>(P) * ((n + w - 1) / w); });
+    const int bn = gemm_width(ctx, nk, [&](int w) { return static_cast<int64_t>(P) * ((n + w - 1) / w); },
+                              [](int) { return static_cast<size_t>(0); });
     const int CJ = static_cast<int>((n + bn - 1) / bn);
     const size_t oa = align_up(2 * static_cast<size_t>(m) * static_cast<size_t>(lds), 1024);
     const size_t ob = align_up(2 * static_cast<size_t>(n) * static_cast<size_t>(lds), 1024);

@@ -1,5 +1,6 @@
 """The memory a call needs: a slot is its matrices, the vectors and one record per
-tile, so a context whose budget holds these solves the problem.
+tile, so a context whose budget holds these solves the problem; a projection needs
+the slices of both operands and the partial sums.
 
 The sizes are the sum over the buffers, each rounded up to 1 KiB: Hp and D copies,
 the two FP64 buffers, FP32 masters, FP16 slices (two per matrix), then the digit
@@ -58,3 +59,28 @@ def test_fp64_schedule_equals_the_oracle_with_more_tiles_than_records():
                 ref = oracle.density(p.H, float(ne))
                 # as for the smaller sizes: 30 products leave 30 n 2^-53 / gap in x, and the stop's 2e-10
                 assert np.linalg.norm(D - ref["D"]) <= 1e-8
+
+
+@pytest.mark.parametrize("m,n", [(4652, 523), (20440, 267), (5843, 521)])
+def test_projection_in_a_budget_of_slices_and_sums(m, n):
+    """Slices (8 n m) and partial sums of 128 x 192 blocks over the upper triangle; with
+    less than its preferred tiles need, the projection takes narrower ones, and the
+    result is the same."""
+    need_gpu()
+    import paper_2301_04642_gb300 as fe
+    nk, ti, tj = -(-m // 64), -(-n // 128), -(-n // 192)
+    blocks = sum(min(ti, (192 * j + 191) // 128 + 1) for j in range(tj))
+    S = max(1, min(max(-(-nk // 128), -(-912 // blocks)), nk // 8))
+    S = -(-nk // -(-nk // S))
+    lds = -(-m // 8) * 8
+    budget = -(-8 * n * lds // 1024) * 1024 + blocks * S * 4 * 128 * 192
+    g = torch.Generator(device="cuda").manual_seed(m)
+    P, Y = [torch.randn(m, n, generator=g, device="cuda", dtype=torch.float64) for _ in range(2)]
+    H = [torch.empty(n, n, device="cuda", dtype=torch.float64) for _ in range(2)]
+    for out, b in zip(H, (0, budget)):
+        with fe.Context(device=0, hbm_budget_bytes=b) as c:
+            c.project(P, Y, out)
+    assert torch.equal(H[0], H[1])
+    with fe.Context(device=0, hbm_budget_bytes=8 * n * lds) as c, pytest.raises(fe.FeError) as ei:
+        c.project(P, Y, H[0])
+    assert ei.value.status == fe.FE_ENOMEM
