@@ -145,3 +145,37 @@ def test_control_step_takes_one_decision_per_block(tmp_path):
     """control_one inside a launch whose other blocks still run: an error recorded
     between two threads' reads must not leave some of them at a barrier."""
     _run(tmp_path, CONTROL_STEP, files=("k_control.cuh", "k_control.cu"))
+
+
+COEFFICIENTS = SETUP + r"""
+int main() {
+    const double in = 1.0, tiny = 0x1p-126;
+    std::vector<double> xs = {0.0, -0.0, in, -in, 0x1.0000010000000p0, 0x1.0000030000000p0, 0x1.fffffeffffffep0,
+                              tiny, 0.75 * tiny, -tiny / 1024, 0x1p-149, 0x1p-150, 0x1.8p-150, 0x1p-151, 0x1p-1074,
+                              0x1.fffffefffffffp127, 0x1.ffffffp127, -0x1p128, 0x1p1023, INFINITY, -INFINITY, NAN};
+    for (int e = -152; e < 129; ++e) xs.push_back(std::ldexp(1.2345678901234567, e)), xs.push_back(-std::ldexp(1.9999999, e));
+    int bad = 0;
+    auto same = [&](float got, double x, const char *what) {
+        const float want = static_cast<float>(x);
+        if (std::isnan(want) ? std::isnan(got) : memcmp(&got, &want, 4) == 0) return;
+        printf("%s %a: %a, not %a\n", what, x, got, want);
+        ++bad;
+    };
+    for (double x : xs) {
+        fe::OutSpec o;
+        fe::set_out(o, 0, 0, x, x, x, 0.0, 1.0);
+        same(o.a, x, "a"), same(o.b1, x, "b1"), same(o.b2, x, "b2");
+        fe::out_d(o, 0, 0, x, 1.0);
+        same(o.a, x, "diagonal a");
+        fe::set_e(o, 0, x, x, x, 0, x, x, x);
+        same(o.b1, x, "e b1"), same(o.g1r, x, "g1r"), same(o.g1c, x, "g1c");
+        same(o.b2, x, "e b2"), same(o.g2r, x, "g2r"), same(o.g2c, x, "g2c");
+    }
+    return bad != 0;
+}
+"""
+
+
+def test_coefficients_are_the_nearest_fp32(tmp_path):
+    """The control step's coefficients over all of FP32: subnormals, overflow, NaN."""
+    _run(tmp_path, COEFFICIENTS, files=("k_control.cuh", "k_control.cu"))
