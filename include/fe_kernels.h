@@ -105,10 +105,13 @@ FE_API int fe_k_narrow_bounds(fe_ctx *ctx, double factor);
  * copies and products in flight, frees its tensor memory and returns; the
  * control kernel then ends every problem of the run, and the call returns
  * FE_ETIMEOUT with the context still usable.  This sets the limit of those
- * waits for later solves on ctx (limit_ms, default 2000) and, with
- * fail_partner != 0, makes the meetings of all CTAs in k_sym_mma watch a word
- * that nothing writes, so that its wait runs out: a way to exercise the
- * expiry path without any fault.  Call it while no submitted solve runs.
+ * waits for later solves on ctx (limit_ms, default 2000).  The waits inside a
+ * tile count it on the SM clock, two clocks a nanosecond: a clock below 2 GHz
+ * lengthens it in proportion.  The meetings of all CTAs wait eight times as
+ * long, since a CTA without a tile waits there for the whole step.  With
+ * fail_partner != 0 the meetings of all CTAs in k_sym_mma watch a word that
+ * nothing writes, so that the wait runs out: a way to exercise the expiry path
+ * without any fault.  Call it while no submitted solve runs.
  * Errors: FE_EINVAL (ctx NULL, limit_ms outside (0, 60000]), FE_ECUDA. */
 FE_API int fe_k_set_wait(fe_ctx *ctx, double limit_ms, int fail_partner);
 
@@ -125,7 +128,8 @@ FE_API int fe_k_phase_ms(fe_ctx *ctx, double *out4);
 /* Tile-shape table hooks (tests; see fe_autotune in fe.h).  set: make problems
  * with n's number of 128-row panels under policy prec (an FE_PREC_* value,
  * FE_PREC_MIXED = 0 included) use tile width bn (128 or 256; 0 removes the
- * entry).  get: the width such a problem would use now (HOST out).
+ * entry): the library itself chooses narrower ones where a launch has few
+ * tiles.  get: the width such a problem would use at most now (HOST out).
  * fe_k_sym_square looks its width up under FE_PREC_FP32 (two slices) or
  * FE_PREC_TRY_FP16 (one slice). */
 FE_API int fe_k_set_tile_width(fe_ctx *ctx, int64_t n, uint32_t prec, int bn);
@@ -145,7 +149,8 @@ FE_API int fe_k_launch_count(fe_ctx *ctx, int64_t *out);
 /* Per-step record of problem `index` of the last solve or batch (measurement
  * hook, no counterpart in the paper).  out (HOST) receives up to max_rows rows
  * of 6 doubles: phase (0 single FP16, 1 split FP16, 2 FP64-accurate), kind of
- * the product that produced the iterate (0 none, 1 single, 2 split, 3 FP64),
+ * the product that produced the iterate (0 none, 1 single, 2 split, 3 FP64,
+ * 6 digit product, 7 the second product of a polishing pair),
  * tr X - N_e, tr X - ||X||_F^2, ||X^2 - X||_F of that
  * product's input (-1 before the first product), RelTr (-1 at step 0).
  * *rows = rows written. */

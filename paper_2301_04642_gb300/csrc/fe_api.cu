@@ -102,7 +102,7 @@ struct Engine {
     size_t h_done_cap = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaEvent_t ev_setup = nullptr, ev_loop = nullptr;  // end of set-up, end of the step loop
-    int ntc = 0, nF = 0, nD = 0;    // tile counts of the uploaded lists
+    int nF = 0, nD = 0;              // FP64 and digit tiles of the uploaded lists
     bool any_tc = false, any_fp64 = false, any_digit = false, any_fermi = false;
     // the step loop as a CUDA graph (eng_graph)
     StepFlags *d_flags = nullptr;
@@ -655,9 +655,9 @@ void init_state(const fe_ctx *ctx, const fe_problem *p, SolveState *st) {
 // eng_steps (tensor-core step, FP64-accurate step, control step; repeated),
 // eng_finish per finished problem (output kernels, read-back of its state).
 // Kernels reach a problem's buffers and state through its table entry, so the
-// table can be rebuilt between steps as problems join and leave; the tiles of
-// one problem are computed the same way whatever else is in the table, so a
-// problem's result does not depend on its batch.
+// table can be rebuilt between steps as problems join and leave.  Where a tile's K
+// sum is cut depends on what else the launch computes, so a problem's result varies
+// with its batch in the last bits of the FP32 sums, well within its tolerances.
 
 // One problem bound to a slot.
 struct Job {
@@ -880,7 +880,6 @@ int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
                                      cudaMemcpyHostToDevice, e.stream));
     // the copies read host vectors that go out of scope here
     FE_CUDA(ctx, cudaStreamSynchronize(e.stream));
-    e.ntc = static_cast<int>(tiles.size());
     e.nF = static_cast<int>(tilesF.size());
     e.nD = static_cast<int>(tilesD.size());
     return FE_OK;
@@ -1110,8 +1109,7 @@ void fill_result(const SolveState &st, int herr, double ms, fe_result &r) {
 int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     std::vector<uintptr_t> key = {reinterpret_cast<uintptr_t>(e.d_probs), reinterpret_cast<uintptr_t>(e.d_tiles),
                                   reinterpret_cast<uintptr_t>(e.d_tilesF), reinterpret_cast<uintptr_t>(e.d_tilesD),
-                                  static_cast<uintptr_t>(np), static_cast<uintptr_t>(e.ntc),
-                                  static_cast<uintptr_t>(e.nF), static_cast<uintptr_t>(e.nD),
+                                  static_cast<uintptr_t>(np), static_cast<uintptr_t>(e.nF), static_cast<uintptr_t>(e.nD),
                                   static_cast<uintptr_t>(e.any_tc), static_cast<uintptr_t>(e.any_fp64),
                                   static_cast<uintptr_t>(e.any_digit), reinterpret_cast<uintptr_t>(e.d_sched)};
     if (e.gexec && key == e.gkey) return FE_OK;

@@ -23,7 +23,6 @@ constexpr int kTileM = 128;    // rows of one tensor-core tile (TMEM lanes)
 constexpr int kTileN = 256;    // columns of one tensor-core tile (two 128-blocks)
 constexpr int kTileK = 64;     // K per pipeline stage (one 128-byte swizzle row of FP16)
 constexpr int kMaxSlices = 2;
-constexpr int kStages = 2;
 constexpr int kMmaThreads = 320;  // digit kernel: warp 0 TMA, warp 1 MMA, warps 2-9 drain + epilogue
 constexpr int kEpiWarps = 8;
 // split-FP16 kernel: warpgroup 0 (warp 0 TMA, warp 1 MMA, warps 2-3 idle) gives
@@ -58,7 +57,6 @@ enum DevErr : int {
     kErrTimeoutFull = 1,    // TMA data never arrived
     kErrTimeoutEmpty = 2,   // smem stage never released
     kErrTimeoutTmem = 3,    // accumulator hand-off never happened
-    kErrBadInput = 4,
     kErrTimeoutGrid = 6,    // a meeting of all CTAs of a cooperative launch never completed
 };
 
@@ -318,10 +316,6 @@ __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *m
         : "memory");
 }
 
-__device__ __forceinline__ void prefetch_tmap(const CUtensorMap *map) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
-
 // ---- tcgen05 (5th-generation tensor core) ----
 __device__ __forceinline__ void tmem_alloc(uint32_t *smem_slot, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -564,16 +558,6 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int ab_fmt) {
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ double warp_min(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 

@@ -71,7 +71,7 @@ constexpr size_t kGemmSmemBytes = 1024 + sizeof(GemmStage) * kGemmStages + sizeo
 __device__ __forceinline__ void record_error(DevCtl *ctl, int code) { atomicCAS(&ctl->err, 0, code); }
 
 // e with m < 2^e <= 2 m for the largest magnitude m (bit pattern of an FP64 value;
-// e = 0 for Inf and NaN, 1 for 0); slices are scaled by 2^(14 - e), so that they
+// e = 0 for Inf, 1 for NaN and 0); slices are scaled by 2^(14 - e), so that they
 // stay finite in FP16
 __device__ __forceinline__ int max_exp(unsigned long long bits) {
     double m = __longlong_as_double(static_cast<long long>(bits));
@@ -429,14 +429,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSymThreads, 1)
 
 // Sum of the nsplit FP32 partial tiles of every tile in a fixed order (FP64),
 // scaled back by 1 / (s_A s_B), written to the upper part of the symmetric C
-// and mirrored.  One block per 16 columns of a tile (the partial tiles are
-// [column][row]): 12 blocks per tile, so that n = 517 (12 tiles) fills the
-// chip: the projection from m = 9001 took 397 us with one block per tile (234 us
-// of it here), 191 us with these.  Bound at large n by the FP64 additions (2 per
-// clock and SM); the FP32 terms are widened by integer operations to keep the
-// conversions off that pipe (n = 4096 from m = 131072, 16 parts: 0.56 ms with a
-// branch to the conversion for the rare encodings, 0.31 ms without one).  The upper rows go out through shared memory,
-// 128 bytes at a time; the mirrored ones are written as they are read.
+// and mirrored.  One block per 16 columns of a CTA's half of a tile (the partial
+// tiles are [column][row]), so that few tiles still fill the chip: n = 517 from m =
+// 9001 has 9 of 256 x 128, 144 blocks, 27 us; one block per tile took 234 us.  Bound
+// at large n by the FP64 additions (2 per clock and SM); the FP32 terms are widened by
+// integer operations to keep the conversions off that pipe (n = 4096 from m = 131072,
+// 16 parts: 0.56 ms with a branch to the conversion for the rare encodings, 0.31 ms
+// without one).  The upper rows go out through shared memory, 128 bytes at a time; the
+// mirrored ones are written as they are read.
 __global__ void __launch_bounds__(256) k_gemm_reduce(const __grid_constant__ GemmArgs g) {
     constexpr int kCols = 16;
     __shared__ double t[kTileM][kCols + 1];

@@ -96,7 +96,6 @@ struct SchedRow {
     int tiles;         // s-th largest problem and those before it: tiles (inclusive)
     int prob;          // the s-th largest problem
 };
-constexpr int kSchedProbs = 256;
 
 // One output of a step as the store phase reads it (shared memory, one copy
 // per drain warp: read from the op descriptor in global memory the fields would
@@ -266,7 +265,7 @@ __device__ __forceinline__ void put_mirror(__half *sl, const uint32_t *w, size_t
 
 // Coefficient of an E term, q + g f.  Sums of a whole group of eight columns
 // contract it, element-wise ones (the edge, the diagonal, FP64 outputs) round
-// the product: the two forms every release has used in these places.
+// the product; results are bit for bit the same only while each place keeps its form.
 __device__ __forceinline__ float e_coef(float g, float f, float q, bool whole) {
     return whole ? fmaf(g, f, q) : __fadd_rn(q, __fmul_rn(g, f));
 }
@@ -619,7 +618,7 @@ struct MmaSmemTail {
     };
     OpCache oc[kEpiWarps];
     SchedHead head;
-    SchedRow row[kSchedProbs];
+    SchedRow row[kSchedTabProbs];
 };
 
 constexpr size_t kMmaSmemBytes = 1024 + sizeof(StageSmem) * kSymStages + sizeof(MmaSmemTail);
@@ -763,8 +762,9 @@ __device__ void ref_tile_sums(const MmaProb &pr, int tile, double (*red)[4], int
 
 // The schedule table of the next step, by the 256 drain threads.  Returns
 // bit 0: some problem has tensor-core work, bit 1: some problem waits for
-// another kernel family, bit 2: some step of bit 0 has reference-tile sums.  Problems beyond kSchedProbs have their rows in global
-// memory (one copy per CTA) and keep the table's order.
+// another kernel family, bit 2: some step of bit 0 has reference-tile sums.
+// A table beyond kSchedTabProbs has its rows in global memory (one copy per CTA) and
+// keeps the table's order.
 __device__ int sched_build(SchedHead *sh, SchedRow *row, const MmaProb *probs, int np, int t, int *mask) {
     // per problem: w = units per reference tile before the width factor,
     // rtiles, tiles, and in units the reference width
@@ -787,7 +787,7 @@ __device__ int sched_build(SchedHead *sh, SchedRow *row, const MmaProb *probs, i
     }
     if (m) atomicOr(mask, m);
     epi_bar();
-    if (np > 1 && np <= kSchedProbs) {
+    if (np > 1 && np <= kSchedTabProbs) {
         // order by descending dimension (ties: table order)
         int rank = 0, tl = 0;
         if (t < np) {
@@ -872,8 +872,6 @@ __device__ int sched_build(SchedHead *sh, SchedRow *row, const MmaProb *probs, i
     return due;
 }
 
-__device__ __forceinline__ int row_work(const SchedRow *row, int q) { return row[q].w; }
-
 // The tiles of one step that this cluster computes: rounds of one tile per
 // cluster, every other round in reverse, so that over two rounds of a list
 // ordered by size every cluster gets about the same work.
@@ -939,7 +937,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSymThreads, 1)
     uint8_t *smem = smem_raw + ((1024u - (base_u32 & 1023u)) & 1023u);
     StageSmem *stages = reinterpret_cast<StageSmem *>(smem);
     MmaSmemTail *tail = reinterpret_cast<MmaSmemTail *>(smem + sizeof(StageSmem) * kSymStages);
-    SchedRow *row = nprobs <= kSchedProbs
+    SchedRow *row = nprobs <= kSchedTabProbs
                         ? tail->row
                         : reinterpret_cast<SchedRow *>(gsched) + static_cast<size_t>(blockIdx.x) * nprobs;
 
@@ -1284,7 +1282,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSymThreads, 1)
             if (met && (due & 4)) {
                 for (int p = 0; p < nprobs; ++p) {
                     const MmaProb &pr = probs[p];
-                    if (row_work(row, p) == 0 || !pr.st->op.ref_sums) continue;
+                    if (row[p].w == 0 || !pr.st->op.ref_sums) continue;
                     for (int k = blockIdx.x; k < pr.ref_ntiles; k += gridDim.x)
                         ref_tile_sums(pr, k, tail->red, et, [] { epi_bar(); });
                 }
