@@ -103,6 +103,7 @@ struct Engine {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaEvent_t ev_setup = nullptr, ev_loop = nullptr;  // end of set-up, end of the step loop
     int nF = 0, nD = 0;              // FP64 and digit tiles of the uploaded lists
+    int sym_grid = 0;                // CTAs of k_sym_mma for the uploaded table
     bool any_tc = false, any_fp64 = false, any_digit = false, any_fermi = false;
     // the step loop as a CUDA graph (eng_graph)
     StepFlags *d_flags = nullptr;
@@ -150,7 +151,7 @@ struct fe_ctx {
     uint32_t prec_default = FE_PREC_MIXED;
     int num_sms = 148;
     int lz_grid = 0;                 // blocks of the cooperative Lanczos launch (all resident)
-    int sym_grid = 0;                // CTAs of a k_sym_mma launch (resident pairs)
+    int sym_grid = 0;                // most CTAs of a k_sym_mma launch (resident pairs)
     Engine eng;                      // blocking solves and batches
     std::mutex smu;                  // slots, used
     std::vector<Slot *> slots;
@@ -812,6 +813,13 @@ void choose_widths(fe_ctx *ctx, std::vector<Job> &jobs) {
         if (!j.bn) j.bn = j.bn2 = std::min(j.ref_bn, width);
 }
 
+// CTAs of a k_sym_mma launch over `tiles` tiles: a pair has no use for more than
+// one tile, and a CTA without one would keep its SM from other streams' kernels for the
+// whole launch, waiting in the meetings (n = 517 at finite temperature: 54 CTAs).
+int sym_ctas(fe_ctx *ctx, size_t tiles) {
+    return 2 * static_cast<int>(std::max<size_t>(1, std::min<size_t>(tiles, ctx->sym_grid / 2)));
+}
+
 // `jobs` get their tile widths here; a problem keeps its widths for the whole
 // solve (the control step reduces the partial slots of the last product's tiles).
 int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
@@ -880,6 +888,7 @@ int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
                                      cudaMemcpyHostToDevice, e.stream));
     // the copies read host vectors that go out of scope here
     FE_CUDA(ctx, cudaStreamSynchronize(e.stream));
+    e.sym_grid = sym_ctas(ctx, tiles.size());
     e.nF = static_cast<int>(tilesF.size());
     e.nD = static_cast<int>(tilesD.size());
     return FE_OK;
@@ -889,7 +898,7 @@ int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
 // CTAs are resident and can meet) up to max_steps with their control steps.
 cudaError_t launch_sym(fe_ctx *ctx, Engine &e, const MmaProb *probs, int np, int max_steps) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctx->sym_grid);
+    cfg.gridDim = dim3(e.sym_grid);
     cfg.blockDim = dim3(kSymThreads);
     cfg.dynamicSmemBytes = mma_smem_bytes();
     cfg.stream = e.stream;
@@ -1111,7 +1120,8 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
                                   reinterpret_cast<uintptr_t>(e.d_tilesF), reinterpret_cast<uintptr_t>(e.d_tilesD),
                                   static_cast<uintptr_t>(np), static_cast<uintptr_t>(e.nF), static_cast<uintptr_t>(e.nD),
                                   static_cast<uintptr_t>(e.any_tc), static_cast<uintptr_t>(e.any_fp64),
-                                  static_cast<uintptr_t>(e.any_digit), reinterpret_cast<uintptr_t>(e.d_sched)};
+                                  static_cast<uintptr_t>(e.any_digit), reinterpret_cast<uintptr_t>(e.d_sched),
+                                  static_cast<uintptr_t>(e.sym_grid)};
     if (e.gexec && key == e.gkey) return FE_OK;
     if (e.gexec) cudaGraphExecDestroy(e.gexec);
     if (e.graph) cudaGraphDestroy(e.graph);
@@ -1160,7 +1170,7 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
         char *gsched = e.d_sched;
         StepFlags *fl = e.d_flags;
         void *args[] = {&probs, &npp, &tl, &err, &runs, &gsched, &fl, &ref_ctas, &max_steps};
-        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_sym_mma), ctx->sym_grid, kSymThreads,
+        FE_CUDA(ctx, add_kernel(ib, reinterpret_cast<const void *>(k_sym_mma), e.sym_grid, kSymThreads,
                                 mma_smem_bytes(), args, nullptr, &kn));
         cudaLaunchAttributeValue coop = {};
         coop.cooperative = 1;
@@ -1983,6 +1993,7 @@ extern "C" int fe_k_sym_square(fe_ctx *ctx, const float *Y, int64_t n, int64_t l
     cudaMemcpyAsync(eg.d_tiles, tl.data(), sizeof(TileEnt) * tl.size(), cudaMemcpyHostToDevice, q);
     cudaMemcpyAsync(s->st, &st0, sizeof(SolveState), cudaMemcpyHostToDevice, q);
     cudaMemsetAsync(eg.d_err, 0, sizeof(int), q);
+    eg.sym_grid = sym_ctas(ctx, tl.size());
     launch_sym(ctx, eg, eg.d_probs, 1, 1);
     ctx->launches += 1;
     cudaMemcpy2DAsync(C, sizeof(float) * ldc, s->Y, sizeof(float) * s->ldy, sizeof(float) * n, n,
