@@ -104,6 +104,7 @@ struct Engine {
     cudaEvent_t ev_setup = nullptr, ev_loop = nullptr;  // end of set-up, end of the step loop
     int nF = 0, nD = 0;              // FP64 and digit tiles of the uploaded lists
     int sym_grid = 0;                // CTAs of k_sym_mma for the uploaded table
+    int sym_steps = 0;               // ... and most steps of one launch in the step graph
     bool any_tc = false, any_fp64 = false, any_digit = false, any_fermi = false;
     // the step loop as a CUDA graph (eng_graph)
     StepFlags *d_flags = nullptr;
@@ -576,6 +577,8 @@ constexpr double kCostChunkCol = 1.5;     // ... growing a little with the colum
 constexpr double kCostTile = 10000.0;     // fill, hand-offs, partials
 constexpr double kCostStore = 230.0;      // store phase, per column
 constexpr double kCostGemmStore = 60.0;   // ... of a k_gemm_split tile
+constexpr double kCostStep = 25000.0;     // a step besides its tiles: meetings, control step
+constexpr double kSliceClocks = 1.6e7;    // about 8 ms (sym_max_steps)
 
 int validate(fe_ctx *ctx, const fe_problem *p) {
     if (!p) return set_err(ctx, FE_EINVAL, "problem is NULL");
@@ -820,6 +823,22 @@ int sym_ctas(fe_ctx *ctx, size_t tiles) {
     return 2 * static_cast<int>(std::max<size_t>(1, std::min<size_t>(tiles, ctx->sym_grid / 2)));
 }
 
+// Most steps of one k_sym_mma launch.  A launch over most of the SMs leaves nothing to
+// other streams (its registers fill an SM), so it ends after about kSliceClocks, or two steps
+// where these take longer, and the graph's next pass goes on; one that leaves a quarter
+// of the SMs free runs all its steps.  Beside finite-temperature solves of n = 8192 (137
+// ms in one launch) a kernel of another stream waited for all of it, now at most 7.7 ms; as
+// launches of single steps it had been 3 ms.  A pass costs 20 us (45 in a batch of 24):
+// 8 ms keep that below 0.5%, 2 ms took 0.7% of a solve at n = 4096.
+int sym_max_steps(fe_ctx *ctx, const std::vector<Job> &jobs, int grid) {
+    if (4 * grid <= 3 * ctx->num_sms) return INT_MAX;
+    double work = 0.0;
+    for (const Job &j : jobs)
+        if (j.bn) work += tile_cost(j.p->n, j.bn) * static_cast<double>(num_tiles_tc(j.p->n, j.bn));
+    const double step = work / (grid / 2) + kCostStep;
+    return std::max(2, static_cast<int>(kSliceClocks / step));
+}
+
 // `jobs` get their tile widths here; a problem keeps its widths for the whole
 // solve (the control step reduces the partial slots of the last product's tiles).
 int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
@@ -889,6 +908,7 @@ int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
     // the copies read host vectors that go out of scope here
     FE_CUDA(ctx, cudaStreamSynchronize(e.stream));
     e.sym_grid = sym_ctas(ctx, tiles.size());
+    e.sym_steps = sym_max_steps(ctx, jobs, e.sym_grid);
     e.nF = static_cast<int>(tilesF.size());
     e.nD = static_cast<int>(tilesD.size());
     return FE_OK;
@@ -1121,7 +1141,7 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
                                   static_cast<uintptr_t>(np), static_cast<uintptr_t>(e.nF), static_cast<uintptr_t>(e.nD),
                                   static_cast<uintptr_t>(e.any_tc), static_cast<uintptr_t>(e.any_fp64),
                                   static_cast<uintptr_t>(e.any_digit), reinterpret_cast<uintptr_t>(e.d_sched),
-                                  static_cast<uintptr_t>(e.sym_grid)};
+                                  static_cast<uintptr_t>(e.sym_grid), static_cast<uintptr_t>(e.sym_steps)};
     if (e.gexec && key == e.gkey) return FE_OK;
     if (e.gexec) cudaGraphExecDestroy(e.gexec);
     if (e.graph) cudaGraphDestroy(e.graph);
@@ -1165,7 +1185,7 @@ int eng_graph(fe_ctx *ctx, Engine &e, int np) {
         FE_CUDA(ctx, cudaGraphAddNode(&prev, body, nullptr, nullptr, 0, &ip));
         cudaGraph_t ib = ip.conditional.phGraph_out[0];
         const TileEnt *tl = e.d_tiles;
-        int npp = np, ref_ctas = ctx->num_sms, max_steps = INT_MAX;
+        int npp = np, ref_ctas = ctx->num_sms, max_steps = e.sym_steps;
         float *runs = e.d_runs;
         char *gsched = e.d_sched;
         StepFlags *fl = e.d_flags;

@@ -52,3 +52,13 @@ def test_small_solve_leaves_the_other_sms():
     lat, loop = _beside(dict(H=torch.from_numpy(p.H).cuda(), ne=440, kT=0.01), 2.0)
     print(len(lat), lat[int(0.95 * len(lat))], lat[-1], loop)
     assert lat[int(0.95 * len(lat))] < 0.25 * loop
+
+
+def test_large_solve_lets_other_streams_in():
+    """n = 4096 at finite temperature: about 130 steps of a fifth of a millisecond on
+    every SM."""
+    n, ne = 4096, 3500
+    p = hp_synth.smeared_reflected(n, ne, 0.01, -2.0, 1.0, 7200, device="cuda")
+    lat, loop = _beside(dict(H=p.H, ne=ne, kT=0.01), 3.0)
+    print(len(lat), lat[int(0.99 * len(lat))], lat[-1], loop)
+    assert lat[int(0.99 * len(lat))] < 0.6 * loop
