@@ -580,6 +580,9 @@ constexpr double kCostGemmStore = 60.0;   // ... of a k_gemm_split tile
 constexpr double kCostStep = 25000.0;     // a step besides its tiles: meetings, control step
 constexpr double kSliceClocks = 1.6e7;    // about 8 ms (sym_max_steps)
 
+constexpr int kServeSteps = 8;   // steps of one launch behind fe_submit, at most
+constexpr int kServePasses = 2;  // ... and passes before new requests may join
+
 int validate(fe_ctx *ctx, const fe_problem *p) {
     if (!p) return set_err(ctx, FE_EINVAL, "problem is NULL");
     if (!p->Hp) return set_err(ctx, FE_EINVAL, "Hp is NULL");
@@ -829,7 +832,7 @@ int sym_ctas(fe_ctx *ctx, size_t tiles) {
 // of the SMs free runs all its steps.  Beside finite-temperature solves of n = 8192 (137
 // ms in one launch) a kernel of another stream waited for all of it, now at most 7.7 ms; as
 // launches of single steps it had been 3 ms.  A pass costs 20 us (45 in a batch of 24):
-// 8 ms keep that below 0.5%, 2 ms took 0.7% of a solve at n = 4096.
+// 8 ms keep that within 0.6%, 2 ms took 0.7% of a solve at n = 4096.
 int sym_max_steps(fe_ctx *ctx, const std::vector<Job> &jobs, int grid) {
     if (4 * grid <= 3 * ctx->num_sms) return INT_MAX;
     double work = 0.0;
@@ -916,7 +919,9 @@ int eng_upload(fe_ctx *ctx, Engine &e, std::vector<Job> &jobs) {
 
 // Launch k_sym_mma over a table: one step, or (cooperatively, so that all its
 // CTAs are resident and can meet) up to max_steps with their control steps.
-cudaError_t launch_sym(fe_ctx *ctx, Engine &e, const MmaProb *probs, int np, int max_steps) {
+// With flags a k_control with the same flags follows.
+cudaError_t launch_sym(fe_ctx *ctx, Engine &e, const MmaProb *probs, int np, int max_steps,
+                       StepFlags *flags = nullptr) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(e.sym_grid);
     cfg.blockDim = dim3(kSymThreads);
@@ -929,14 +934,16 @@ cudaError_t launch_sym(fe_ctx *ctx, Engine &e, const MmaProb *probs, int np, int
     cfg.numAttrs = max_steps > 1 ? 1 : 0;
     ctx->launches += 1;
     return cudaLaunchKernelEx(&cfg, k_sym_mma, probs, np, static_cast<const TileEnt *>(e.d_tiles), e.d_err, e.d_runs,
-                              e.d_sched, static_cast<StepFlags *>(nullptr), ctx->num_sms, max_steps);
+                              e.d_sched, flags, ctx->num_sms, max_steps);
 }
 
-// The error word and the meeting counter of k_sym_mma, cleared before each run.
+// The error word, the meeting counter of k_sym_mma and the step flags, cleared before
+// each run.
 cudaError_t clear_ctl(Engine &e) {
     cudaError_t r = cudaMemsetAsync(&e.d_err->err, 0, sizeof(int), e.stream);
     if (r == cudaSuccess) r = cudaMemsetAsync(&e.d_err->hold, 0, sizeof(int), e.stream);
     if (r == cudaSuccess) r = cudaMemsetAsync(&e.d_err->sym_bar, 0, sizeof(unsigned), e.stream);
+    if (r == cudaSuccess) r = cudaMemsetAsync(e.d_flags, 0, sizeof(StepFlags), e.stream);
     return r;
 }
 
@@ -1041,12 +1048,41 @@ int eng_setup(fe_ctx *ctx, Engine &e, const std::vector<Job> &jobs, int k0, int 
     return FE_OK;
 }
 
+// The kernels of the other families, one step each.
+void other_families(fe_ctx *ctx, Engine &e, int np) {
+    cudaStream_t s = e.stream;
+    if (e.any_fp64) {
+        k_fp64_step<<<std::max(1, std::min(e.nF, 8 * ctx->num_sms)), 256, 0, s>>>(e.d_probs, e.d_tilesF, e.nF, e.d_err);
+        ++ctx->launches;
+    }
+    if (e.any_digit) {
+        k_digit_prep<<<2 * ctx->num_sms, 256, 0, s>>>(e.d_probs, np, e.d_err);
+        k_digit_mma<<<std::max(1, std::min(e.nD, ctx->num_sms)), kMmaThreads, digit_smem_bytes(), s>>>(
+            e.d_probs, e.d_tilesD, e.nD, e.d_err);
+        ctx->launches += 2;
+    }
+}
+
+// One round of the server over the table: passes as in the step graph, each up to
+// kServeSteps steps in one launch of k_sym_mma, so that a request beside blocking
+// solves waits for a turn of the SMs once per pass and not once per step (n = 512
+// beside finite-temperature solves of n = 8192: 289 ms with a launch per step, 95 with
+// these).  FP64 problems take one step a pass.
+void eng_serve(fe_ctx *ctx, Engine &e, int np) {
+    const int steps = std::min(kServeSteps, e.sym_steps);
+    StepFlags *flags = e.any_tc ? e.d_flags : nullptr;
+    for (int p = 0; p < (e.any_tc && !e.any_fp64 ? kServePasses : kServeSteps); ++p) {
+        if (e.any_tc) launch_sym(ctx, e, e.d_probs, np, steps, flags);
+        other_families(ctx, e, np);
+        k_control<<<np, 256, 0, e.stream>>>(e.d_probs, np, e.d_err, flags, 0, 0, -1);
+        ++ctx->launches;
+    }
+}
+
 // `count` expansion steps over every problem in the table; with `pev` each
 // tensor-core and FP64 launch is bracketed by events (4 per step).
 void eng_steps(fe_ctx *ctx, Engine &e, int np, int count, const std::vector<cudaEvent_t> *pev) {
     cudaStream_t s = e.stream;
-    const int grid_f = std::max(1, std::min(e.nF, 8 * ctx->num_sms));
-    const int grid_d = std::max(1, std::min(e.nD, ctx->num_sms));
     for (int it = 0; it < count; ++it) {
         if (pev) cudaEventRecord((*pev)[4 * it + 0], s);
         if (e.any_tc) {
@@ -1058,16 +1094,7 @@ void eng_steps(fe_ctx *ctx, Engine &e, int np, int count, const std::vector<cuda
         }
         if (pev) cudaEventRecord((*pev)[4 * it + 1], s);
         if (pev) cudaEventRecord((*pev)[4 * it + 2], s);
-        if (e.any_fp64) {
-            k_fp64_step<<<grid_f, 256, 0, s>>>(e.d_probs, e.d_tilesF, e.nF, e.d_err);
-            ++ctx->launches;
-        }
-        if (e.any_digit) {
-            k_digit_prep<<<2 * ctx->num_sms, 256, 0, s>>>(e.d_probs, np, e.d_err);
-            k_digit_mma<<<grid_d, kMmaThreads, digit_smem_bytes(), s>>>(e.d_probs, e.d_tilesD, e.nD,
-                                                                        e.d_err);
-            ctx->launches += 2;
-        }
+        other_families(ctx, e, np);
         if (pev) cudaEventRecord((*pev)[4 * it + 3], s);
         k_control<<<np, 256, 0, s>>>(e.d_probs, np, e.d_err, nullptr, 0, 0, 0);
         ++ctx->launches;
@@ -1264,7 +1291,6 @@ int run_problems_once(fe_ctx *ctx, std::vector<Job> &jobs, fe_result *rs) {
     if (use_graph) {
         rc = eng_graph(ctx, e, np);
         if (rc != FE_OK) return rc;
-        FE_CUDA(ctx, cudaMemsetAsync(e.d_flags, 0, sizeof(StepFlags), s));
         FE_CUDA(ctx, cudaGraphLaunch(e.gexec, s));
         FE_CUDA(ctx, cudaMemcpyAsync(&e.h_flags, e.d_flags, sizeof(StepFlags), cudaMemcpyDeviceToHost, s));
     } else {
@@ -1407,13 +1433,12 @@ int run_problems(fe_ctx *ctx, std::vector<Job> &jobs, fe_result *rs) {
 // Continuous batching behind fe_submit / fe_poll.  One worker thread owns a
 // second engine (its own stream).  Each tick it starts the waiting requests
 // that fit the free part of the HBM budget (first fit, in submission order),
-// runs kServeSteps expansion steps over every running request at once, reads
+// runs some expansion steps over every running request at once (eng_serve), reads
 // the done flags, and finishes the requests that converged (D written, slot
 // released, result published for fe_poll).  Requests therefore join and
 // leave the batch at step granularity, and short solves are not held back by
 // long ones.
 
-constexpr int kServeSteps = 8;
 constexpr size_t kMaxTickets = 1 << 16;
 constexpr double kAdmitWaitMs = 60000.0;
 
@@ -1529,7 +1554,7 @@ void serve_loop(fe_ctx *ctx) {
         }
         int herr = 0;
         if (rc == FE_OK) {
-            eng_steps(ctx, e, np, kServeSteps, nullptr);
+            eng_serve(ctx, e, np);
             for (int k = 0; k < np; ++k)
                 cudaMemcpyAsync(&e.h_done[k], &all[k]->slot->st->done, sizeof(int),
                                 cudaMemcpyDeviceToHost, e.stream);

@@ -82,7 +82,7 @@ struct TileF64 {
     int slot;
 };
 
-// Step bookkeeping of the graph-driven step loop (see k_control).  With
+// Step bookkeeping of a pass of the step loop (see k_control).  With
 // max_steps > 1, k_sym_mma runs the control steps between its products itself;
 // `controlled` tells the k_control behind it that every tensor-core step issued
 // is still to run.  The problems stay in step: when the control step leaves some
@@ -196,9 +196,10 @@ struct StepFlags {
     unsigned n_tc;             // passes after the first with k_sym_mma switched on
     unsigned controlled;       // k_sym_mma ran the control step of its last product
 };
-// Control step: one block per problem.  With flags (inside the step graph)
-// the last block to finish also sets the graph's loop condition and the switch
-// of k_sym_mma.  Once a kernel of the run has recorded an error in ctl (a bounded
+// Control step: one block per problem.  With flags (behind a k_sym_mma with the same
+// flags) the last block to finish also closes the pass: inside the step graph it sets
+// the loop condition and, with has_tc = 1, the switch of k_sym_mma; has_tc < 0: the
+// pass is not in a graph.  Once a kernel of the run has recorded an error in ctl (a bounded
 // wait ran out), every problem ends with FE_ETIMEOUT.
 __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, StepFlags *flags,
                           cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_tc, int has_tc);

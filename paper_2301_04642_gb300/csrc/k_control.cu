@@ -29,7 +29,8 @@ __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, S
     if (!flags || threadIdx.x != 0) return;
     // Inside the step graph: collect what the next pass needs over all problems;
     // the block that finishes last sets the graph's conditions (loop on while any
-    // problem is active, k_sym_mma on while any has tensor-core work).
+    // problem is active, k_sym_mma on while any has tensor-core work).  Passes outside
+    // a graph (has_tc < 0) have no conditions.
     unsigned bits = stepped ? kStepped : 0u;
     if (p < nprobs) {
         const SolveState *st = probs[p].st;
@@ -41,8 +42,8 @@ __global__ void k_control(const MmaProb *probs, int nprobs, const DevCtl *ctl, S
     __threadfence();
     const unsigned m = atomicExch(&flags->mask, 0u);
     atomicExch(&flags->count, 0u);
-    cudaGraphSetConditional(h_loop, (m & kActive) ? 1u : 0u);
-    if (has_tc) cudaGraphSetConditional(h_tc, (m & kTc) ? 1u : 0u);
+    if (has_tc >= 0) cudaGraphSetConditional(h_loop, (m & kActive) ? 1u : 0u);
+    if (has_tc > 0) cudaGraphSetConditional(h_tc, (m & kTc) ? 1u : 0u);
     flags->n_ctl += 1;
     if (m & kStepped) flags->n_steps += 1;
     if (m & kTc) flags->n_tc += 1;

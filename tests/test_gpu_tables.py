@@ -72,10 +72,11 @@ def test_families_due_in_different_steps(fp64):
     _solve(m)
 
 
-def test_expired_meeting_inside_the_step_graph():
+@pytest.mark.parametrize("served", [False, True])
+def test_expired_meeting_between_steps(served):
     """The truncated expansion takes Gershgorin bounds, so no certificate launch comes
-    before the step graph: the meeting that runs out (a word nothing writes, 1 ms) is
-    one between two steps of the graph's kernel."""
+    before the steps: the meeting that runs out (a word nothing writes, 1 ms) is one
+    between two steps, in the step graph's kernel or in a served pass."""
     need_gpu()
     import paper_2301_04642_gb300 as fe
     p = hp_synth.smeared(400, 320, 0.02, -2.0, 1.0, 6300)
@@ -83,12 +84,16 @@ def test_expired_meeting_inside_the_step_graph():
     D = [torch.empty_like(H) for _ in range(2)]
     kw = dict(ne=320, kT=0.02, method=fe.FE_METHOD_TRFOE)
     with fe.Context(device=0) as c:
-        r0 = c.solve(H, D=D[0], **kw)
+        def solve(D=None):
+            return c.wait(c.submit(H, D=D, **kw), timeout_s=60) if served else c.solve(H, D=D, check=False, **kw)
+
+        r0 = solve(D[0])
         c.set_wait(limit_ms=1.0, fail_partner=True)
-        r = c.solve(H, check=False, **kw)
-        assert r["status"] == fe.FE_ETIMEOUT and "timed out" in c.last_error()
+        r = solve()
+        assert r["status"] == r["rc"] == fe.FE_ETIMEOUT
+        assert served or "timed out" in c.last_error()
         c.set_wait(limit_ms=2000.0, fail_partner=False)
-        r1 = c.solve(H, D=D[1], **kw)
+        r1 = solve(D[1])
     assert r1["status"] == 0 and r1["iters"] == r0["iters"] and torch.equal(D[0], D[1])
 
 
