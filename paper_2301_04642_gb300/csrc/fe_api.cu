@@ -393,16 +393,18 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
     if (bytes > ctx->budget)
         return set_err(ctx, FE_ENOMEM, "problem needs " + std::to_string(bytes) +
                                            " bytes, more than the HBM budget");
-    // evict unused cached slots until it fits
-    while (ctx->used + bytes > ctx->budget) {
+    // free an unused cached slot, if there is one
+    auto evict = [&] {
         auto it = std::find_if(ctx->slots.begin(), ctx->slots.end(),
                                [](Slot *s) { return !s->in_use; });
-        if (it == ctx->slots.end())
-            return set_err(ctx, FE_ENOMEM, "HBM budget exhausted by active solves");
+        if (it == ctx->slots.end()) return false;
         Slot *v = *it;
         ctx->slots.erase(it);
         free_slot(ctx, v);
-    }
+        return true;
+    };
+    while (ctx->used + bytes > ctx->budget)
+        if (!evict()) return set_err(ctx, FE_ENOMEM, "HBM budget exhausted by active solves");
     Slot *s = new Slot();
     s->n = n;
     s->method = method;
@@ -410,7 +412,10 @@ int acquire_slot(fe_ctx *ctx, int n, int method, Slot **out) {
     s->ldy = ldy;
     s->lds = lds;
     s->ldx = ldx;
-    cudaError_t e = cudaMalloc(&s->arena, bytes);
+    // the device may hold less than the budget (the program's own allocations since
+    // fe_create): cached slots make way for that too
+    cudaError_t e;
+    while ((e = cudaMalloc(&s->arena, bytes)) != cudaSuccess && evict()) cudaGetLastError();
     if (e != cudaSuccess) {
         delete s;
         cudaGetLastError();

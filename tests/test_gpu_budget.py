@@ -84,3 +84,25 @@ def test_projection_in_a_budget_of_slices_and_sums(m, n):
     with fe.Context(device=0, hbm_budget_bytes=8 * n * lds) as c, pytest.raises(fe.FeError) as ei:
         c.project(P, Y, H[0])
     assert ei.value.status == fe.FE_ENOMEM
+
+
+@pytest.mark.parametrize("served", [False, True])
+def test_cached_slots_make_way_when_the_device_is_full(served):
+    """The budget is taken at fe_create; a program that then allocates most of the
+    device leaves room for one slot, whatever sizes came before."""
+    need_gpu()
+    import paper_2301_04642_gb300 as fe
+    probs = [hp_synth.gapped_reflected(n, n // 2, (-3.0, -0.05), (0.05, 1.0), n, device="cuda") for n in (3000, 3100, 3200)]
+    with fe.Context(device=0) as c:
+        c.solve(probs[0].H, 1500)  # the engines' own buffers
+        c.wait(c.submit(probs[0].H, 1500))
+        torch.cuda.empty_cache()
+        fill = torch.empty(torch.cuda.mem_get_info()[0] - (400 << 20), dtype=torch.uint8, device="cuda")
+        for p in probs + probs[:1]:  # 0.52 to 0.59 GB a slot
+            if served:
+                r = c.wait(c.submit(p.H, p.ne), timeout_s=90)
+                assert r["rc"] == 0
+            else:
+                assert c.solve(p.H, p.ne)["status"] == 0
+        del fill
+        torch.cuda.empty_cache()
