@@ -1165,7 +1165,8 @@ void fill_result(const SolveState &st, int herr, double ms, fe_result &r) {
 // The step loop of the uploaded table as an instantiated CUDA graph (built once
 // per table layout), with no host round trip:
 //   WHILE(any problem active) { IF(tensor-core work) k_sym_mma, which runs
-//     products and their control steps until another family is due;
+//     products and their control steps until another family is due or its steps
+//     (sym_steps) are done;
 //     k_fp64_step; k_digit_prep, k_digit_mma; k_control }
 int eng_graph(fe_ctx *ctx, Engine &e, int np) {
     std::vector<uintptr_t> key = {reinterpret_cast<uintptr_t>(e.d_probs), reinterpret_cast<uintptr_t>(e.d_tiles),
